@@ -190,7 +190,7 @@ int hweno_bind(hweno_t* h, double* state_dev, void* ws) {
   p += l.MD;
   h->w.NOD = reinterpret_cast<double*>(p);
   p += l.NOD;
-  h->w.PRIM = reinterpret_cast<double*>(p);
+  h->w.PRIM = reinterpret_cast<float2*>(p);
   p += l.PRIM;
   h->w.FX = reinterpret_cast<double*>(p);
   p += l.FX;
@@ -650,7 +650,7 @@ extern "C" int hweno_rhs_static(int dim, int system, int64_t nx, int64_t ny, dou
   p += l.MD;
   h.w.NOD = reinterpret_cast<double*>(p);
   p += l.NOD;
-  h.w.PRIM = reinterpret_cast<double*>(p);
+  h.w.PRIM = reinterpret_cast<float2*>(p);
   p += l.PRIM;
   h.w.FX = reinterpret_cast<double*>(p);
   p += l.FX;

@@ -45,13 +45,13 @@ struct BatchArgs {
 
 template <int DIM>
 __device__ __forceinline__ void batch_cells(const BatchInst& I, long long p0, int tpi, int slot) {
+  __shared__ Leftover lo;
   double wsx = 0.0, wsy = 0.0;
   for (int t = 0; t < tpi; ++t) {
-    const long long p = p0 + (long long)t * kThreads + threadIdx.x;
     double a = 0.0, b = 0.0;
-    if (p < I.g.plane) cell_body<DIM, SYS_EULER>(I.g, I.S, I.w, p, a, b);
-    wsx = fmax(wsx, a);
-    wsy = fmax(wsy, b);
+    cell_tile<DIM, SYS_EULER, 0>(I.g, I.S, I.w, p0 + (long long)t * kThreads, a, b, lo, true);
+    wsx = speed_bits(a) > speed_bits(wsx) ? a : wsx;
+    wsy = speed_bits(b) > speed_bits(wsy) ? b : wsy;
   }
   block_max2(wsx, wsy, I.w.alpha + slot * I.w.astride);
   __syncthreads();  // the reduction's shared arrays are reused by the next item
@@ -61,10 +61,9 @@ template <int DIM>
 __device__ __forceinline__ void batch_faces(const BatchInst& I, int dir, long long f0, int tpi, int slot) {
   const long long nf = dir == 0 ? (long long)(I.g.nx + 1) * I.g.ny : (long long)(I.g.ny + 1) * I.g.nx;
   const double alpha = __longlong_as_double((long long)I.w.alpha[slot * I.w.astride + dir]);
-  for (int t = 0; t < tpi; ++t) {
-    const long long f = f0 + (long long)t * kThreads + threadIdx.x;
-    if (f < nf) face_body<DIM, SYS_EULER>(I.g, I.S, I.w, dir, f, alpha);
-  }
+  __shared__ Leftover lo;
+  for (int t = 0; t < tpi; ++t)
+    face_tile<DIM, SYS_EULER, 0>(I.g, I.S, I.w, dir, f0 + (long long)t * kThreads, nf, alpha, lo, true);
 }
 
 template <int DIM>
@@ -453,6 +452,7 @@ int hweno_batch_bind(hweno_batch_t* b, double* state_dev, void* ws) {
     h.w.alpha = b->alpha + 2 * i;
     h.w.astride = 2 * b->n;
     hi[i].g = grid_of(&h);
+    hi[i].g.pairs = 1;  // many instances share the FP64 pipe
     hi[i].w = h.w;
     hi[i].S = h.state;
     hi[i].dim = h.dim;

@@ -128,12 +128,27 @@ inline Layout layout_of(const hweno_ctx* h) {
   return l;
 }
 
+// x as hi + lo of two FP32 numbers
+inline void to_pair(double x, float* p) {
+  p[0] = (float)x;
+  p[1] = (float)(x - (double)p[0]);
+}
+
+// The nonlinear part in pairs (hweno_pair.cuh) trades FP64 instructions for several times as many FP32
+// ones, which pays where the FP64 pipe is kept busy.  A 1D grid of at most one warp per scheduler (19456
+// cells) leaves it idle and waits for each thread's chain of instructions instead, which is the
+// longer one in pairs: one stage of 2048 cells 43 us in FP64, 53 us in pairs.  A 2D grid of 64^2
+// cells (128 warps of cells, 260 of faces) already gains: 64 us in FP64, 48 us in pairs.
+constexpr long long kPairMinCells1D = hw::kSMs * 4LL * 32;
+inline int pairs_of(const hweno_ctx* h) { return h->dim == 2 || h->nx > kPairMinCells1D; }
+
 inline Grid grid_of(const hweno_ctx* h) {
   Grid g;
   g.nx = (int)h->nx;
   g.ny = (int)h->ny;
   g.bc = h->bc;
   g.flags = h->flags;
+  g.pairs = pairs_of(h);
   g.plane = (long long)h->nx * h->ny;
   g.dx = h->dx;
   g.dy = h->dy;
@@ -214,10 +229,21 @@ inline Grid grid_of(const hweno_ctx* h) {
     g.uvd[d][0] = 1.3125 / hs[d];
     g.uvd[d][1] = 0.1875 / hs[d];
     g.ucsv[d] = csv * hs[d];
+    g.l3[d] = 3.0 / 64.0 * hs[d];
+    g.l9[d] = 9.0 / 64.0 * hs[d];
+    g.l34[d] = 0.75 / hs[d];
+    to_pair(hs[d], g.pg.h[d]);
+    to_pair(1.0 / hs[d], g.pg.ih[d]);
     g.e2fih[d] = hw::DCoef2::ef / hs[d];
     g.e2gih[d] = hw::DCoef2::eg / hs[d];
   }
   g.ig1 = 1.0 / g1;
+  to_pair(g.gm1, g.pg.gm1);
+  to_pair(g.eps, g.pg.eps);
+  to_pair(g.G + 2.0, g.pg.ig1);
+  to_pair(g.Gd + 2.0, g.pg.id1);
+  g.pg.G = (float)g.G;
+  g.pg.Gd = (float)g.Gd;
   g.grav = h->grav;
   for (int sd = 0; sd < 4; ++sd) {
     g.side[sd] = h->side[sd];

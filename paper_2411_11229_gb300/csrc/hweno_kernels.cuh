@@ -24,6 +24,7 @@
 // face states of the ghost cells at the ends of every line.
 #pragma once
 #include "hweno_math.cuh"
+#include "hweno_pair.cuh"
 
 namespace hw {
 
@@ -32,7 +33,8 @@ struct Work {
   double* B;     // stage base M(S^n): [NF][NC][plane]
   double* MD;    // modified derivatives (V~, W~): [DIM][NC][plane]
   double* NOD;   // nodal values per direction, normal frame: [DIM][NG][NC][plane]
-  double* PRIM;  // Euler primitives (sqrt(rho), u[, v], H): [NP][plane]
+  float2* PRIM;  // Euler primitives (sqrt(rho), u[, v], H) as pairs (hweno_pair.cuh): [NP][plane]; grids
+                 // that take no pairs (Grid::pairs) keep them in FP64 in the same bytes
   double* FX;    // x-face fluxes, original frame: [NF][NC][ny][nx+1]
   double* FY;    // y-face fluxes: [NF][NC][ny+1][nx]
   unsigned long long* alpha;  // wavespeed slots (bit patterns of non-negative doubles): slot s of
@@ -53,6 +55,7 @@ struct Work {
 };
 
 constexpr int kThreads = 128;
+constexpr int kSMs = 152;  // streaming multiprocessors of the GPU
 
 // The units of FU in thread registers: a zero read at a per-thread address of the zeroed slots
 // scal[4..7], so that the compiler can neither fold it nor keep it in a uniform register.
@@ -70,32 +73,42 @@ __device__ __forceinline__ void swap_frame(double* q) {
   }
 }
 
-// max over the block of (a, b), then one atomicMax per block on the bit patterns
+// The bit pattern of a wavespeed (non-negative, so its order is the numbers'), 0 for a NaN
+__device__ __forceinline__ unsigned long long speed_bits(double x) {
+  const unsigned long long b = dbl_bits(x);
+  return b <= 0x7ff0000000000000ull ? b : 0ull;
+}
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long b) {
+  const unsigned int hi = __reduce_max_sync(0xffffffffu, (unsigned int)(b >> 32));
+  const unsigned int lo = __reduce_max_sync(0xffffffffu, (unsigned int)(b >> 32) == hi ? (unsigned int)b : 0u);
+  return ((unsigned long long)hi << 32) | lo;
+}
+// max over the block of the wavespeeds (a, b), then one atomicMax per block, all on the bit patterns
+// (a maximum of FP64 numbers is an instruction of the FP64 pipe)
 __device__ __forceinline__ void block_max2(double a, double b, unsigned long long* dst) {
-  __shared__ double sa[32], sb[32];
-  for (int o = 16; o > 0; o >>= 1) {
-    a = fmax(a, __shfl_xor_sync(0xffffffffu, a, o));
-    b = fmax(b, __shfl_xor_sync(0xffffffffu, b, o));
-  }
+  __shared__ unsigned long long sm[2][32];
+  unsigned long long x = warp_max(speed_bits(a)), y = warp_max(speed_bits(b));
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (lane == 0) {
-    sa[wid] = a;
-    sb[wid] = b;
+    sm[0][wid] = x;
+    sm[1][wid] = y;
   }
   __syncthreads();
   if (wid == 0) {
     const int nw = blockDim.x >> 5;
-    a = lane < nw ? sa[lane] : 0.0;
-    b = lane < nw ? sb[lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) {
-      a = fmax(a, __shfl_xor_sync(0xffffffffu, a, o));
-      b = fmax(b, __shfl_xor_sync(0xffffffffu, b, o));
-    }
+    x = warp_max(lane < nw ? sm[0][lane] : 0ull);
+    y = warp_max(lane < nw ? sm[1][lane] : 0ull);
     if (lane == 0) {
-      atomicMax(dst, dbl_bits(a));
-      atomicMax(dst + 1, dbl_bits(b));
+      atomicMax(dst, x);
+      atomicMax(dst + 1, y);
     }
   }
+}
+// whether x is a finite number, and whether it is greater than zero, in the integer pipe
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool positive_bits(double x) {
+  const unsigned long long b = dbl_bits(x);
+  return b - 1ull < 0x7ff0000000000000ull;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -246,15 +259,138 @@ __device__ __forceinline__ void r2_cell(const double (&U3)[3][NC], const double 
     r2_cell_vw<NC, SYS, false>(U3, D3, e, dir, g, md, fs, f);
 }
 
-// Cell work of one stage at cell p: primitives and wavespeeds (returned in wsx, wsy), nodal
-// values per direction, modified derivatives (and, for R2, the face states of the cell).
+// The modified derivative of cell p in direction d (and, for R2, the cell's face states) with the
+// FP64 weights: the cells that cell_body leaves to it.
+template <int DIM, int SYS, int VAR>
+__device__ __forceinline__ void cell_limiter(const Grid& g, const double* __restrict__ S, const Work& w, long long p,
+                                             int d) {
+  constexpr int NC = Traits<DIM, SYS>::NC;
+  const long long plane = g.plane;
+  const FU f = fu_of(w.scal);
+  const int i = (int)(p % g.nx), j = (int)(p / g.nx);
+  double U3[3][NC], D3[3][NC];
+  load_stencil3<DIM, SYS, VAR, NC>(g, S, d, i, j, d == 0 ? i : j, nullptr, U3, D3);
+  Eig<NC> e;
+  if (SYS == SYS_EULER) {
+    const double* U = U3[1];
+    const double ir = rcp(U[0], f);
+    const double u = f.mul(U[1], ir), v = NC == 4 ? f.mul(U[2], ir) : 0.0;
+    const double ke = NC == 4 ? fma(U[1], u, f.mul(U[2], v)) : f.mul(U[1], u);
+    const double pr = g.gm1 * fma(-0.5, ke, U[NC - 1]);
+    const double c2 = f.mul(g.gamma * pr, ir);
+    const double ic = rsqrt_fast(c2, f);
+    e.setup(u, v, f.mul(f.add(U[NC - 1], pr), ir), f.mul(c2, ic), ic, g.gm1);
+  }
+  double out[NC];
+  if (VAR == 2) {
+    double fs[4][NC];
+    r2_cell<NC, SYS>(U3, D3, e, d, g, out, fs, f);
+    double* FSd = w.FS + (long long)d * 4 * NC * plane;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int k = 0; k < NC; ++k) FSd[(q * NC + k) * plane + p] = fs[q][k];
+  } else {
+    modified_derivative<NC, SYS>(U3, D3, e, d, g, out, f);
+  }
+  if (SYS == SYS_EULER && d == 1) swap_frame<NC>(out);
+#pragma unroll
+  for (int k = 0; k < NC; ++k) w.MD[((long long)d * NC + k) * plane + p] = out[k];
+}
+
+// The same in every direction with the nonlinear part in pairs (hweno_pair.cuh): U, pu, pv, pH, pc2 the
+// cell's state and its velocities, enthalpy and c^2.  Returns false, having written nothing, where
+// the FP64 weights are needed.
+template <int DIM, int SYS, int VAR>
+__device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* __restrict__ S, const Work& w,
+                                                  long long p, int i, int j, const double* U, P2 pu, P2 pv, P2 pH,
+                                                  P2 pc2, const FU& f) {
+  constexpr int NC = Traits<DIM, SYS>::NC;
+  const long long plane = g.plane;
+  // FP64: p_0'(x_i) = 3/4 (u_{i+1} - u_{i-1})/h - (v_{i-1} + v_{i+1})/4 and (R2) the linear parts of the
+  // values and the derivatives at the two faces
+  double md[DIM][NC], um[DIM][NC], up[DIM][NC], dm[DIM][NC], dp[DIM][NC];
+  P4 dU[2][NC], Z[2][NC];
+  {
+    P2 uc[NC], du[2][DIM][NC], z[2][DIM][NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) uc[k] = p_from(U[k]);
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+      double U3[3][NC], D3[3][NC];
+      load_stencil3<DIM, SYS, VAR, NC>(g, S, d, i, j, d == 0 ? i : j, U, U3, D3);
+      const double k21 = g.uvd[d][0], k3 = g.uvd[d][1];
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        md[d][k] = fma(g.l34[d], f.sub(U3[2][k], U3[0][k]), -0.25 * f.add(D3[0][k], D3[2][k]));
+        // the differences are taken between pairs: U to 48 bits is enough for the correction
+        const P2 u1 = uc[SYS == SYS_EULER && NC == 4 && d == 1 && (k == 1 || k == 2) ? 3 - k : k];
+        du[0][d][k] = p_renorm(p_sub(u1, p_from(U3[0][k])));
+        du[1][d][k] = p_renorm(p_sub(p_from(U3[2][k]), u1));
+        z[0][d][k] = p_from(D3[0][k]);
+        z[1][d][k] = p_from(D3[2][k]);
+        if (VAR == 2) {
+          const double d0 = f.sub(U3[1][k], U3[0][k]), d1 = f.sub(U3[2][k], U3[1][k]);
+          um[d][k] = fma(0.125, d0, fma(0.5625, d1, fma(-g.l3[d], D3[0][k], -g.l9[d] * D3[2][k])));
+          up[d][k] = fma(-0.125, d1, fma(-0.5625, d0, fma(g.l3[d], D3[2][k], g.l9[d] * D3[0][k])));
+          dm[d][k] = fma(k21, d1, fma(-k3, d0, fma(0.0625, D3[0][k], -0.1875 * D3[2][k])));
+          dp[d][k] = fma(k21, d0, fma(-k3, d1, fma(-0.1875, D3[0][k], 0.0625 * D3[2][k])));
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        dU[q][k] = p_pack(du[q][0][k], du[q][DIM - 1][k]);
+        Z[q][k] = p_pack(z[q][0][k], z[q][DIM - 1][k]);
+      }
+  }
+  EigP<NC, F2> e;
+  if (SYS == SYS_EULER) {
+    const P2 un = DIM == 2 ? pv : pu, ut = DIM == 2 ? pu : pv;
+    e.setup(p_pack(pu, un), p_pack(pv, ut), p_pack(pH, pH), p_pack(pc2, pc2), p_const<F2>(g.pg.gm1));
+  }
+  const P4 h = p_pack(p_const<float>(g.pg.h[0]), p_const<float>(g.pg.h[DIM - 1]));
+  P4 nm[NC], np[NC], nt[NC];
+  if (!p_cell<NC, SYS, VAR == 2>(dU, Z, e, h, g.pg, nm, np, nt)) return false;
+#pragma unroll
+  for (int d = 0; d < DIM; ++d) {
+    const P2 ih = p_const<float>(g.pg.ih[d]);
+    double out[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const P2 n = p_mul(d == 0 ? p_lane0(nt[k]) : p_lane1(nt[k]), ih);
+      out[k] = f.add(md[d][k], f.add(d_from(n.h), d_from(n.l)));
+    }
+    if (VAR == 2) {
+      double* FSd = w.FS + (long long)d * 4 * NC * plane;
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        const P2 a = d == 0 ? p_lane0(nm[k]) : p_lane1(nm[k]), b = d == 0 ? p_lane0(np[k]) : p_lane1(np[k]);
+        const double u1 = U[SYS == SYS_EULER && NC == 4 && d == 1 && (k == 1 || k == 2) ? 3 - k : k];
+        FSd[k * plane + p] = f.add(u1, f.add(um[d][k], f.add(d_from(a.h), d_from(a.l))));
+        FSd[(NC + k) * plane + p] = dm[d][k];
+        FSd[(2 * NC + k) * plane + p] = f.add(u1, f.add(up[d][k], f.add(d_from(b.h), d_from(b.l))));
+        FSd[(3 * NC + k) * plane + p] = dp[d][k];
+      }
+    }
+    if (SYS == SYS_EULER && d == 1) swap_frame<NC>(out);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) w.MD[((long long)d * NC + k) * plane + p] = out[k];
+  }
+  return true;
+}
+
+// Cell work of one stage at cell p: wavespeeds (returned in wsx, wsy), primitives, nodal values per
+// direction, modified derivatives (and, for R2, the face states of the cell).  Returns
+// false where the modified derivatives are left to cell_limiter.
 template <int DIM, int SYS, int VAR = 0>
-__device__ __forceinline__ void cell_body(const Grid& g, const double* __restrict__ S, const Work& w, long long p_in,
-                                          double& wsx, double& wsy) {
+__device__ __forceinline__ bool cell_body(const Grid& g, const double* __restrict__ S, const Work& w, long long p,
+                                         double& wsx, double& wsy) {
   using T = Traits<DIM, SYS>;
   constexpr int NC = T::NC, NG = T::NG;
   const long long plane = g.plane;
-  const long long p = HW_IDX(p_in, plane);
   const FU f = fu_of(w.scal);
   {
     const int i = (int)(p % g.nx), j = (int)(p / g.nx);
@@ -266,32 +402,21 @@ __device__ __forceinline__ void cell_body(const Grid& g, const double* __restric
       if (DIM == 2) Wd[k] = S[(2 * NC + k) * plane + p];
     }
     // primitives and wavespeeds
-    double u = 0, v = 0, pr = 0, ir = 0, H = 0, c = 0, ic = 0;
+    double u = 0, v = 0, pr = 0, ir = 0;
     if (SYS == SYS_EULER) {
       ir = rcp(U[0], f);
       u = f.mul(U[1], ir);
       if (DIM == 2) v = f.mul(U[2], ir);
       const double ke = DIM == 2 ? fma(U[1], u, f.mul(U[2], v)) : f.mul(U[1], u);
       pr = g.gm1 * fma(-0.5, ke, U[NC - 1]);
-      H = f.mul(f.add(U[NC - 1], pr), ir);
-      const double c2 = f.mul(g.gamma * pr, ir);
-      ic = rsqrt(c2);
-      c = f.mul(c2, ic);
-      wsx = fabs(u) + c;
-      wsy = DIM == 2 ? fabs(v) + c : 0.0;
-      if (!(U[0] > 0.0) || !(pr > 0.0) || !isfinite(wsx) || !isfinite(wsy)) atomicOr(w.status, 1u);
-      w.PRIM[p] = sqrt(U[0]);
-      w.PRIM[plane + p] = u;
-      if (DIM == 2) {
-        w.PRIM[2 * plane + p] = v;
-        w.PRIM[3 * plane + p] = H;
-      } else {
-        w.PRIM[2 * plane + p] = H;
-      }
+      const double c = sqrt_fast(f.mul(g.gamma * pr, ir), f);
+      wsx = f.add(fabs(u), c);
+      wsy = DIM == 2 ? f.add(fabs(v), c) : 0.0;
+      if (!positive_bits(U[0]) || !positive_bits(pr) || !finite_bits(wsx) || !finite_bits(wsy)) atomicOr(w.status, 1u);
     } else if (SYS == SYS_BURGERS) {
       wsx = fabs(U[0]);
       wsy = DIM == 2 ? wsx : 0.0;
-      if (!isfinite(wsx)) atomicOr(w.status, 1u);
+      if (!finite_bits(wsx)) atomicOr(w.status, 1u);
     } else {
       wsx = fabs(g.ax);
       wsy = DIM == 2 ? fabs(g.ay) : 0.0;
@@ -352,38 +477,81 @@ __device__ __forceinline__ void cell_body(const Grid& g, const double* __restric
         if (DIM == 2) nod[(2 * NC + k) * plane + p] = Mx[k];
       }
     }
-    // modified derivatives (Eq. limiter), one per direction
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) {
-      const int a0 = d == 0 ? i : j;
-      double U3[3][NC], D3[3][NC];
-      load_stencil3<DIM, SYS, VAR, NC>(g, S, d, i, j, a0, U, U3, D3);
-      Eig<NC> e;
-      if (SYS == SYS_EULER) e.setup(d == 0 ? u : v, d == 0 ? v : u, H, c, ic, g.gm1);
-      double out[NC];
-      if (VAR == 2) {
-        double fs[4][NC];
-        r2_cell<NC, SYS>(U3, D3, e, d, g, out, fs, f);
-        double* FSd = w.FS + (long long)d * 4 * NC * plane;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int k = 0; k < NC; ++k) FSd[(q * NC + k) * plane + p] = fs[q][k];
-      } else {
-        modified_derivative<NC, SYS>(U3, D3, e, d, g, out, f);
+    // modified derivatives (Eq. limiter), one per direction; the weighted derivative of R2 needs the
+    // weights themselves
+    if (DIM == 1 && !g.pairs) {
+      if (SYS == SYS_EULER && VAR != 2) {
+        double* P = reinterpret_cast<double*>(w.PRIM);
+        P[p] = sqrt_fast(U[0], f);
+        P[plane + p] = u;
+        P[2 * plane + p] = f.mul(f.add(U[NC - 1], pr), ir);
       }
-      if (SYS == SYS_EULER && d == 1) swap_frame<NC>(out);
-#pragma unroll
-      for (int k = 0; k < NC; ++k) w.MD[((long long)d * NC + k) * plane + p] = out[k];
+      return false;
     }
+    if (VAR == 2 && (g.flags & FLAG_V_WEIGHTED)) return false;
+    P2 pu = {0.0f, 0.0f}, pv = pu, pH = pu, pc2 = pu;
+    if (SYS == SYS_EULER) {
+      P2 q[NC], inv;
+#pragma unroll
+      for (int k = 0; k < NC; ++k) q[k] = p_from(U[k]);
+      const P2 gm1 = P2{g.pg.gm1[0], g.pg.gm1[1]};
+      p_prim<NC>(q, gm1, pu, pv, pH, pc2);
+      pc2 = p_add(pc2, p_mul(gm1, pc2));  // gamma p / rho
+      if (VAR != 2) {
+        const P2 sr = p_sqrt(q[0], inv);
+        w.PRIM[p] = make_float2(sr.h, sr.l);
+        w.PRIM[plane + p] = make_float2(pu.h, pu.l);
+        if (DIM == 2) w.PRIM[2 * plane + p] = make_float2(pv.h, pv.l);
+        w.PRIM[DIM * plane + plane + p] = make_float2(pH.h, pH.l);
+      }
+    }
+    return cell_limiter_pair<DIM, SYS, VAR>(g, S, w, p, i, j, U, pu, pv, pH, p_renorm(pc2), f);
+  }
+}
+
+// The cells or faces of one block whose nonlinear weights are to be evaluated in FP64: the block's
+// threads take them in turn afterwards, so that a warp with a single one of them does not run the
+// FP64 path for its other lanes (an FP64 warp instruction costs the same with one lane active).
+struct Leftover {
+  int n;
+  unsigned short item[2 * kThreads];
+};
+
+// The cells p0 .. p0 + kThreads - 1 of a block, one per thread; every thread of the block calls it.
+// reused: the block calls it again with the same list.
+template <int DIM, int SYS, int VAR>
+__device__ __forceinline__ void cell_tile(const Grid& g, const double* __restrict__ S, const Work& w, long long p0,
+                                          double& wsx, double& wsy, Leftover& lo, bool reused) {
+  const long long p = p0 + threadIdx.x;
+  if (DIM == 1 && !g.pairs) {
+    if (p < g.plane) {
+      cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy);
+      cell_limiter<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), 0);
+    }
+    return;
+  }
+  if (reused) __syncthreads();
+  if (threadIdx.x == 0) lo.n = 0;
+  __syncthreads();
+  if (p < g.plane) {
+    if (!cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy)) {
+      const int k = atomicAdd(&lo.n, DIM);
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) lo.item[k + d] = (unsigned short)(threadIdx.x * 2 + d);
+    }
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < lo.n; k += kThreads) {
+    const int it = lo.item[k];
+    cell_limiter<DIM, SYS, VAR>(g, S, w, HW_IDX(p0 + (it >> 1), g.plane), it & 1);
   }
 }
 
 template <int DIM, int SYS, int VAR>
-__global__ void __launch_bounds__(kThreads) k_cell(Grid g, const double* __restrict__ S, Work w, int slot) {
-  const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
+__global__ void __launch_bounds__(kThreads, 4) k_cell(Grid g, const double* __restrict__ S, Work w, int slot) {
+  __shared__ Leftover lo;
   double wsx = 0.0, wsy = 0.0;
-  if (p < g.plane) cell_body<DIM, SYS, VAR>(g, S, w, p, wsx, wsy);
+  cell_tile<DIM, SYS, VAR>(g, S, w, (long long)blockIdx.x * kThreads, wsx, wsy, lo, false);
   block_max2(wsx, wsy, w.alpha + slot * w.astride);
 }
 
@@ -454,9 +622,11 @@ __device__ __forceinline__ void r1_face_states(const double (&Uq)[4][NC], const 
 
 // ---------------------------------------------------------------------------------------------
 // Face work of one stage: face f of direction dir (x faces: f = j (nx+1) + i; y faces:
-// f = j nx + i), alpha = the LF coefficient of that direction.
-template <int DIM, int SYS, int VAR = 0>
-__device__ __forceinline__ void face_body(const Grid& g, const double* __restrict__ S, const Work& w, int dir,
+// f = j nx + i), alpha = the LF coefficient of that direction.  PAIR: the nonlinear part of the
+// interpolation in pairs (hweno_pair.cuh); returns false, having written nothing, where the FP64
+// weights are needed.
+template <int DIM, int SYS, int VAR, bool PAIR>
+__device__ __forceinline__ bool face_body(const Grid& g, const double* __restrict__ S, const Work& w, int dir,
                                           long long f, double alpha) {
   using T = Traits<DIM, SYS>;
   constexpr int NC = T::NC, NG = T::NG;
@@ -484,7 +654,42 @@ __device__ __forceinline__ void face_body(const Grid& g, const double* __restric
     pc[q] = HW_IDX(dir == 0 ? (long long)line * g.nx + a : (long long)a * g.nx + line, plane);
   }
   const int fown = dir == 0 ? 1 : 2, foth = dir == 0 ? 2 : 1;
+  // local LF: the larger spectral radius of the two cells of the face
+  if (VAR && (g.flags & FLAG_ALPHA_LOCAL)) {
+    const double al = fixed[1] ? g.fixA[fside[1]] : w.WS[dir * plane + pc[1]];
+    const double ar = fixed[2] ? g.fixA[fside[2]] : w.WS[dir * plane + pc[2]];
+    alpha = fmax(al, ar);
+  }
+  const double* nod = w.NOD + (long long)dir * NG * NC * plane;
+  double* out = dir == 0 ? w.FX : w.FY;
+  const long long oplane = dir == 0 ? (long long)g.ny * (g.nx + 1) : (long long)(g.ny + 1) * g.nx;
+  const long long fo = HW_IDX(dir == 0 ? (long long)line * (g.nx + 1) + fa : (long long)fa * g.nx + line, oplane);
+  if (DIM == 2) {
+    // Eq. (mixed), linear in the nodal values: independent of everything below.  Nodal values of
+    // mirrored neighbours (normal frame): f and the mixed value change sign except for the normal
+    // momentum, the normal-derivative flux changes sign only for the normal momentum.
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      double o[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        o[q] = neg_if(nod[(2 * NC + k) * plane + pc[q]], refl[q] && k != 1);
+        if (VAR && fixed[q]) o[q] = 0.0;
+      }
+      const int ko = SYS == SYS_EULER && dir == 1 && (k == 1 || k == 2) ? 3 - k : k;
+      out[(foth * NC + ko) * oplane + fo] = fma(7.0 / 12.0, fu.add(o[1], o[2]), (-1.0 / 12.0) * fu.add(o[0], o[3]));
+    }
+  }
+  const double a_adv = dir == 0 ? g.ax : g.ay;
+  const P2 ih = p_const<float>(g.pg.ih[dir]);
   double Um[NC], Up[NC], Dm[NC], Dp[NC];
+  // Lax-Friedrichs fluxes (Eq. flux-LF): FS/2 + vf and HS/2 + vh, with FS = f(U^-) + f(U^+),
+  // vf = -alpha (U^+ - U^-)/2, HS and vh likewise from f'(U) D and D.  Where the two states of an
+  // Euler face are close (PAIR, and the near faces of R2), FS and HS are the flux and the Jacobian
+  // product of the sums of the states and derivatives (both are homogeneous of degree one), and what
+  // the mean of the two fluxes differs by joins vf and vh (p_flux_pair): half of the flux arithmetic.
+  double FS[NC], HS[NC], vf[NC], vh[NC];
+  bool summed = false;
   if (VAR == 2) {
     // R2: the face states were formed per cell (the low and high ghosts by k_r2_ghost)
     const double* FSd = w.FS + (long long)dir * 4 * NC * plane;
@@ -518,69 +723,145 @@ __device__ __forceinline__ void face_body(const Grid& g, const double* __restric
       }
       if (VAR && fixed[q]) load_fixed<NC, SYS>(g, fside[q], dir, Uq[q], Zq[q]);
     }
-    // characteristic fields at the face: Roe average of the two adjacent cells
-    Eig<NC> e;
-    if (SYS == SYS_EULER) {
-      const int ou = dir == 0 ? 1 : 2, ov = dir == 0 ? 2 : 1;
-      const int oh = DIM == 2 ? 3 : 2;
-      double sl = w.PRIM[pc[1]], sr = w.PRIM[pc[2]];
-      // a mirrored neighbour has the opposite normal velocity
-      double ul = neg_if(w.PRIM[ou * plane + pc[1]], refl[1]);
-      double ur = neg_if(w.PRIM[ou * plane + pc[2]], refl[2]);
-      double vl = 0, vr = 0;
-      if (DIM == 2) {
-        vl = w.PRIM[ov * plane + pc[1]];
-        vr = w.PRIM[ov * plane + pc[2]];
+    if (PAIR) {
+      double dU[3][NC];
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int k = 0; k < NC; ++k) dU[q][k] = fu.sub(Uq[q + 1][k], Uq[q][k]);
+      // the Hermite derivatives of Eq. (P'xi), which are linear in the stencil, and the linear parts of
+      // the interface values less the centre values; for the Euler equations the sums of both sides,
+      // the values' linear part among the pairs
+      const double k21 = g.uvd[dir][0], k3 = g.uvd[dir][1], l3 = g.l3[dir], l9 = g.l9[dir];
+      double Us[NC], Ds[NC], da[NC], zo[NC], zi[NC];
+      if (SYS == SYS_EULER) {
+        const double k42 = 2.0 * k21;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+          Us[k] = fu.add(Uq[1][k], Uq[2][k]);
+          da[k] = fu.sub(dU[0][k], dU[2][k]);
+          zo[k] = fu.sub(Zq[3][k], Zq[0][k]);
+          zi[k] = fu.sub(Zq[2][k], Zq[1][k]);
+          Ds[k] = fma(k42, dU[1][k],
+                      fma(-k3, fu.add(dU[0][k], dU[2][k]),
+                          fma(0.0625, fu.add(Zq[0][k], Zq[3][k]), -0.1875 * fu.add(Zq[1][k], Zq[2][k]))));
+        }
+      } else {
+        Um[0] = fma(0.125, dU[0][0], fma(0.5625, dU[1][0], fma(-l3, Zq[0][0], -l9 * Zq[2][0])));
+        Up[0] = fma(-0.125, dU[2][0], fma(-0.5625, dU[1][0], fma(l3, Zq[3][0], l9 * Zq[1][0])));
+        Dm[0] = fma(k21, dU[1][0], fma(-k3, dU[0][0], fma(0.0625, Zq[0][0], -0.1875 * Zq[2][0])));
+        Dp[0] = fma(k21, dU[1][0], fma(-k3, dU[2][0], fma(-0.1875, Zq[1][0], 0.0625 * Zq[3][0])));
       }
-      double Hl = w.PRIM[oh * plane + pc[1]], Hr = w.PRIM[oh * plane + pc[2]];
-      if (VAR && fixed[1]) {
-        const double* P = g.fixP[fside[1]];
-        sl = P[0];
-        ul = P[ou];
-        if (DIM == 2) vl = P[ov];
-        Hl = P[oh];
+      EigP<NC, F2> e;
+      if (SYS == SYS_EULER) {
+        // Roe average of the two adjacent cells from their primitives; a mirrored neighbour has the
+        // opposite normal velocity
+        P4 c[2][NC];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+#pragma unroll
+          for (int k = 0; k < NC; ++k) {
+            const int kn = NC == 4 && dir == 1 && (k == 1 || k == 2) ? 3 - k : k;
+            const float2 t = w.PRIM[kn * plane + pc[1 + q]];
+            P2 x = P2{t.x, t.y};
+            if (VAR && fixed[1 + q]) x = p_from(g.fixP[fside[1 + q]][kn]);
+            if (k == 1 && refl[1 + q]) x = p_neg(x);
+            c[q][k] = p_pack(x, x);
+          }
+        }
+        e.setup_roe(c[0], c[1], p_const<F2>(g.pg.gm1));
       }
-      if (VAR && fixed[2]) {
-        const double* P = g.fixP[fside[2]];
-        sr = P[0];
-        ur = P[ou];
-        if (DIM == 2) vr = P[ov];
-        Hr = P[oh];
+      P4 n[NC];
+      P2 sum[NC], dif[NC], hdif[NC];
+      float size[NC];
+      if (!p_face<NC, SYS>(dU, Zq, da, zo, zi, e, g.pg, dir, n, sum, dif, hdif, size)) return false;
+      if (SYS == SYS_EULER) {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+          Us[k] = fu.add(Us[k], fu.add(d_from(sum[k].h), d_from(sum[k].l)));
+        }
+        if (!p_flux_pair<NC>(Us, Ds, dif, hdif, size, alpha, ih, g.pg, fu, vf, vh)) return false;
+        Phys<DIM, SYS>::flux_jvp(Us, Ds, FS, HS, a_adv, g.gm1, fu);
+        summed = true;
+      } else {
+        const P2 a = p_lane0(n[0]), b = p_lane1(n[0]);
+        Um[0] = fu.add(Uq[1][0], fu.add(Um[0], fu.add(d_from(a.h), d_from(a.l))));
+        Up[0] = fu.add(Uq[2][0], fu.add(Up[0], fu.add(d_from(b.h), d_from(b.l))));
       }
-      const double iw = rcp(fu.add(sl, sr), fu);
-      const double ub = fu.mul(fma(sl, ul, fu.mul(sr, ur)), iw);
-      const double vb = DIM == 2 ? fu.mul(fma(sl, vl, fu.mul(sr, vr)), iw) : 0.0;
-      const double Hb = fu.mul(fma(sl, Hl, fu.mul(sr, Hr)), iw);
-      const double c2 = g.gm1 * fma(-0.5, DIM == 2 ? fma(ub, ub, fu.mul(vb, vb)) : fu.mul(ub, ub), Hb);
-      const double ic = rsqrt(c2);
-      e.setup(ub, vb, Hb, fu.mul(c2, ic), ic, g.gm1);
+    } else {
+      // characteristic fields at the face: Roe average of the two adjacent cells
+      Eig<NC> e;
+      if (SYS == SYS_EULER) {
+        double sq[2], uq[2], vq[2], Hq[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const double* U = Uq[1 + q];
+          if (DIM == 1 && !g.pairs) {
+            const double* P = reinterpret_cast<const double*>(w.PRIM);
+            const bool fx = VAR && fixed[1 + q];
+            const double* F = g.fixP[fside[1 + q]];
+            sq[q] = fx ? F[0] : P[pc[1 + q]];
+            uq[q] = neg_if(fx ? F[1] : P[plane + pc[1 + q]], refl[1 + q]);
+            Hq[q] = fx ? F[2] : P[2 * plane + pc[1 + q]];
+            vq[q] = 0.0;
+            continue;
+          }
+          const double ir = rcp(U[0], fu);
+          uq[q] = fu.mul(U[1], ir);
+          vq[q] = DIM == 2 ? fu.mul(U[2], ir) : 0.0;
+          const double ke = DIM == 2 ? fma(U[1], uq[q], fu.mul(U[2], vq[q])) : fu.mul(U[1], uq[q]);
+          Hq[q] = fu.mul(fu.add(U[NC - 1], g.gm1 * fma(-0.5, ke, U[NC - 1])), ir);
+          sq[q] = sqrt_fast(U[0], fu);
+        }
+        const double iw = rcp(fu.add(sq[0], sq[1]), fu);
+        const double ub = fu.mul(fma(sq[0], uq[0], fu.mul(sq[1], uq[1])), iw);
+        const double vb = DIM == 2 ? fu.mul(fma(sq[0], vq[0], fu.mul(sq[1], vq[1])), iw) : 0.0;
+        const double Hb = fu.mul(fma(sq[0], Hq[0], fu.mul(sq[1], Hq[1])), iw);
+        const double c2 = g.gm1 * fma(-0.5, DIM == 2 ? fma(ub, ub, fu.mul(vb, vb)) : fu.mul(ub, ub), Hb);
+        const double ic = rsqrt_fast(c2, fu);
+        e.setup(ub, vb, Hb, fu.mul(c2, ic), ic, g.gm1);
+      }
+      if (VAR && (g.flags & FLAG_V_WEIGHTED))
+        r1_face_states<NC, SYS, true>(Uq, Zq, e, g, dir, Um, Up, Dm, Dp, fu);
+      else
+        r1_face_states<NC, SYS, false>(Uq, Zq, e, g, dir, Um, Up, Dm, Dp, fu);
     }
-    if (VAR && (g.flags & FLAG_V_WEIGHTED))
-      r1_face_states<NC, SYS, true>(Uq, Zq, e, g, dir, Um, Up, Dm, Dp, fu);
-    else
-      r1_face_states<NC, SYS, false>(Uq, Zq, e, g, dir, Um, Up, Dm, Dp, fu);
   }
-  // local LF: the larger spectral radius of the two cells of the face
-  if (VAR && (g.flags & FLAG_ALPHA_LOCAL)) {
-    const double al = fixed[1] ? g.fixA[fside[1]] : w.WS[dir * plane + pc[1]];
-    const double ar = fixed[2] ? g.fixA[fside[2]] : w.WS[dir * plane + pc[2]];
-    alpha = fmax(al, ar);
+  if (VAR == 2) {
+    double Us[NC], Ds[NC];
+    P2 dif[NC], hdif[NC];
+    float size[NC];
+    const P2 h = p_const<float>(g.pg.h[dir]);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      Us[k] = fu.add(Um[k], Up[k]);
+      Ds[k] = fu.add(Dm[k], Dp[k]);
+      dif[k] = p_from(fu.sub(Up[k], Um[k]));
+      hdif[k] = p_mul(h, p_from(fu.sub(Dp[k], Dm[k])));
+      size[k] = p_from(Ds[k]).h * h.h;
+    }
+    if (p_flux_pair<NC>(Us, Ds, dif, hdif, size, alpha, ih, g.pg, fu, vf, vh)) {
+      Phys<DIM, SYS>::flux_jvp(Us, Ds, FS, HS, a_adv, g.gm1, fu);
+      summed = true;
+    }
   }
-  // Lax-Friedrichs fluxes at the interpolated states (Eq. flux-LF)
-  const double a_adv = dir == 0 ? g.ax : g.ay;
-  double FUm[NC], FUp[NC], HDm[NC], HDp[NC];
-  Phys<DIM, SYS>::flux_jvp(Um, Dm, FUm, HDm, a_adv, g.gm1, fu);
-  Phys<DIM, SYS>::flux_jvp(Up, Dp, FUp, HDp, a_adv, g.gm1, fu);
-  const double* nod = w.NOD + (long long)dir * NG * NC * plane;
-  double* out = dir == 0 ? w.FX : w.FY;
-  const long long oplane = dir == 0 ? (long long)g.ny * (g.nx + 1) : (long long)(g.ny + 1) * g.nx;
-  const long long fo = HW_IDX(dir == 0 ? (long long)line * (g.nx + 1) + fa : (long long)fa * g.nx + line, oplane);
+  if (!summed) {
+    double FUm[NC], FUp[NC], HDm[NC], HDp[NC];
+    Phys<DIM, SYS>::flux_jvp(Um, Dm, FUm, HDm, a_adv, g.gm1, fu);
+    Phys<DIM, SYS>::flux_jvp(Up, Dp, FUp, HDp, a_adv, g.gm1, fu);
+    const double ma = -0.5 * alpha;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      FS[k] = fu.add(FUm[k], FUp[k]);
+      HS[k] = fu.add(HDm[k], HDp[k]);
+      vf[k] = fu.mul(ma, fu.sub(Up[k], Um[k]));
+      vh[k] = fu.mul(ma, fu.sub(Dp[k], Dm[k]));
+    }
+  }
   const bool cd2 = VAR && (g.flags & FLAG_CD2) != 0;
-  double fh[NC], hh[NC], mh[NC];
+  double fh[NC], hh[NC];
 #pragma unroll
   for (int k = 0; k < NC; ++k) {
-    // nodal values of mirrored neighbours (normal frame): f and the mixed value change sign except
-    // for the normal momentum, the normal-derivative flux changes sign only for the normal momentum
     const bool nm = k == 1;
     const bool s0 = refl[0] && !nm, s1 = refl[1] && !nm, s2 = refl[2] && !nm, s3 = refl[3] && !nm;
     double f0 = neg_if(nod[k * plane + pc[0]], s0), f1 = neg_if(nod[k * plane + pc[1]], s1);
@@ -599,55 +880,63 @@ __device__ __forceinline__ void face_body(const Grid& g, const double* __restric
     }
     double Df, Dh;
     if (cd2) {
-      // D-terms (Eqs. Cd-2, DfDh)
-      Df = fma(DCoef2::cf, fu.add(fu.sub(f0, f1), fu.sub(f3, f2)), g.c2h[dir] * fu.sub(ha, hb));
-      Dh = fma(g.e2fih[dir], fu.sub(f0, f3), fma(g.e2gih[dir], fu.sub(f1, f2), DCoef2::eh * fu.add(ha, hb)));
+      // D-terms (Eqs. Cd-2, DfDh), with the viscous part
+      Df = fma(DCoef2::cf, fu.add(fu.sub(f0, f1), fu.sub(f3, f2)), fma(g.c2h[dir], fu.sub(ha, hb), vf[k]));
+      Dh = fma(g.e2fih[dir], fu.sub(f0, f3), fma(g.e2gih[dir], fu.sub(f1, f2), fma(DCoef2::eh, fu.add(ha, hb), vh[k])));
     } else {
-      // D-terms (Eqs. Cd-1, DfDh)
-      Df = fma(DCoef::cf, fu.add(fu.sub(f0, f1), fu.sub(f3, f2)), g.chh[dir] * fu.sub(ha, hb));
-      Dh = fma(g.efih[dir], fu.sub(f0, f3), fma(g.egih[dir], fu.sub(f2, f1), DCoef::eh * fu.add(ha, hb)));
+      // D-terms (Eqs. Cd-1, DfDh), with the viscous part
+      Df = fma(DCoef::cf, fu.add(fu.sub(f0, f1), fu.sub(f3, f2)), fma(g.chh[dir], fu.sub(ha, hb), vf[k]));
+      Dh = fma(g.efih[dir], fu.sub(f0, f3), fma(g.egih[dir], fu.sub(f2, f1), fma(DCoef::eh, fu.add(ha, hb), vh[k])));
     }
-    fh[k] = fma(0.5, fma(-alpha, fu.sub(Up[k], Um[k]), fu.add(FUm[k], FUp[k])), Df);
-    hh[k] = fma(0.5, fma(-alpha, fu.sub(Dp[k], Dm[k]), fu.add(HDm[k], HDp[k])), Dh);
-    if (DIM == 2) {
-      double o0 = neg_if(nod[(2 * NC + k) * plane + pc[0]], s0);
-      double o1 = neg_if(nod[(2 * NC + k) * plane + pc[1]], s1);
-      double o2 = neg_if(nod[(2 * NC + k) * plane + pc[2]], s2);
-      double o3 = neg_if(nod[(2 * NC + k) * plane + pc[3]], s3);
-      if (VAR) {
-        if (fixed[0]) o0 = 0.0;
-        if (fixed[1]) o1 = 0.0;
-        if (fixed[2]) o2 = 0.0;
-        if (fixed[3]) o3 = 0.0;
-      }
-      // Eq. (mixed)
-      mh[k] = fma(7.0 / 12.0, fu.add(o1, o2), (-1.0 / 12.0) * fu.add(o0, o3));
-    }
+    fh[k] = fma(0.5, FS[k], Df);
+    hh[k] = fma(0.5, HS[k], Dh);
   }
   if (SYS == SYS_EULER && dir == 1) {
     swap_frame<NC>(fh);
     swap_frame<NC>(hh);
-    swap_frame<NC>(mh);
   }
 #pragma unroll
   for (int k = 0; k < NC; ++k) {
     out[k * oplane + fo] = fh[k];
     out[(fown * NC + k) * oplane + fo] = hh[k];
-    if (DIM == 2) out[(foth * NC + k) * oplane + fo] = mh[k];
   }
+  return true;
 }
 
-// 2D: three blocks of 128 per SM, so that the stencil constants of the direction (StencilK) stay in
-// registers; 1D: four
+// The faces f0 .. f0 + kThreads - 1 (of nf) of direction dir, one per thread; every thread of the
+// block calls it.  reused: as cell_tile.
 template <int DIM, int SYS, int VAR>
-__global__ void __launch_bounds__(kThreads, DIM == 2 ? 3 : 4) k_face(Grid g, const double* __restrict__ S, Work w,
-                                                                    int slot) {
+__device__ __forceinline__ void face_tile(const Grid& g, const double* __restrict__ S, const Work& w, int dir,
+                                          long long f0, long long nf, double alpha, Leftover& lo, bool reused) {
+  const long long f = f0 + threadIdx.x;
+  // R2: only the fluxes (k_cell formed the face states); the weighted derivative needs the weights
+  // themselves
+  if (VAR == 2 || !g.pairs || (VAR && (g.flags & FLAG_V_WEIGHTED))) {
+    if (f < nf) face_body<DIM, SYS, VAR, false>(g, S, w, dir, f, alpha);
+    return;
+  }
+  if (reused) __syncthreads();
+  if (threadIdx.x == 0) lo.n = 0;
+  __syncthreads();
+  if (f < nf && !face_body<DIM, SYS, VAR, true>(g, S, w, dir, f, alpha))
+    lo.item[atomicAdd(&lo.n, 1)] = (unsigned short)threadIdx.x;
+  __syncthreads();
+  for (int k = threadIdx.x; k < lo.n; k += kThreads)
+    face_body<DIM, SYS, VAR, false>(g, S, w, dir, f0 + lo.item[k], alpha);
+}
+
+// Bound by the FP64 pipe (77 % busy; 165 FP64 instructions per 2D Euler face, 666 with the FP64 weights),
+// with the latency of the pairs' FP32 work between: four blocks of 128 per SM (128 registers, some
+// spilled) cover it better than three (2D Euler 2048^2 with k_cell likewise: 4.70 against 4.75 ms per
+// stage) or five (4.94 ms).
+template <int DIM, int SYS, int VAR>
+__global__ void __launch_bounds__(kThreads, 4) k_face(Grid g, const double* __restrict__ S, Work w, int slot) {
+  __shared__ Leftover lo;
   const int dir = blockIdx.y;
   const int n = dir == 0 ? g.nx : g.ny;
   const int nlines = dir == 0 ? g.ny : g.nx;
-  const long long f = (long long)blockIdx.x * kThreads + threadIdx.x;
-  if (f >= (long long)(n + 1) * nlines) return;
-  face_body<DIM, SYS, VAR>(g, S, w, dir, f, __longlong_as_double((long long)w.alpha[slot * w.astride + dir]));
+  face_tile<DIM, SYS, VAR>(g, S, w, dir, (long long)blockIdx.x * kThreads, (long long)(n + 1) * nlines,
+                           __longlong_as_double((long long)w.alpha[slot * w.astride + dir]), lo, false);
 }
 
 // ---------------------------------------------------------------------------------------------

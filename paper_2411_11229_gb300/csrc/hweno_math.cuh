@@ -26,11 +26,18 @@ struct Traits {
   static constexpr int NP = SYS == SYS_EULER ? (DIM == 2 ? 4 : 3) : 0;  // primitives per cell
 };
 
+// Constants of the pair arithmetic (hweno_pair.cuh), each as hi + lo of two FP32 numbers: the mesh
+// sizes and their inverses, gamma - 1, eps, 1/gamma1 and 1/d1; G = gamma0/gamma1, Gd = d0/d1.
+struct PairGrid {
+  float h[2][2], ih[2][2], gm1[2], eps[2], ig1[2], id1[2], G, Gd;
+};
+
 // Parameters shared by all kernels of one grid.
 struct Grid {
   int nx, ny;   // ny = 1 in 1D
   int bc;
   int flags;    // FLAG_* (read by the extended kernels only)
+  int pairs;    // whether the nonlinear part is taken in pairs where it may be (see hweno_host.cuh)
   long long plane;  // nx * ny
   double dx, dy, inv_dx, inv_dy;
   double gamma, gm1;
@@ -56,6 +63,10 @@ struct Grid {
   // the derivative at the face; ucsv = h/(4 d1), the limiter's derivative coefficient.
   double bS1[2], bN1[2], bS2[2], bN2[2], bT1, bT2;
   double udm[2][4], udp[2][4], uvd[2][2], ucsv[2];
+  // The linear scheme (hweno_pair.cuh holds the nonlinear part beside it): h/64 times 3 and 9, the
+  // derivative coefficients of p_0 at a face; 3/(4h), that of the cell difference in p_0' at a centre.
+  double l3[2], l9[2], l34[2];
+  PairGrid pg;
   double h[2], ih[2], chh[2], efih[2], egih[2], hih[2];
   // Extended scheme (read only by the kernels instantiated with VAR != 0):
   //   side: boundary type of x-low, x-high, y-low, y-high; grav: g of Eq. (euler2d-s);
@@ -104,7 +115,22 @@ __device__ __forceinline__ double rcp(double x, const FU& f = HW_PLAIN_FU) {
   const double e = fma(-x, r, f.one);
   return fma(r, fma(e, e, e), r);
 }
-__device__ __forceinline__ double sqr(double x) { return x * x; }
+// sqrt(x) and 1/sqrt(x) for normal, positive x, likewise: r = rsqrt.approx.ftz.f64, e = 1 - x r^2, and
+// (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + ...: five FP64 instructions each, against 12 slots of the FP64
+// pipe for sqrt() and 9 for rsqrt().  NaN for x <= 0.
+__device__ __forceinline__ double rsqrt_approx(double x) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return r;
+}
+__device__ __forceinline__ double sqrt_fast(double x, const FU& f) {
+  const double r = rsqrt_approx(x), s = f.mul(x, r), e = fma(-s, r, f.one);
+  return fma(s, f.mul(e, fma(0.375, e, 0.5)), s);
+}
+__device__ __forceinline__ double rsqrt_fast(double x, const FU& f) {
+  const double r = rsqrt_approx(x), e = fma(-f.mul(x, r), r, f.one);
+  return fma(r, f.mul(e, fma(0.375, e, 0.5)), r);
+}
 
 // ---------------------------------------------------------------------------------------------
 // Smoothness indicators (Eq. GHYZ, explicit forms) of the stencil {i-1, i, i+1} from the cell
