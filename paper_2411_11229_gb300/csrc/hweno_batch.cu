@@ -44,12 +44,13 @@ struct BatchArgs {
 };
 
 template <int DIM>
-__device__ __forceinline__ void batch_cells(const BatchInst& I, long long p0, int tpi, int slot) {
-  __shared__ Leftover lo;
+__device__ __forceinline__ void batch_cells(const BatchInst& I, long long p0, int tpi, int slot, Leftover& lo,
+                                            const PairSlots& sm) {
   double wsx = 0.0, wsy = 0.0;
   for (int t = 0; t < tpi; ++t) {
     double a = 0.0, b = 0.0;
-    cell_tile<DIM, SYS_EULER, 0>(I.g, I.S, I.w, p0 + (long long)t * kThreads, a, b, lo, true);
+    cell_tile<DIM, SYS_EULER, 0>(I.g, I.S, I.w, p0 + (long long)t * kThreads, a, b, lo, sm,
+                                 true);
     wsx = speed_bits(a) > speed_bits(wsx) ? a : wsx;
     wsy = speed_bits(b) > speed_bits(wsy) ? b : wsy;
   }
@@ -58,12 +59,13 @@ __device__ __forceinline__ void batch_cells(const BatchInst& I, long long p0, in
 }
 
 template <int DIM>
-__device__ __forceinline__ void batch_faces(const BatchInst& I, int dir, long long f0, int tpi, int slot) {
+__device__ __forceinline__ void batch_faces(const BatchInst& I, int dir, long long f0, int tpi, int slot,
+                                            Leftover& lo, const PairSlots& sm) {
   const long long nf = dir == 0 ? (long long)(I.g.nx + 1) * I.g.ny : (long long)(I.g.ny + 1) * I.g.nx;
   const double alpha = __longlong_as_double((long long)I.w.alpha[slot * I.w.astride + dir]);
-  __shared__ Leftover lo;
   for (int t = 0; t < tpi; ++t)
-    face_tile<DIM, SYS_EULER, 0>(I.g, I.S, I.w, dir, f0 + (long long)t * kThreads, nf, alpha, lo, true);
+    face_tile<DIM, SYS_EULER, 0>(I.g, I.S, I.w, dir, f0 + (long long)t * kThreads, nf, alpha, lo,
+                                 sm, true);
 }
 
 template <int DIM>
@@ -83,24 +85,27 @@ __device__ __forceinline__ void batch_update(const BatchInst& I, long long p0, i
 
 // One Runge-Kutta stage of every instance.  Launched cooperatively with every block resident.
 __global__ void __launch_bounds__(kThreads) k_batch_stage(BatchArgs a) {
+  __shared__ Leftover lo;
+  __shared__ ulonglong2 slots[kStencilSlots * kThreads];
+  const PairSlots sm{slots + threadIdx.x};
   cg::grid_group grid = cg::this_grid();
   const long long span = (long long)kThreads * a.tiles_per_item;
   for (int it = blockIdx.x; it < a.ncells; it += gridDim.x) {
     const int2 c = a.cells[it];
     const BatchInst& I = a.inst[HW_IDX(c.x, a.ninst)];
     if (I.dim == 1)
-      batch_cells<1>(I, c.y * span, a.tiles_per_item, a.slot);
+      batch_cells<1>(I, c.y * span, a.tiles_per_item, a.slot, lo, sm);
     else
-      batch_cells<2>(I, c.y * span, a.tiles_per_item, a.slot);
+      batch_cells<2>(I, c.y * span, a.tiles_per_item, a.slot, lo, sm);
   }
   grid.sync();
   for (int it = blockIdx.x; it < a.nfaces; it += gridDim.x) {
     const int4 f = a.faces[it];
     const BatchInst& I = a.inst[HW_IDX(f.x, a.ninst)];
     if (I.dim == 1)
-      batch_faces<1>(I, 0, f.z * span, a.tiles_per_item, a.slot);
+      batch_faces<1>(I, 0, f.z * span, a.tiles_per_item, a.slot, lo, sm);
     else
-      batch_faces<2>(I, f.y, f.z * span, a.tiles_per_item, a.slot);
+      batch_faces<2>(I, f.y, f.z * span, a.tiles_per_item, a.slot, lo, sm);
   }
   grid.sync();
   for (int it = blockIdx.x; it < a.ncells; it += gridDim.x) {
@@ -118,29 +123,35 @@ __global__ void __launch_bounds__(kThreads) k_batch_stage(BatchArgs a) {
 // stream order replaces the grid barriers.
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_batch_cells(BatchArgs a) {
+  __shared__ Leftover lo;
+  __shared__ ulonglong2 slots[4 * Traits<DIM, SYS_EULER>::NC * kThreads];
+  const PairSlots sm{slots + threadIdx.x};
   const long long span = (long long)kThreads * a.tiles_per_item;
-  const int lo = DIM == 2 ? 0 : a.ncells2, hi = DIM == 2 ? a.ncells2 : a.ncells;
-  for (int it = lo + blockIdx.x; it < hi; it += gridDim.x) {
+  const int first = DIM == 2 ? 0 : a.ncells2, last = DIM == 2 ? a.ncells2 : a.ncells;
+  for (int it = first + blockIdx.x; it < last; it += gridDim.x) {
     const int2 c = a.cells[it];
-    batch_cells<DIM>(a.inst[HW_IDX(c.x, a.ninst)], c.y * span, a.tiles_per_item, a.slot);
+    batch_cells<DIM>(a.inst[HW_IDX(c.x, a.ninst)], c.y * span, a.tiles_per_item, a.slot, lo, sm);
   }
 }
 
 template <int DIM>
 __global__ void __launch_bounds__(kThreads, 3) k_batch_faces(BatchArgs a) {
+  __shared__ Leftover lo;
+  __shared__ ulonglong2 slots[4 * Traits<DIM, SYS_EULER>::NC * kThreads];
+  const PairSlots sm{slots + threadIdx.x};
   const long long span = (long long)kThreads * a.tiles_per_item;
-  const int lo = DIM == 2 ? 0 : a.nfaces2, hi = DIM == 2 ? a.nfaces2 : a.nfaces;
-  for (int it = lo + blockIdx.x; it < hi; it += gridDim.x) {
+  const int first = DIM == 2 ? 0 : a.nfaces2, last = DIM == 2 ? a.nfaces2 : a.nfaces;
+  for (int it = first + blockIdx.x; it < last; it += gridDim.x) {
     const int4 f = a.faces[it];
-    batch_faces<DIM>(a.inst[HW_IDX(f.x, a.ninst)], DIM == 2 ? f.y : 0, f.z * span, a.tiles_per_item, a.slot);
+    batch_faces<DIM>(a.inst[HW_IDX(f.x, a.ninst)], DIM == 2 ? f.y : 0, f.z * span, a.tiles_per_item, a.slot, lo, sm);
   }
 }
 
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_batch_update(BatchArgs a) {
   const long long span = (long long)kThreads * a.tiles_per_item;
-  const int lo = DIM == 2 ? 0 : a.ncells2, hi = DIM == 2 ? a.ncells2 : a.ncells;
-  for (int it = lo + blockIdx.x; it < hi; it += gridDim.x) {
+  const int first = DIM == 2 ? 0 : a.ncells2, last = DIM == 2 ? a.ncells2 : a.ncells;
+  for (int it = first + blockIdx.x; it < last; it += gridDim.x) {
     const int2 c = a.cells[it];
     batch_update<DIM>(a.inst[HW_IDX(c.x, a.ninst)], c.y * span, a.tiles_per_item, a);
   }

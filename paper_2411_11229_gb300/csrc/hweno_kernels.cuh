@@ -54,8 +54,6 @@ struct Work {
   double* WS;
 };
 
-constexpr int kThreads = 128;
-constexpr int kSMs = 152;  // streaming multiprocessors of the GPU
 
 // The units of FU in thread registers: a zero read at a per-thread address of the zeroed slots
 // scal[4..7], so that the compiler can neither fold it nor keep it in a uniform register.
@@ -304,13 +302,12 @@ __device__ __forceinline__ void cell_limiter(const Grid& g, const double* __rest
 template <int DIM, int SYS, int VAR>
 __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* __restrict__ S, const Work& w,
                                                   long long p, int i, int j, const double* U, P2 pu, P2 pv, P2 pH,
-                                                  P2 pc2, const FU& f) {
+                                                  P2 pc2, const PairSlots& sm, const FU& f) {
   constexpr int NC = Traits<DIM, SYS>::NC;
   const long long plane = g.plane;
   // FP64: p_0'(x_i) = 3/4 (u_{i+1} - u_{i-1})/h - (v_{i-1} + v_{i+1})/4 and (R2) the linear parts of the
   // values and the derivatives at the two faces
   double md[DIM][NC], um[DIM][NC], up[DIM][NC], dm[DIM][NC], dp[DIM][NC];
-  P4 dU[2][NC], Z[2][NC];
   {
     P2 uc[NC], du[2][DIM][NC], z[2][DIM][NC];
 #pragma unroll
@@ -342,8 +339,8 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
     for (int q = 0; q < 2; ++q)
 #pragma unroll
       for (int k = 0; k < NC; ++k) {
-        dU[q][k] = p_pack(du[q][0][k], du[q][DIM - 1][k]);
-        Z[q][k] = p_pack(z[q][0][k], z[q][DIM - 1][k]);
+        sm.set(q * NC + k, p_pack(du[q][0][k], du[q][DIM - 1][k]));
+        sm.set((2 + q) * NC + k, p_pack(z[q][0][k], z[q][DIM - 1][k]));
       }
   }
   EigP<NC, F2> e;
@@ -353,7 +350,7 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
   }
   const P4 h = p_pack(p_const<float>(g.pg.h[0]), p_const<float>(g.pg.h[DIM - 1]));
   P4 nm[NC], np[NC], nt[NC];
-  if (!p_cell<NC, SYS, VAR == 2>(dU, Z, e, h, g.pg, nm, np, nt)) return false;
+  if (!p_cell<NC, SYS, VAR == 2>(sm, e, h, g.pg, nm, np, nt)) return false;
 #pragma unroll
   for (int d = 0; d < DIM; ++d) {
     const P2 ih = p_const<float>(g.pg.ih[d]);
@@ -387,7 +384,7 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
 // false where the modified derivatives are left to cell_limiter.
 template <int DIM, int SYS, int VAR = 0>
 __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restrict__ S, const Work& w, long long p,
-                                         double& wsx, double& wsy) {
+                                          double& wsx, double& wsy, const PairSlots& sm) {
   using T = Traits<DIM, SYS>;
   constexpr int NC = T::NC, NG = T::NG;
   const long long plane = g.plane;
@@ -505,7 +502,7 @@ __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restric
         w.PRIM[DIM * plane + plane + p] = make_float2(pH.h, pH.l);
       }
     }
-    return cell_limiter_pair<DIM, SYS, VAR>(g, S, w, p, i, j, U, pu, pv, pH, p_renorm(pc2), f);
+    return cell_limiter_pair<DIM, SYS, VAR>(g, S, w, p, i, j, U, pu, pv, pH, p_renorm(pc2), sm, f);
   }
 }
 
@@ -521,11 +518,12 @@ struct Leftover {
 // reused: the block calls it again with the same list.
 template <int DIM, int SYS, int VAR>
 __device__ __forceinline__ void cell_tile(const Grid& g, const double* __restrict__ S, const Work& w, long long p0,
-                                          double& wsx, double& wsy, Leftover& lo, bool reused) {
+                                          double& wsx, double& wsy, Leftover& lo, const PairSlots& sm,
+                                          bool reused) {
   const long long p = p0 + threadIdx.x;
   if (DIM == 1 && !g.pairs) {
     if (p < g.plane) {
-      cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy);
+      cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm);
       cell_limiter<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), 0);
     }
     return;
@@ -534,7 +532,7 @@ __device__ __forceinline__ void cell_tile(const Grid& g, const double* __restric
   if (threadIdx.x == 0) lo.n = 0;
   __syncthreads();
   if (p < g.plane) {
-    if (!cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy)) {
+    if (!cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm)) {
       const int k = atomicAdd(&lo.n, DIM);
 #pragma unroll
       for (int d = 0; d < DIM; ++d) lo.item[k + d] = (unsigned short)(threadIdx.x * 2 + d);
@@ -547,11 +545,15 @@ __device__ __forceinline__ void cell_tile(const Grid& g, const double* __restric
   }
 }
 
+// Bound by the FP64 pipe (85 % busy): 123 FP64 instructions per 2D Euler cell against 545 with the FP64
+// weights; 1024^2 0.24 ms per launch against 0.97 ms.
 template <int DIM, int SYS, int VAR>
 __global__ void __launch_bounds__(kThreads, 4) k_cell(Grid g, const double* __restrict__ S, Work w, int slot) {
   __shared__ Leftover lo;
+  __shared__ ulonglong2 slots[4 * Traits<DIM, SYS>::NC * kThreads];
   double wsx = 0.0, wsy = 0.0;
-  cell_tile<DIM, SYS, VAR>(g, S, w, (long long)blockIdx.x * kThreads, wsx, wsy, lo, false);
+  cell_tile<DIM, SYS, VAR>(g, S, w, (long long)blockIdx.x * kThreads, wsx, wsy, lo, PairSlots{slots + threadIdx.x},
+                           false);
   block_max2(wsx, wsy, w.alpha + slot * w.astride);
 }
 
@@ -627,7 +629,7 @@ __device__ __forceinline__ void r1_face_states(const double (&Uq)[4][NC], const 
 // weights are needed.
 template <int DIM, int SYS, int VAR, bool PAIR>
 __device__ __forceinline__ bool face_body(const Grid& g, const double* __restrict__ S, const Work& w, int dir,
-                                          long long f, double alpha) {
+                                          long long f, double alpha, const PairSlots& sm) {
   using T = Traits<DIM, SYS>;
   constexpr int NC = T::NC, NG = T::NG;
   const long long plane = g.plane;
@@ -774,7 +776,7 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
       P4 n[NC];
       P2 sum[NC], dif[NC], hdif[NC];
       float size[NC];
-      if (!p_face<NC, SYS>(dU, Zq, da, zo, zi, e, g.pg, dir, n, sum, dif, hdif, size)) return false;
+      if (!p_face<NC, SYS>(dU, Zq, da, zo, zi, e, g.pg, dir, sm, n, sum, dif, hdif, size)) return false;
       if (SYS == SYS_EULER) {
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
@@ -907,36 +909,41 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
 // block calls it.  reused: as cell_tile.
 template <int DIM, int SYS, int VAR>
 __device__ __forceinline__ void face_tile(const Grid& g, const double* __restrict__ S, const Work& w, int dir,
-                                          long long f0, long long nf, double alpha, Leftover& lo, bool reused) {
+                                          long long f0, long long nf, double alpha, Leftover& lo,
+                                          const PairSlots& sm, bool reused) {
   const long long f = f0 + threadIdx.x;
   // R2: only the fluxes (k_cell formed the face states); the weighted derivative needs the weights
   // themselves
   if (VAR == 2 || !g.pairs || (VAR && (g.flags & FLAG_V_WEIGHTED))) {
-    if (f < nf) face_body<DIM, SYS, VAR, false>(g, S, w, dir, f, alpha);
+    if (f < nf) face_body<DIM, SYS, VAR, false>(g, S, w, dir, f, alpha, sm);
     return;
   }
   if (reused) __syncthreads();
   if (threadIdx.x == 0) lo.n = 0;
   __syncthreads();
-  if (f < nf && !face_body<DIM, SYS, VAR, true>(g, S, w, dir, f, alpha))
+  if (f < nf && !face_body<DIM, SYS, VAR, true>(g, S, w, dir, f, alpha, sm))
     lo.item[atomicAdd(&lo.n, 1)] = (unsigned short)threadIdx.x;
   __syncthreads();
   for (int k = threadIdx.x; k < lo.n; k += kThreads)
-    face_body<DIM, SYS, VAR, false>(g, S, w, dir, f0 + lo.item[k], alpha);
+    face_body<DIM, SYS, VAR, false>(g, S, w, dir, f0 + lo.item[k], alpha, sm);
 }
 
-// Bound by the FP64 pipe (77 % busy; 165 FP64 instructions per 2D Euler face, 666 with the FP64 weights),
-// with the latency of the pairs' FP32 work between: four blocks of 128 per SM (128 registers, some
-// spilled) cover it better than three (2D Euler 2048^2 with k_cell likewise: 4.70 against 4.75 ms per
-// stage) or five (4.94 ms).
+// Bound by the FP64 pipe (86 % busy at 1024^2; about 170 FP64 instructions per 2D Euler face against 666
+// with the FP64 weights everywhere), with the latency of the pairs' FP32 work between: four blocks of 128
+// per SM (128 registers) cover it better than three or five (2D Euler 2048^2 with k_cell likewise: 4.70
+// against 4.75 and 4.94 ms per stage, before the pairs' loops).  2D Euler 1024^2: 0.70 ms per launch
+// against 2.33 ms with the FP64 weights.
 template <int DIM, int SYS, int VAR>
 __global__ void __launch_bounds__(kThreads, 4) k_face(Grid g, const double* __restrict__ S, Work w, int slot) {
   __shared__ Leftover lo;
+  constexpr bool kSlots = SYS == SYS_EULER && VAR != 2;  // scalar laws and R2's faces use none
+  __shared__ ulonglong2 slots[kSlots ? 4 * Traits<DIM, SYS>::NC * kThreads : 1];
   const int dir = blockIdx.y;
   const int n = dir == 0 ? g.nx : g.ny;
   const int nlines = dir == 0 ? g.ny : g.nx;
   face_tile<DIM, SYS, VAR>(g, S, w, dir, (long long)blockIdx.x * kThreads, (long long)(n + 1) * nlines,
-                           __longlong_as_double((long long)w.alpha[slot * w.astride + dir]), lo, false);
+                           __longlong_as_double((long long)w.alpha[slot * w.astride + dir]), lo,
+                           PairSlots{slots + (kSlots ? threadIdx.x : 0)}, false);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -13,6 +13,9 @@
 
 namespace hw {
 
+constexpr int kThreads = 128;  // of a block
+constexpr int kSMs = 152;      // streaming multiprocessors of the GPU
+
 enum { SYS_ADV = 0, SYS_BURGERS = 1, SYS_EULER = 2 };
 enum { BC_PERIODIC = 0, BC_TRANSMISSIVE = 1, BC_REFLECTIVE = 2, BC_FIXED = 3 };
 // scheme variants of the extended kernels (VAR != 0)

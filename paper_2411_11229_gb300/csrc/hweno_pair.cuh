@@ -365,6 +365,34 @@ __device__ __forceinline__ void p_prim(const P2* U, P2 gm1, P2& u, P2& v, P2& H,
   pr = p_mul(p, ir);
 }
 
+// A thread's pairs in shared memory, 16 bytes a slot: the arrays of the loops over vectors and
+// characteristic fields, which stay loops.  Unrolled, the kernels' code is several times the
+// instruction cache's reach and its fetches are waited for.  at: this thread's first slot.
+struct PairSlots {
+  ulonglong2* at;
+  __device__ __forceinline__ P4 get(int k) const {
+    const ulonglong2 t = at[k * kThreads];
+    return P4{F2{t.x}, F2{t.y}};
+  }
+  __device__ __forceinline__ void set(int k, P4 x) const { at[k * kThreads] = make_ulonglong2(x.h.v, x.l.v); }
+};
+constexpr int kStencilSlots = 16;  // four vectors of four components
+
+// Projects the four vectors of slots v NC + k in place.  A field that is small beside its vector comes
+// out of the products with h and l of like size: they are renormalised for the squares that follow.
+template <int NC>
+__device__ __forceinline__ void p_project_slots(const EigP<NC, F2>& e, const PairSlots& sm) {
+#pragma unroll 1
+  for (int v = 0; v < 4; ++v) {
+    P4 q[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) q[k] = sm.get(v * NC + k);
+    e.project(q, q);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) sm.set(v * NC + k, p_renorm(q[k]));
+  }
+}
+
 // Whether the corrections are finite: a denominator that left the FP32 range shows in them
 template <int NC>
 __device__ __forceinline__ bool p_finite(const P4* n) {
@@ -384,10 +412,11 @@ __device__ __forceinline__ bool p_finite(const P4* n) {
 // (zo) and Z2 - Z1 (zi), are taken in FP64.  Returns false where any field needs the FP64 weights.
 template <int NC, int SYS>
 __device__ __forceinline__ bool p_face(const double (&dU)[3][NC], const double (&Z)[4][NC], const double* da_,
-                                       const double* zo_, const double* zi_, const EigP<NC, F2>& e, const PairGrid& pg, int dir, P4* n, P2* sum, P2* dif, P2* hdif,
+                                       const double* zo_, const double* zi_, const EigP<NC, F2>& e,
+                                       const PairGrid& pg, int dir, const PairSlots& sm, P4* n, P2* sum, P2* dif, P2* hdif,
                                        float* size) {
   const P4 h = p_const<F2>(pg.h[dir]), eps = p_const<F2>(pg.eps), ig = p_const<F2>(pg.ig1);
-  P4 d1[NC], d2[NC], y1[NC], y2[NC];  // per side: the differences and end derivatives of its stencil
+  P4 d1, d2, y1, y2;  // a scalar law's, per side: the differences and end derivatives of its stencil
   {
     P2 d[3][NC], z[4][NC];
 #pragma unroll
@@ -428,27 +457,41 @@ __device__ __forceinline__ bool p_face(const double (&dU)[3][NC], const double (
         size[k] = fmaxf(fmaxf(fabsf(d[0][k].h), fmaxf(fabsf(d[1][k].h), fabsf(d[2][k].h))), a * pg.h[dir][0]);
       }
     }
+    if (SYS == SYS_EULER) {
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
-      d1[k] = p_pack(d[0][k], d[1][k]);
-      d2[k] = p_pack(d[1][k], d[2][k]);
-      y1[k] = p_pack(z[0][k], z[1][k]);
-      y2[k] = p_pack(z[2][k], z[3][k]);
+      for (int k = 0; k < NC; ++k) {
+        sm.set(0 * NC + k, p_pack(d[0][k], d[1][k]));
+        sm.set(1 * NC + k, p_pack(d[1][k], d[2][k]));
+        sm.set(2 * NC + k, p_pack(z[0][k], z[1][k]));
+        sm.set(3 * NC + k, p_pack(z[2][k], z[3][k]));
+      }
+    } else {
+      d1 = p_pack(d[0][0], d[1][0]);
+      d2 = p_pack(d[1][0], d[2][0]);
+      y1 = p_pack(z[0][0], z[1][0]);
+      y2 = p_pack(z[2][0], z[3][0]);
     }
-  }
-  if (SYS == SYS_EULER) {
-    e.project(d1, d1);
-    e.project(d2, d2);
-    e.project(y1, y1);
-    e.project(y2, y2);
   }
   P4 c[NC];
   bool ok = true;
+  if (SYS == SYS_EULER) {
+    p_project_slots<NC>(e, sm);
+#pragma unroll 1
+    for (int s = 0; s < NC; ++s) {
+      PStencil<F2> st;
+      d1 = sm.get(s);
+      d2 = sm.get(NC + s);
+      ok = p_stencil(d1, d2, sm.get(2 * NC + s), sm.get(3 * NC + s), p_add(p_sqr(d1), eps), p_add(p_sqr(d2), eps), h,
+                     st) &&
+           ok;
+      sm.set(s, p_face_values(st, ig, pg.G));
+    }
 #pragma unroll
-  for (int s = 0; s < NC; ++s) {
+    for (int s = 0; s < NC; ++s) c[s] = sm.get(s);
+  } else {
     PStencil<F2> st;
-    ok = p_stencil(d1[s], d2[s], y1[s], y2[s], p_add(p_sqr(d1[s]), eps), p_add(p_sqr(d2[s]), eps), h, st) && ok;
-    c[s] = p_face_values(st, ig, pg.G);
+    ok = p_stencil(d1, d2, y1, y2, p_add(p_sqr(d1), eps), p_add(p_sqr(d2), eps), h, st);
+    c[0] = p_face_values(st, ig, pg.G);
   }
   if (SYS == SYS_EULER) {
     e.back(c, n);
@@ -466,30 +509,34 @@ __device__ __forceinline__ bool p_face(const double (&dU)[3][NC], const double (
 
 // The corrections of one cell in both directions (lane d: direction d, in its normal frame; in 1D the
 // lanes are the same) from the cells i-1..i+1: nt of h times the modified derivative and, FACES (R2),
-// nm and np of the values at the right and the left face.  dU: differences, Z: end derivatives.
+// nm and np of the values at the right and the left face.  Slots: the two differences and the two end
+// derivatives.
 template <int NC, int SYS, bool FACES>
-__device__ __forceinline__ bool p_cell(P4 (&dU)[2][NC], P4 (&Z)[2][NC], const EigP<NC, F2>& e, P4 h,
-                                       const PairGrid& pg, P4* nm, P4* np, P4* nt) {
-  if (SYS == SYS_EULER) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      e.project(dU[q], dU[q]);
-      e.project(Z[q], Z[q]);
-    }
-  }
+__device__ __forceinline__ bool p_cell(const PairSlots& sm, const EigP<NC, F2>& e, P4 h, const PairGrid& pg, P4* nm,
+                                       P4* np, P4* nt) {
+  if (SYS == SYS_EULER) p_project_slots<NC>(e, sm);
   const P4 eps = p_const<F2>(pg.eps), ig = p_const<F2>(pg.ig1), id = p_const<F2>(pg.id1);
   P4 cm[NC], cp[NC], ct[NC];
   bool ok = true;
-#pragma unroll
+#pragma unroll 1
   for (int s = 0; s < NC; ++s) {
     PStencil<F2> st;
-    ok = p_stencil(dU[0][s], dU[1][s], Z[0][s], Z[1][s], p_add(p_sqr(dU[0][s]), eps), p_add(p_sqr(dU[1][s]), eps), h,
+    const P4 d1 = sm.get(s), d2 = sm.get(NC + s);
+    ok = p_stencil(d1, d2, sm.get(2 * NC + s), sm.get(3 * NC + s), p_add(p_sqr(d1), eps), p_add(p_sqr(d2), eps), h,
                    st) &&
          ok;
-    ct[s] = p_limited(st, id, pg.Gd);
+    sm.set(s, p_limited(st, id, pg.Gd));
     if (FACES) {
-      cm[s] = p_right_value(st, ig, pg.G);
-      cp[s] = p_left_value(st, ig, pg.G);
+      sm.set(NC + s, p_right_value(st, ig, pg.G));
+      sm.set(2 * NC + s, p_left_value(st, ig, pg.G));
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < NC; ++s) {
+    ct[s] = sm.get(s);
+    if (FACES) {
+      cm[s] = sm.get(NC + s);
+      cp[s] = sm.get(2 * NC + s);
     }
   }
   if (SYS == SYS_EULER) {
