@@ -15,8 +15,12 @@
 //                D-terms and mixed fluxes to the flux adjoints and the nodal flux VJPs, and adds
 //                the identity part of M.
 // Contributions are stored per face / per cell and gathered (no atomics: deterministic).
+// In 2D, k_adj_cell_pair and k_adj_face_pair form the same contributions with the transposes of the
+// nonlinear part in pairs (hweno_adjoint_pair.cuh) and list the cells and faces that need the FP64 weights
+// for k_adj_cell and k_adj_face.  1D grids are too small to fill the FP64 pipe and keep the FP64 kernels.
 #include <cmath>
 #include "hweno_adjoint.cuh"
+#include "hweno_adjoint_pair.cuh"
 #include "hweno_host.cuh"
 
 using namespace hwh;
@@ -28,7 +32,22 @@ struct AdjWork {
   double* CD;  // face contributions to the own-direction derivative, same layout
   double* CM;  // modified-derivative contributions: [dir][cell][3 U + 2 D][NC] (original frame)
   const double* scal;  // the handle's scalars; [4..7] are zero (read by fu_of)
+  // 2D: the cells and faces that k_adj_cell_pair and k_adj_face_pair leave to the FP64 kernels:
+  // count[0] cells * 2 + direction in cells, count[1] faces of both directions in faces
+  unsigned int* count;
+  unsigned int *cells, *faces;
 };
+
+// Appends v for the threads with add set; every thread of the warp calls it, at once per warp.
+__device__ __forceinline__ void list_append(unsigned int* count, unsigned int* list, unsigned int v, bool add) {
+  const unsigned int m = __ballot_sync(0xffffffffu, add);
+  if (m == 0u) return;
+  const int lane = threadIdx.x & 31, first = __ffs(m) - 1;
+  unsigned int at = 0u;
+  if (lane == first) at = atomicAdd(count, (unsigned int)__popc(m));
+  at = __shfl_sync(0xffffffffu, at, first) + __popc(m & ((1u << lane) - 1u));
+  if (add) list[at] = v;
+}
 
 template <int DIM>
 __device__ __forceinline__ long long nfaces_dir(const Grid& g, int dir) {
@@ -37,13 +56,10 @@ __device__ __forceinline__ long long nfaces_dir(const Grid& g, int dir) {
 
 // -------------------------------------------------------------------------------------------
 template <int DIM>
-__global__ void __launch_bounds__(kThreads) k_adj_cell(Grid g, const double* __restrict__ S, const double* __restrict__ muM,
-                                                       AdjWork aw) {
+__device__ __forceinline__ void adj_cell(const Grid& g, const double* __restrict__ S, const double* __restrict__ muM,
+                                         const AdjWork& aw, int d, long long p) {
   constexpr int NC = DIM == 1 ? 3 : 4;
-  const int d = blockIdx.y;
   const long long plane = g.plane;
-  const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
-  if (p >= plane) return;
   const int i = (int)(p % g.nx), j = (int)(p / g.nx);
   const int n = d == 0 ? g.nx : g.ny;
   const int a0 = d == 0 ? i : j;
@@ -164,17 +180,29 @@ __global__ void __launch_bounds__(kThreads) k_adj_cell(Grid g, const double* __r
   }
 }
 
+// 1D: every cell; 2D: the cells of the list
+template <int DIM>
+__global__ void __launch_bounds__(kThreads) k_adj_cell(Grid g, const double* __restrict__ S, const double* __restrict__ muM,
+                                                       AdjWork aw) {
+  long long k = (long long)blockIdx.x * kThreads + threadIdx.x;
+  if (DIM == 1) {
+    if (k < g.plane) adj_cell<1>(g, S, muM, aw, 0, k);
+    return;
+  }
+  const unsigned int n = aw.count[0];
+  for (; k < n; k += (long long)gridDim.x * kThreads) {
+    const unsigned int c = aw.cells[k];
+    adj_cell<DIM>(g, S, muM, aw, (int)(c & 1u), HW_IDX(c >> 1, g.plane));
+  }
+}
+
 // -------------------------------------------------------------------------------------------
 template <int DIM>
-__global__ void __launch_bounds__(kThreads) k_adj_face(Grid g, const double* __restrict__ S, const double* __restrict__ muL,
-                                                       AdjWork aw, const double* __restrict__ alpha2) {
+__device__ __forceinline__ void adj_face(const Grid& g, const double* __restrict__ S, const double* __restrict__ muL,
+                                         const AdjWork& aw, const double* __restrict__ alpha2, int dir, long long f) {
   constexpr int NC = DIM == 1 ? 3 : 4;
-  const int dir = blockIdx.y;
   const long long plane = g.plane;
   const int n = dir == 0 ? g.nx : g.ny;
-  const int nlines = dir == 0 ? g.ny : g.nx;
-  const long long f = (long long)blockIdx.x * kThreads + threadIdx.x;
-  if (f >= (long long)(n + 1) * nlines) return;
   int fa, line;
   if (dir == 0) {
     line = (int)(f / (n + 1));
@@ -381,6 +409,466 @@ __global__ void __launch_bounds__(kThreads) k_adj_face(Grid g, const double* __r
       aw.CD[base + q * NC + k] = Zqb[q][k];
     }
   }
+}
+
+// 1D: every face; 2D: the faces of the list
+template <int DIM>
+__global__ void __launch_bounds__(kThreads) k_adj_face(Grid g, const double* __restrict__ S, const double* __restrict__ muL,
+                                                       AdjWork aw, const double* __restrict__ alpha2) {
+  long long k = (long long)blockIdx.x * kThreads + threadIdx.x;
+  const long long nfx = (long long)(g.nx + 1) * g.ny;
+  if (DIM == 1) {
+    if (k < nfx) adj_face<1>(g, S, muL, aw, alpha2, 0, k);
+    return;
+  }
+  const unsigned int n = aw.count[1];
+  for (; k < n; k += (long long)gridDim.x * kThreads) {
+    const long long f = HW_IDX(aw.faces[k], nfx + (long long)(g.ny + 1) * g.nx);
+    adj_face<DIM>(g, S, muL, aw, alpha2, f < nfx ? 0 : 1, f < nfx ? f : f - nfx);
+  }
+}
+
+// -------------------------------------------------------------------------------------------
+// The pairs of a thread in shared memory (unrolled, k_adj_face_pair's 96 KB of instructions waited for
+// themselves: 5.2 of 14 stall cycles, 1.14 ms per 512^2 launch against 0.52 ms)
+// slots: vector v, component k; field s, vector v; one per field
+constexpr int kPairSlots = 36;
+__device__ __forceinline__ int slot_q(int v, int k) { return v * 4 + k; }
+__device__ __forceinline__ int slot_w(int s, int v) { return 16 + s * 4 + v; }
+__device__ __forceinline__ int slot_c(int s) { return 32 + s; }
+
+// The same contributions of a 2D cell (both directions: the lanes of its pairs) with the transpose of
+// the limiter's nonlinear part in pairs; false where the FP64 kernel is needed.
+__device__ __forceinline__ bool adj_cell_pair(const Grid& g, const double* __restrict__ S,
+                                              const double* __restrict__ muM, const AdjWork& aw, long long p,
+                                              const PairSlots& sm) {
+  constexpr int NC = 4;
+  const long long plane = g.plane;
+  const FU fu = fu_of(aw.scal);
+  const int i = (int)(p % g.nx), j = (int)(p / g.nx);
+  bool refl[2][2];
+  double ob[2][NC];
+  P4 U1[NC];
+  {
+    // the differences in FP64: the derivatives of the weights see them relative to themselves
+    P2 du[2][2][NC], z[2][2][NC];
+    double Uc[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) Uc[k] = S[k * plane + p];
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      const int n = d == 0 ? g.nx : g.ny, a0 = d == 0 ? i : j, fld = d == 0 ? 1 : 2;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {  // the neighbours i - 1, i + 1
+        const int ac = bc_map(a0 - 1 + 2 * q, n, g.bc, refl[d][q]);
+        const long long pc = HW_IDX(d == 0 ? (long long)j * g.nx + ac : (long long)ac * g.nx + i, plane);
+        double U[NC], D[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+          U[k] = S[k * plane + pc];
+          D[k] = S[(fld * NC + k) * plane + pc];
+        }
+        if (d == 1) {
+          swap_frame<NC>(U);
+          swap_frame<NC>(D);
+        }
+        mirror_U<NC>(U, refl[d][q]);
+        mirror_D<NC>(D, refl[d][q]);
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+          const double c = Uc[d == 1 && (k == 1 || k == 2) ? 3 - k : k];
+          du[q][d][k] = p_from(q == 0 ? fu.sub(c, U[k]) : fu.sub(U[k], c));
+          z[q][d][k] = p_from(D[k]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < NC; ++k) ob[d][k] = muM[(fld * NC + k) * plane + p];
+      if (d == 1) swap_frame<NC>(ob[d]);
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      U1[k] = p_pack(p_from(Uc[k]), p_from(Uc[k == 1 || k == 2 ? 3 - k : k]));
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        sm.set(slot_q(q, k), p_pack(du[q][0][k], du[q][1][k]));
+        sm.set(slot_q(2 + q, k), p_pack(z[q][0][k], z[q][1][k]));
+      }
+    }
+  }
+  unsigned int big = 0u;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) big = max(big, max(seed_bits(ob[0][k]), seed_bits(ob[1][k])));
+  int sh;
+  if (!seed_scale(big, sh)) return false;
+  const P4 gm1 = p_const<F2>(g.pg.gm1);
+  // the cell's characteristic fields
+  const P4 ir = p_rcp(U1[0]), u = p_mul(U1[1], ir), v = p_mul(U1[2], ir);
+  const P4 pr = p_mul(gm1, p_sub(U1[3], p_scale(p_add(p_mul(U1[1], u), p_mul(U1[2], v)), 0.5f)));
+  const P4 ep = p_add(U1[3], pr), prir = p_mul(pr, ir);
+  EigP<NC, F2> e;
+  e.setup(u, v, p_mul(ep, ir), p_renorm(p_add(prir, p_mul(gm1, prir))), gm1);
+  // seeds: of h v~ in the characteristic fields
+  const P4 h = p_pack(p_const<float>(g.pg.h[0]), p_const<float>(g.pg.h[1]));
+  const P4 ih = p_pack(p_const<float>(g.pg.ih[0]), p_const<float>(g.pg.ih[1]));
+  P4 qb[NC], c[NC];
+#pragma unroll
+  for (int k = 0; k < NC; ++k) qb[k] = p_mul(p_pack(p_from_scaled(ob[0][k], sh), p_from_scaled(ob[1][k], sh)), ih);
+  p_back_t(e, qb, c);
+#pragma unroll
+  for (int s = 0; s < NC; ++s) sm.set(slot_c(s), c[s]);
+#pragma unroll 1
+  for (int v = 0; v < 4; ++v) {
+    P4 q[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) q[k] = sm.get(slot_q(v, k));
+    e.project(q, q);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) sm.set(slot_w(k, v), p_renorm(q[k]));
+  }
+  const P4 eps = p_const<F2>(g.pg.eps), id = p_const<F2>(g.pg.id1);
+  bool ok = true;
+#pragma unroll 1
+  for (int s = 0; s < NC; ++s) {
+    P4 w0, w1, w2, w3;
+    sm.set(slot_c(s), p_correction_vjp<CORR_LIMITED>(sm.get(slot_w(s, 0)), sm.get(slot_w(s, 1)), sm.get(slot_w(s, 2)),
+                                                     sm.get(slot_w(s, 3)), h, eps, id, g.pg.Gd, sm.get(slot_c(s)), w0,
+                                                     w1, w2, w3, ok));
+    sm.set(slot_w(s, 0), w0);
+    sm.set(slot_w(s, 1), w1);
+    sm.set(slot_w(s, 2), w2);
+    sm.set(slot_w(s, 3), w3);
+  }
+#pragma unroll
+  for (int s = 0; s < NC; ++s) c[s] = sm.get(slot_c(s));
+  if (!ok || !p_finite<NC>(c)) return false;
+  EigPBar<F2> eb;
+  eb.zero();
+  p_back_eig(c, qb, eb);
+#pragma unroll 1
+  for (int v = 0; v < 4; ++v) {
+    P4 q[NC], wb[NC], t[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      q[k] = sm.get(slot_q(v, k));
+      wb[k] = sm.get(slot_w(k, v));
+    }
+    p_project_vjp(e, q, wb, t, eb);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) sm.set(slot_q(v, k), t[k]);
+  }
+  P4 c2b;
+  p_setup_vjp(e, gm1, eb, c2b);
+  // c^2 = gamma p / rho, H = (E + p) / rho
+  const P4 gc = p_add(c2b, p_mul(gm1, c2b)), Hi = p_mul(eb.H, ir);
+  P4 Ub[NC];
+#pragma unroll
+  for (int k = 0; k < NC; ++k) Ub[k] = p_sub(sm.get(slot_q(0, k)), sm.get(slot_q(1, k)));
+  Ub[3] = p_add(Ub[3], Hi);
+  p_prim_vjp(U1, ir, u, v, gm1, p_add(p_mul(gc, pr), p_mul(eb.H, ep)), eb.u, eb.v, p_add(p_mul(gc, ir), Hi), Ub);
+  if (!p_finite<NC>(Ub)) return false;
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    auto lane = [&](P4 x) { return d_from_scaled(d == 0 ? p_lane0(x) : p_lane1(x), sh, fu); };
+    double o[5][NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      // the linear part of v~: 3/4 (u_{i+1} - u_{i-1})/h - (v_{i-1} + v_{i+1})/4
+      o[0][k] = fma(-g.l34[d], ob[d][k], -lane(sm.get(slot_q(0, k))));
+      o[1][k] = lane(Ub[k]);
+      o[2][k] = fma(g.l34[d], ob[d][k], lane(sm.get(slot_q(1, k))));
+      o[3][k] = fma(-0.25, ob[d][k], lane(sm.get(slot_q(2, k))));
+      o[4][k] = fma(-0.25, ob[d][k], lane(sm.get(slot_q(3, k))));
+    }
+    // mirrored neighbours: back through the sign table
+    mirror_U<NC>(o[0], refl[d][0]);
+    mirror_U<NC>(o[2], refl[d][1]);
+    mirror_D<NC>(o[3], refl[d][0]);
+    mirror_D<NC>(o[4], refl[d][1]);
+    double* out = aw.CM + ((long long)d * plane + p) * 5 * NC;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      if (d == 1) swap_frame<NC>(o[q]);
+#pragma unroll
+      for (int k = 0; k < NC; ++k) out[q * NC + k] = o[q][k];
+    }
+  }
+  return true;
+}
+
+// Bound by its FP32 work (54 % of the FMA pipe, FP64 26 %): three blocks of 128 per SM (168 registers, 74 KB
+// of slots each).  2D Euler 1024^2: 0.51 ms per launch against 2.32 ms for the FP64 kernel.
+__global__ void __launch_bounds__(kThreads, 3) k_adj_cell_pair(Grid g, const double* __restrict__ S,
+                                                               const double* __restrict__ muM, AdjWork aw) {
+  const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
+  extern __shared__ ulonglong2 adj_pair_slots[];
+  const bool left =
+      p < g.plane && !adj_cell_pair(g, S, muM, aw, HW_IDX(p, g.plane), PairSlots{adj_pair_slots + threadIdx.x});
+#pragma unroll
+  for (unsigned int d = 0; d < 2; ++d) list_append(aw.count, aw.cells, (unsigned int)p * 2u + d, left);
+}
+
+// -------------------------------------------------------------------------------------------
+// The contributions of a 2D face with the transpose of the interpolation's nonlinear part in pairs;
+// false where the FP64 kernel is needed.
+__device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __restrict__ S,
+                                              const double* __restrict__ muL, const AdjWork& aw,
+                                              const double* __restrict__ alpha2, int dir, long long f, const PairSlots& sm) {
+  constexpr int NC = 4;
+  const long long plane = g.plane;
+  const int n = dir == 0 ? g.nx : g.ny;
+  int fa, line;
+  if (dir == 0) {
+    line = (int)(f / (n + 1));
+    fa = (int)(f % (n + 1));
+  } else {
+    fa = (int)(f / g.nx);
+    line = (int)(f % g.nx);
+  }
+  const FU fu = fu_of(aw.scal);
+  const int fown = dir == 0 ? 1 : 2;
+  bool refl[4];
+  double Uq[2][NC];                  // the inner cells
+  double Um[NC], Up[NC], Dm[NC], Dp[NC];  // interface states less the corrections
+  const double k21 = g.uvd[dir][0], k3 = g.uvd[dir][1], l3 = g.l3[dir], l9 = g.l9[dir];
+  {
+    double U[4][NC], Z[4][NC];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int a = bc_map(fa - 2 + q, n, g.bc, refl[q]);
+      const long long pc = HW_IDX(dir == 0 ? (long long)line * g.nx + a : (long long)a * g.nx + line, plane);
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        U[q][k] = S[k * plane + pc];
+        Z[q][k] = S[(fown * NC + k) * plane + pc];
+      }
+      if (dir == 1) {
+        swap_frame<NC>(U[q]);
+        swap_frame<NC>(Z[q]);
+      }
+      mirror_U<NC>(U[q], refl[q]);
+      mirror_D<NC>(Z[q], refl[q]);
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const double a = fu.sub(U[1][k], U[0][k]), b = fu.sub(U[2][k], U[1][k]), c = fu.sub(U[3][k], U[2][k]);
+      Um[k] = fma(0.125, a, fma(0.5625, b, fma(-l3, Z[0][k], -l9 * Z[2][k])));
+      Up[k] = fma(-0.125, c, fma(-0.5625, b, fma(l3, Z[3][k], l9 * Z[1][k])));
+      Dm[k] = fma(k21, b, fma(-k3, a, fma(0.0625, Z[0][k], -0.1875 * Z[2][k])));
+      Dp[k] = fma(k21, b, fma(-k3, c, fma(-0.1875, Z[1][k], 0.0625 * Z[3][k])));
+      Uq[0][k] = U[1][k];
+      Uq[1][k] = U[2][k];
+      const P2 pb = p_from(b);
+      // per side (lane): the differences and the end derivatives of its stencil
+      sm.set(slot_q(0, k), p_pack(p_from(a), pb));
+      sm.set(slot_q(1, k), p_pack(pb, p_from(c)));
+      sm.set(slot_q(2, k), p_pack(p_from(Z[0][k]), p_from(Z[1][k])));
+      sm.set(slot_q(3, k), p_pack(p_from(Z[2][k]), p_from(Z[3][k])));
+    }
+  }
+  // primitives of the two inner cells (lanes) and their Roe average
+  const P4 gm1 = p_const<F2>(g.pg.gm1);
+  P4 UI[NC];
+#pragma unroll
+  for (int k = 0; k < NC; ++k) UI[k] = p_pack(p_from(Uq[0][k]), p_from(Uq[1][k]));
+  P4 inv;
+  const P4 ir = p_rcp(UI[0]), u = p_mul(UI[1], ir), v = p_mul(UI[2], ir), sq = p_sqrt(UI[0], inv);
+  const P4 pr = p_mul(gm1, p_sub(UI[3], p_scale(p_add(p_mul(UI[1], u), p_mul(UI[2], v)), 0.5f)));
+  const P4 ep = p_add(UI[3], pr), H = p_mul(ep, ir);
+  const P2 iw_ = p_rcp(p_renorm(p_sum(sq)));
+  const P4 iw = p_pack(iw_, iw_), wt = p_mul(sq, iw);  // the weights of the average
+  const P2 ub = p_sum(p_mul(wt, u)), vb = p_sum(p_mul(wt, v)), Hb = p_sum(p_mul(wt, H));
+  EigP<NC, F2> e;
+  {
+    const P2 q2 = p_add(p_sqr(ub), p_sqr(vb));
+    const P2 c2 = p_renorm(p_mul(p_const<float>(g.pg.gm1), p_sub(Hb, p_scale(q2, 0.5f))));
+    e.setup(p_pack(ub, ub), p_pack(vb, vb), p_pack(Hb, Hb), p_pack(c2, c2), gm1);
+  }
+  const P4 h = p_const<F2>(g.pg.h[dir]), eps = p_const<F2>(g.pg.eps), ig = p_const<F2>(g.pg.ig1);
+#pragma unroll 1
+  for (int v = 0; v < 4; ++v) {
+    P4 q[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) q[k] = sm.get(slot_q(v, k));
+    e.project(q, q);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) sm.set(slot_w(k, v), p_renorm(q[k]));
+  }
+  P4 nb[NC];
+  {
+    P4 c[NC], nn[NC];
+    bool ok = true;
+#pragma unroll 1
+    for (int s = 0; s < NC; ++s) {
+      PStencil<F2> st;
+      const P4 w0 = sm.get(slot_w(s, 0)), w1 = sm.get(slot_w(s, 1));
+      ok = p_stencil(w0, w1, sm.get(slot_w(s, 2)), sm.get(slot_w(s, 3)), p_add(p_sqr(w0), eps), p_add(p_sqr(w1), eps),
+                     h, st) &&
+           ok;
+      sm.set(slot_c(s), p_face_values(st, ig, g.pg.G));
+    }
+#pragma unroll
+    for (int s = 0; s < NC; ++s) c[s] = sm.get(slot_c(s));
+    e.back(c, nn);
+    if (!ok || !p_finite<NC>(nn)) return false;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const P2 a = p_lane0(nn[k]), b = p_lane1(nn[k]);
+      Um[k] = fu.add(Uq[0][k], fu.add(Um[k], fu.add(d_from(a.h), d_from(a.l))));
+      Up[k] = fu.add(Uq[1][k], fu.add(Up[k], fu.add(d_from(b.h), d_from(b.l))));
+    }
+  }
+  // FP64: the fluxes' transposes, as in adj_face
+  double Umb[NC], Upb[NC], Dmb[NC], Dpb[NC];
+  {
+    double Fb[NC], Hb2[NC];
+    const double hih = g.hih[dir], ha = hih * alpha2[dir];
+    const bool hasL = fa - 1 >= 0, hasR = fa <= n - 1;
+    const long long cL = dir == 0 ? (long long)line * g.nx + (fa - 1) : (long long)(fa - 1) * g.nx + line;
+    const long long cR = dir == 0 ? (long long)line * g.nx + fa : (long long)fa * g.nx + line;
+    double nuf[NC], nuh[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const double rf = hasR ? muL[k * plane + HW_IDX(cR, plane)] : 0.0;
+      const double lf = hasL ? muL[k * plane + HW_IDX(cL, plane)] : 0.0;
+      const double rh = hasR ? muL[(fown * NC + k) * plane + HW_IDX(cR, plane)] : 0.0;
+      const double lh = hasL ? muL[(fown * NC + k) * plane + HW_IDX(cL, plane)] : 0.0;
+      nuf[k] = fu.sub(rf, lf);
+      nuh[k] = fu.sub(rh, lh);
+    }
+    if (dir == 1) {
+      swap_frame<NC>(nuf);
+      swap_frame<NC>(nuh);
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      Umb[k] = ha * nuf[k];
+      Upb[k] = -Umb[k];
+      Dmb[k] = ha * nuh[k];
+      Dpb[k] = -Dmb[k];
+      Fb[k] = hih * nuf[k];
+      Hb2[k] = hih * nuh[k];
+    }
+    const Prim<NC> qm = prim_of<NC>(Um, g.gm1, fu), qp = prim_of<NC>(Up, g.gm1, fu);
+    flux_bwd<NC>(Um, qm, g.gm1, Fb, Umb, fu);
+    flux_bwd<NC>(Up, qp, g.gm1, Fb, Upb, fu);
+    jvp_bwd<NC>(Um, qm, Dm, g.gm1, Hb2, Umb, Dmb, fu);
+    jvp_bwd<NC>(Up, qp, Dp, g.gm1, Hb2, Upb, Dpb, fu);
+  }
+  // pairs: the transpose of the corrections
+  unsigned int big = 0u;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) big = max(big, max(seed_bits(Umb[k]), seed_bits(Upb[k])));
+  int sh;
+  if (!seed_scale(big, sh)) return false;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) nb[k] = p_pack(p_from_scaled(Umb[k], sh), p_from_scaled(Upb[k], sh));
+  P4 c[NC];
+  p_back_t(e, nb, c);
+#pragma unroll
+  for (int s = 0; s < NC; ++s) sm.set(slot_c(s), c[s]);
+#pragma unroll 1
+  for (int s = 0; s < NC; ++s) {
+    bool ok = true;
+    P4 w0, w1, w2, w3;
+    sm.set(slot_c(s), p_correction_vjp<CORR_FACE>(sm.get(slot_w(s, 0)), sm.get(slot_w(s, 1)), sm.get(slot_w(s, 2)),
+                                                  sm.get(slot_w(s, 3)), h, eps, ig, g.pg.G, sm.get(slot_c(s)), w0, w1,
+                                                  w2, w3, ok));
+    sm.set(slot_w(s, 0), w0);
+    sm.set(slot_w(s, 1), w1);
+    sm.set(slot_w(s, 2), w2);
+    sm.set(slot_w(s, 3), w3);
+  }
+#pragma unroll
+  for (int s = 0; s < NC; ++s) c[s] = sm.get(slot_c(s));
+  EigPBar<F2> eb;
+  eb.zero();
+  p_back_eig(c, nb, eb);
+#pragma unroll 1
+  for (int v = 0; v < 4; ++v) {
+    P4 q[NC], wb[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      q[k] = sm.get(slot_q(v, k));
+      wb[k] = sm.get(slot_w(k, v));
+    }
+    P4 b[NC];
+    p_project_vjp(e, q, wb, b, eb);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) sm.set(slot_q(v, k), b[k]);
+  }
+  P4 c2b, UIb[NC];
+  p_setup_vjp(e, gm1, eb, c2b);
+  {
+    // both lanes held the same basis: the sums of their adjoints; c^2 = gm1 (H - (u^2 + v^2)/2), then the
+    // Roe average x = (s_l x_l + s_r x_r) iw
+    const P2 gc = p_mul(p_const<float>(g.pg.gm1), p_sum(c2b));
+    const P2 Hs = p_add(p_sum(eb.H), gc);
+    const P2 us = p_sub(p_sum(eb.u), p_mul(gc, ub)), vs = p_sub(p_sum(eb.v), p_mul(gc, vb));
+    const P4 H4 = p_pack(Hs, Hs), u4 = p_pack(us, us), v4 = p_pack(vs, vs);
+    const P4 t = p_add(p_mul(u4, u), p_add(p_mul(v4, v), p_mul(H4, H)));
+    const P2 iwb_ = p_sum(p_mul(sq, t));
+    const P4 iwb = p_mul(p_pack(iwb_, iwb_), p_sqr(iw));
+    const P4 sb = p_sub(p_mul(iw, t), iwb);
+    const P4 Hl = p_mul(H4, wt), Hi = p_mul(Hl, ir);
+    const P2 zero = p_const<float>(0.0);
+    UIb[0] = p_mul(p_mul(sb, p_scale(sq, 0.5f)), ir);
+    UIb[1] = UIb[2] = p_pack(zero, zero);
+    UIb[3] = Hi;
+    p_prim_vjp(UI, ir, u, v, gm1, p_mul(Hl, ep), p_mul(u4, wt), p_mul(v4, wt), Hi, UIb);
+  }
+  if (!p_finite<NC>(UIb)) return false;
+  // FP64: the transposes of the linear parts, and the pairs added
+  const long long fo = HW_IDX(dir == 0 ? (long long)line * (g.nx + 1) + fa : (long long)fa * g.nx + line,
+                              dir == 0 ? (long long)(g.nx + 1) * g.ny : (long long)(g.ny + 1) * g.nx);
+  const long long base = ((dir == 0 ? 0 : (long long)(g.nx + 1) * g.ny) + fo) * 4 * NC;
+  double Ub[4][NC], Zb[4][NC];
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    const P4 b1 = sm.get(slot_q(0, k)), b2 = sm.get(slot_q(1, k)), z1 = sm.get(slot_q(2, k)), z2 = sm.get(slot_q(3, k));
+    const P2 a0 = p_lane0(b1), a1 = p_add(p_lane1(b1), p_lane0(b2)), a2 = p_lane1(b2);
+    const double m0 = d_from_scaled(p_neg(a0), sh, fu);
+    const double m1 = d_from_scaled(p_add(p_sub(a0, a1), p_lane0(UIb[k])), sh, fu);
+    const double m2 = d_from_scaled(p_add(p_sub(a1, a2), p_lane1(UIb[k])), sh, fu);
+    const double m3 = d_from_scaled(a2, sh, fu);
+    const double c1 = fma(0.5625, fu.sub(Umb[k], Upb[k]), k21 * fu.add(Dmb[k], Dpb[k]));
+    Ub[0][k] = fma(-0.125, Umb[k], fma(k3, Dmb[k], m0));
+    Ub[1][k] = fma(1.125, Umb[k], fma(-k3, Dmb[k], fu.sub(m1, c1)));
+    Ub[2][k] = fma(1.125, Upb[k], fma(k3, Dpb[k], fu.add(m2, c1)));
+    Ub[3][k] = fma(-0.125, Upb[k], fma(-k3, Dpb[k], m3));
+    Zb[0][k] = fma(-l3, Umb[k], fma(0.0625, Dmb[k], d_from_scaled(p_lane0(z1), sh, fu)));
+    Zb[1][k] = fma(l9, Upb[k], fma(-0.1875, Dpb[k], d_from_scaled(p_lane1(z1), sh, fu)));
+    Zb[2][k] = fma(-l9, Umb[k], fma(-0.1875, Dmb[k], d_from_scaled(p_lane0(z2), sh, fu)));
+    Zb[3][k] = fma(l3, Upb[k], fma(0.0625, Dpb[k], d_from_scaled(p_lane1(z2), sh, fu)));
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    mirror_U<NC>(Ub[q], refl[q]);
+    mirror_D<NC>(Zb[q], refl[q]);
+    if (dir == 1) {
+      swap_frame<NC>(Ub[q]);
+      swap_frame<NC>(Zb[q]);
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      aw.CU[base + q * NC + k] = Ub[q][k];
+      aw.CD[base + q * NC + k] = Zb[q][k];
+    }
+  }
+  return true;
+}
+
+// Bound by the FP64 pipe (72 % busy; the fluxes' transposes) with the pairs' latency between.  1024^2: 2.1 ms
+// per launch against 5.95 ms for the FP64 kernel; two or four blocks per SM: the adjoint step 11.6 and
+// 11.7 ms against 11.4 ms.
+__global__ void __launch_bounds__(kThreads, 3) k_adj_face_pair(Grid g, const double* __restrict__ S,
+                                                               const double* __restrict__ muL, AdjWork aw,
+                                                               const double* __restrict__ alpha2) {
+  const int dir = blockIdx.y;
+  const long long nfx = (long long)(g.nx + 1) * g.ny, nf = dir == 0 ? nfx : (long long)(g.ny + 1) * g.nx;
+  const long long f = (long long)blockIdx.x * kThreads + threadIdx.x;
+  extern __shared__ ulonglong2 adj_pair_slots[];
+  const bool left = f < nf && !adj_face_pair(g, S, muL, aw, alpha2, dir, f, PairSlots{adj_pair_slots + threadIdx.x});
+  list_append(aw.count + 1, aw.faces, (unsigned int)(f + (dir == 0 ? 0 : nfx)), left);
 }
 
 // -------------------------------------------------------------------------------------------
@@ -606,7 +1094,7 @@ unsigned int bounds_take_adjoint(int* line) {
 namespace {
 
 struct AdjLayout {
-  size_t S1, S2, lam2, lam1, lamB, muM, muL, CU, CD, CM, total;
+  size_t S1, S2, lam2, lam1, lamB, muM, muL, CU, CD, CM, lists, total;
 };
 
 AdjLayout adj_layout(const hweno_ctx* h) {
@@ -617,7 +1105,9 @@ AdjLayout adj_layout(const hweno_ctx* h) {
   l.S1 = l.S2 = l.lam2 = l.lam1 = l.lamB = l.muM = l.muL = align_up(nst);
   l.CU = l.CD = align_up((nfx + nfy) * 4 * nc * 8);
   l.CM = align_up((size_t)h->dim * h->nx * h->ny * 5 * nc * 8);
-  l.total = 7 * l.S1 + l.CU + l.CD + l.CM;
+  // the counts, then the lists of cells (two directions each) and faces
+  l.lists = h->dim == 2 ? align_up((64 + 2 * (size_t)h->nx * h->ny + nfx + nfy) * sizeof(unsigned int)) : 0;
+  l.total = 7 * l.S1 + l.CU + l.CD + l.CM + l.lists;
   return l;
 }
 
@@ -640,6 +1130,10 @@ AdjPtrs adj_ptrs(const hweno_ctx* h, void* ws) {
   a.aw.CD = reinterpret_cast<double*>(p);
   p += l.CD;
   a.aw.CM = reinterpret_cast<double*>(p);
+  p += l.CM;
+  a.aw.count = reinterpret_cast<unsigned int*>(p);
+  a.aw.cells = a.aw.count + 64;
+  a.aw.faces = a.aw.cells + 2 * h->nx * h->ny;
   a.aw.scal = h->w.scal;
   return a;
 }
@@ -649,7 +1143,7 @@ int stage_vjp(const hweno_ctx* h, const Grid& g, const double* S, const double* 
               const double* muL, const hw::AdjWork& aw, double* lam) {
   const cudaStream_t st = h->stream;
   const unsigned bc = blocks_for(g.plane);
-  // shared memory for the saved forward intermediates: one slot per thread and value
+  // the FP64 kernels' shared memory for the saved forward intermediates: one slot per thread and value
   constexpr int NC = DIM == 1 ? 3 : 4;
   constexpr size_t cell_sm = (size_t)hw::kCellSaved * NC * hw::kThreads * sizeof(double);
   constexpr size_t face_sm = (size_t)hw::kFaceSaved * NC * hw::kThreads * sizeof(double);
@@ -658,11 +1152,27 @@ int stage_vjp(const hweno_ctx* h, const Grid& g, const double* S, const double* 
       cudaFuncSetAttribute(hw::k_adj_cell<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cell_sm) !=
           cudaSuccess)
     return HWENO_ECUDA;
-  hw::k_adj_cell<DIM><<<dim3(bc, DIM), hw::kThreads, cell_sm, st>>>(g, S, muM, aw);
   const long long nfx = (long long)(g.nx + 1) * g.ny;
   const long long nfy = DIM == 2 ? (long long)(g.ny + 1) * g.nx : 0;
-  hw::k_adj_face<DIM><<<dim3(blocks_for(nfx > nfy ? nfx : nfy), DIM), hw::kThreads, face_sm, st>>>(g, S, muL, aw,
-                                                                                                  alpha2);
+  const unsigned bf = blocks_for(nfx > nfy ? nfx : nfy);
+  if (DIM == 1) {
+    hw::k_adj_cell<1><<<bc, hw::kThreads, cell_sm, st>>>(g, S, muM, aw);
+    hw::k_adj_face<1><<<bf, hw::kThreads, face_sm, st>>>(g, S, muL, aw, alpha2);
+  } else {
+    // most of the work in pairs, the rest (listed on the way) in FP64: two blocks per SM take it in turn
+    const unsigned bl = 2u * hw::kSMs;
+    constexpr size_t pair_sm = (size_t)hw::kPairSlots * hw::kThreads * sizeof(ulonglong2);
+    if (cudaFuncSetAttribute(hw::k_adj_face_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_sm) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(hw::k_adj_cell_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_sm) !=
+            cudaSuccess)
+      return HWENO_ECUDA;
+    if (cudaMemsetAsync(aw.count, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) return HWENO_ECUDA;
+    hw::k_adj_cell_pair<<<bc, hw::kThreads, pair_sm, st>>>(g, S, muM, aw);
+    hw::k_adj_face_pair<<<dim3(bf, 2), hw::kThreads, pair_sm, st>>>(g, S, muL, aw, alpha2);
+    hw::k_adj_cell<DIM><<<bl < 2 * bc ? bl : 2 * bc, hw::kThreads, cell_sm, st>>>(g, S, muM, aw);
+    hw::k_adj_face<DIM><<<bl < 2 * bf ? bl : 2 * bf, hw::kThreads, face_sm, st>>>(g, S, muL, aw, alpha2);
+  }
   hw::k_adj_gather<DIM><<<bc, hw::kThreads, 0, st>>>(g, S, muM, muL, aw, lam);
   return cudaGetLastError() == cudaSuccess ? HWENO_OK : HWENO_ECUDA;
 }
@@ -699,7 +1209,7 @@ int adjoint_from_stages(hweno_t* h, const AdjPtrs& a, const double* Sn, const do
   hw::k_rk_first<<<rk_blocks(h), 256, 0, h->stream>>>(rk_n(h), a.muM, a.muL, dt, a.lam1, a.lamB);
   if ((rc = launch_status())) return rc;
   if ((rc = vjp(Sn, 0, a.muM, a.muL, lam_out))) return rc;
-  h->launches += 9 + 3;
+  h->launches += (h->dim == 1 ? 9 : 15) + 3;
   return HWENO_OK;
 }
 
@@ -789,7 +1299,7 @@ int hweno_stage_vjp(hweno_t* h, const double* S, const double* alpha2, const dou
   if ((uintptr_t)adj_ws & 255) return HWENO_EINVAL;
   const AdjPtrs a = adj_ptrs(h, adj_ws);
   const Grid g = grid_of(h);
-  h->launches += 3;
+  h->launches += h->dim == 1 ? 3 : 5;
   return h->dim == 1 ? stage_vjp<1>(h, g, S, alpha2, muM, muL, a.aw, lam)
                      : stage_vjp<2>(h, g, S, alpha2, muM, muL, a.aw, lam);
 }
