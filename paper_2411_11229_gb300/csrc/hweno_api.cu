@@ -224,24 +224,18 @@ int hweno_rhs(hweno_t* h, const double* S, double* Lo, double* Mo) {
   return stage(h, S, const_cast<double*>(S), 1, 0, 0.0, 3, Lo, Mo);
 }
 
-int hweno_step(hweno_t* h, double dt) {
-  if (!h) return HWENO_EINVAL;
-  if (!h->ws || !h->state) return HWENO_ESTATE;
-  if (!std::isfinite(dt)) return HWENO_EINVAL;
-  for (int st = 0; st < 3; ++st) {
-    int rc = stage(h, h->state, h->state, 0, st, dt, st, nullptr, nullptr);
-    if (rc) return rc;
-  }
-  return HWENO_OK;
-}
+int hweno_step(hweno_t* h, double dt) { return h ? hweno_steps(h, dt, 1) : HWENO_EINVAL; }
 
 int hweno_steps(hweno_t* h, double dt, int nsteps) {
   if (!h || nsteps < 0) return HWENO_EINVAL;
-  for (int s = 0; s < nsteps; ++s) {
-    int rc = hweno_step(h, dt);
-    if (rc) return rc;
-  }
-  return HWENO_OK;
+  if (nsteps == 0) return HWENO_OK;
+  if (!h->ws || !h->state) return HWENO_ESTATE;
+  if (!std::isfinite(dt)) return HWENO_EINVAL;
+  bool done = false;
+  int rc = line_steps(h, dt, nsteps, &done);
+  for (int s = 0; s < nsteps && !rc && !done; ++s)
+    for (int st = 0; st < 3 && !rc; ++st) rc = stage(h, h->state, h->state, 0, st, dt, st, nullptr, nullptr);
+  return rc;
 }
 
 int hweno_set_time(hweno_t* h, double t, double t_end) {
@@ -269,7 +263,8 @@ int hweno_run(hweno_t* h, double t_end, int64_t max_steps, int64_t* steps_done) 
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
   long long chunk_launches = 0;
-  if (!h->profiling && max_steps >= kChunk &&
+  const bool line = h->dim == 1 && h->var == 0 && h->nx <= kLineMaxCells;  // one launch a chunk as it is
+  if (!h->profiling && !line && max_steps >= kChunk &&
       cudaStreamCreateWithFlags(&priv, cudaStreamNonBlocking) == cudaSuccess &&
       cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess &&
       cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess) {
@@ -316,7 +311,7 @@ int hweno_run(hweno_t* h, double t_end, int64_t max_steps, int64_t* steps_done) 
       }
       h->launches += chunk_launches;
     } else {
-      for (int64_t k = 0; k < (left < kChunk ? left : kChunk) && !rc; ++k) rc = hweno_step(h, 0.0);
+      rc = hweno_steps(h, 0.0, (int)(left < kChunk ? left : kChunk));
       if (rc) break;
     }
   }
@@ -673,10 +668,11 @@ extern "C" int hweno_rhs_static(int dim, int system, int64_t nx, int64_t ny, dou
 extern "C" long long hweno_bounds_status(int* where) {
 #ifdef HWENO_BOUNDS_CHECK
   if (cudaDeviceSynchronize() != cudaSuccess) return HWENO_ECUDA;
-  int l0 = 0, l1 = 0, l2 = 0;
+  int l0 = 0, l1 = 0, l2 = 0, l3 = 0;
   const unsigned int c0 = hw::bounds_take(&l0), c1 = hwh::bounds_take_batch(&l1), c2 = hwh::bounds_take_adjoint(&l2);
-  if (where) *where = c0 ? l0 : (c1 ? 100000 + l1 : (c2 ? 200000 + l2 : 0));
-  return (long long)c0 + c1 + c2;
+  const unsigned int c3 = hwh::bounds_take_line(&l3);
+  if (where) *where = c0 ? l0 : (c1 ? 100000 + l1 : (c2 ? 200000 + l2 : (c3 ? 300000 + l3 : 0)));
+  return (long long)c0 + c1 + c2 + c3;
 #else
   if (where) *where = 0;
   return -1;

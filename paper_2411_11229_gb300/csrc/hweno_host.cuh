@@ -134,13 +134,15 @@ inline void to_pair(double x, float* p) {
   p[1] = (float)(x - (double)p[0]);
 }
 
+// Cells of a 1D grid that one block of each SM can hold (hweno_line.cu)
+constexpr long long kLineMaxCells = hw::kSMs * (hw::kThreads - 4LL);
+
 // The nonlinear part in pairs (hweno_pair.cuh) trades FP64 instructions for several times as many FP32
-// ones, which pays where the FP64 pipe is kept busy.  A 1D grid of at most one warp per scheduler (19456
-// cells) leaves it idle and waits for each thread's chain of instructions instead, which is the
-// longer one in pairs: one stage of 2048 cells 43 us in FP64, 53 us in pairs.  A 2D grid of 64^2
+// ones, which pays where the FP64 pipe is kept busy.  A 1D grid of at most one warp per scheduler
+// leaves it idle and waits for each thread's chain of instructions instead, which is the longer one in
+// pairs: one stage of 2048 cells in the stage kernels 43 us in FP64, 53 us in pairs.  A 2D grid of 64^2
 // cells (128 warps of cells, 260 of faces) already gains: 64 us in FP64, 48 us in pairs.
-constexpr long long kPairMinCells1D = hw::kSMs * 4LL * 32;
-inline int pairs_of(const hweno_ctx* h) { return h->dim == 2 || h->nx > kPairMinCells1D; }
+inline int pairs_of(const hweno_ctx* h) { return h->dim == 2 || h->nx > kLineMaxCells; }
 
 inline Grid grid_of(const hweno_ctx* h) {
   Grid g;
@@ -340,7 +342,13 @@ inline int stage(hweno_ctx* h, const double* S_in, double* S_out, int mode, int 
 // bounds-checked build: the out-of-range index records of the batched and adjoint translation
 // units (count since the last call, first source line; 0 in a normal build)
 unsigned int bounds_take_batch(int* line);
+unsigned int bounds_take_line(int* line);
 unsigned int bounds_take_adjoint(int* line);
+
+// nsteps steps (CFL for dt <= 0) of a small 1D grid of the plain scheme in one cooperative launch
+// (hweno_line.cu), for any 1D grid that one block per SM holds: the stage kernels take 41 us an Euler
+// stage whatever its size, the one launch 28 us.  *done: whether the grid was one of these.
+int line_steps(hweno_ctx* h, double dt, int nsteps, bool* done);
 
 inline int stage_replay(hweno_ctx* h, double* S, int st, double dt, const double* alpha2_dev) {
   return stage(h, S, S, 0, st, dt, st, nullptr, nullptr, alpha2_dev);

@@ -379,6 +379,35 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
   return true;
 }
 
+// Velocities, pressure, 1/rho of a cell, and its wavespeeds per direction
+template <int DIM, int SYS>
+struct CellState {
+  double u = 0.0, v = 0.0, pr = 0.0, ir = 0.0;
+  // returns whether the state is physical
+  __device__ __forceinline__ bool set(const double* U, const Grid& g, const FU& f, double& wsx, double& wsy) {
+    constexpr int NC = Traits<DIM, SYS>::NC;
+    if (SYS == SYS_EULER) {
+      ir = rcp(U[0], f);
+      u = f.mul(U[1], ir);
+      if (DIM == 2) v = f.mul(U[2], ir);
+      const double ke = DIM == 2 ? fma(U[1], u, f.mul(U[2], v)) : f.mul(U[1], u);
+      pr = g.gm1 * fma(-0.5, ke, U[NC - 1]);
+      const double c = sqrt_fast(f.mul(g.gamma * pr, ir), f);
+      wsx = f.add(fabs(u), c);
+      wsy = DIM == 2 ? f.add(fabs(v), c) : 0.0;
+      return positive_bits(U[0]) && positive_bits(pr) && finite_bits(wsx) && finite_bits(wsy);
+    }
+    if (SYS == SYS_BURGERS) {
+      wsx = fabs(U[0]);
+      wsy = DIM == 2 ? wsx : 0.0;
+      return finite_bits(wsx);
+    }
+    wsx = fabs(g.ax);
+    wsy = DIM == 2 ? fabs(g.ay) : 0.0;
+    return true;
+  }
+};
+
 // Cell work of one stage at cell p: wavespeeds (returned in wsx, wsy), primitives, nodal values per
 // direction, modified derivatives (and, for R2, the face states of the cell).  Returns
 // false where the modified derivatives are left to cell_limiter.
@@ -399,25 +428,9 @@ __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restric
       if (DIM == 2) Wd[k] = S[(2 * NC + k) * plane + p];
     }
     // primitives and wavespeeds
-    double u = 0, v = 0, pr = 0, ir = 0;
-    if (SYS == SYS_EULER) {
-      ir = rcp(U[0], f);
-      u = f.mul(U[1], ir);
-      if (DIM == 2) v = f.mul(U[2], ir);
-      const double ke = DIM == 2 ? fma(U[1], u, f.mul(U[2], v)) : f.mul(U[1], u);
-      pr = g.gm1 * fma(-0.5, ke, U[NC - 1]);
-      const double c = sqrt_fast(f.mul(g.gamma * pr, ir), f);
-      wsx = f.add(fabs(u), c);
-      wsy = DIM == 2 ? f.add(fabs(v), c) : 0.0;
-      if (!positive_bits(U[0]) || !positive_bits(pr) || !finite_bits(wsx) || !finite_bits(wsy)) atomicOr(w.status, 1u);
-    } else if (SYS == SYS_BURGERS) {
-      wsx = fabs(U[0]);
-      wsy = DIM == 2 ? wsx : 0.0;
-      if (!finite_bits(wsx)) atomicOr(w.status, 1u);
-    } else {
-      wsx = fabs(g.ax);
-      wsy = DIM == 2 ? fabs(g.ay) : 0.0;
-    }
+    CellState<DIM, SYS> c;
+    if (!c.set(U, g, f, wsx, wsy)) atomicOr(w.status, 1u);
+    const double u = c.u, v = c.v, pr = c.pr, ir = c.ir;
     if (VAR && (g.flags & FLAG_ALPHA_LOCAL)) {
       w.WS[p] = wsx;
       if (DIM == 2) w.WS[plane + p] = wsy;
@@ -1011,18 +1024,22 @@ __device__ __forceinline__ void update_body(const Grid& g, double* __restrict__ 
   }
 }
 
+// The CFL step for the wavespeeds axs, ays at time t, clamped to the end time te (if positive)
+template <int DIM>
+__device__ __forceinline__ double cfl_dt(const Grid& g, double axs, double ays, double t, double te) {
+  double dt = DIM == 2 ? g.cfl / fma(axs, g.inv_dx, ays * g.inv_dy) : g.cfl * g.dx / axs;
+  if (te > 0.0 && t + dt > te) dt = fmax(te - t, 0.0);
+  return dt;
+}
+
 // The step size of a stage: dt_fixed > 0, or (dt_fixed <= 0) at stage 0 the CFL step from the
 // wavespeed slot (clamped to t_end); stages 1 and 2 reuse the value stored in scal[0].
 template <int DIM>
 __device__ __forceinline__ double stage_dt(const Grid& g, const Work& w, int stage, double dt_fixed, int slot) {
   if (stage != 0) return w.scal[0];
   if (dt_fixed > 0.0) return dt_fixed;
-  const double axs = __longlong_as_double((long long)w.alpha[slot * w.astride]);
-  const double ays = __longlong_as_double((long long)w.alpha[slot * w.astride + 1]);
-  double dt = DIM == 2 ? g.cfl / fma(axs, g.inv_dx, ays * g.inv_dy) : g.cfl * g.dx / axs;
-  const double t = w.scal[1], te = w.scal[2];
-  if (te > 0.0 && t + dt > te) dt = fmax(te - t, 0.0);
-  return dt;
+  return cfl_dt<DIM>(g, __longlong_as_double((long long)w.alpha[slot * w.astride]),
+                     __longlong_as_double((long long)w.alpha[slot * w.astride + 1]), w.scal[1], w.scal[2]);
 }
 
 // dt of stage 0 is stored in scal[0] by block 0 and reused by stages 1 and 2; the time advances
