@@ -305,9 +305,12 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
                                                   P2 pc2, const PairSlots& sm, const FU& f) {
   constexpr int NC = Traits<DIM, SYS>::NC;
   const long long plane = g.plane;
-  // FP64: p_0'(x_i) = 3/4 (u_{i+1} - u_{i-1})/h - (v_{i-1} + v_{i+1})/4 and (R2) the linear parts of the
-  // values and the derivatives at the two faces
-  double md[DIM][NC], um[DIM][NC], up[DIM][NC], dm[DIM][NC], dp[DIM][NC];
+  // FP64: p_0'(x_i) = 3/4 (u_{i+1} - u_{i-1})/h - (v_{i-1} + v_{i+1})/4 and (R2) the derivatives at the two
+  // faces; the linear parts of R2's values less the centre value in pairs, which hold them to the last
+  // bit of the states where the stencil's differences are small beside these
+  double md[DIM][NC], dm[DIM][NC], dp[DIM][NC];
+  P4 um[NC], up[NC];
+  bool small = true;
   {
     P2 uc[NC], du[2][DIM][NC], z[2][DIM][NC];
 #pragma unroll
@@ -322,14 +325,16 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
         md[d][k] = fma(g.l34[d], f.sub(U3[2][k], U3[0][k]), -0.25 * f.add(D3[0][k], D3[2][k]));
         // the differences are taken between pairs: U to 48 bits is enough for the correction
         const P2 u1 = uc[SYS == SYS_EULER && NC == 4 && d == 1 && (k == 1 || k == 2) ? 3 - k : k];
-        du[0][d][k] = p_renorm(p_sub(u1, p_from(U3[0][k])));
-        du[1][d][k] = p_renorm(p_sub(p_from(U3[2][k]), u1));
+        if (VAR != 2) {
+          du[0][d][k] = p_renorm(p_sub(u1, p_from(U3[0][k])));
+          du[1][d][k] = p_renorm(p_sub(p_from(U3[2][k]), u1));
+        }
         z[0][d][k] = p_from(D3[0][k]);
         z[1][d][k] = p_from(D3[2][k]);
         if (VAR == 2) {
           const double d0 = f.sub(U3[1][k], U3[0][k]), d1 = f.sub(U3[2][k], U3[1][k]);
-          um[d][k] = fma(0.125, d0, fma(0.5625, d1, fma(-g.l3[d], D3[0][k], -g.l9[d] * D3[2][k])));
-          up[d][k] = fma(-0.125, d1, fma(-0.5625, d0, fma(g.l3[d], D3[2][k], g.l9[d] * D3[0][k])));
+          du[0][d][k] = p_from(d0);  // its face values want the differences themselves
+          du[1][d][k] = p_from(d1);
           dm[d][k] = fma(k21, d1, fma(-k3, d0, fma(0.0625, D3[0][k], -0.1875 * D3[2][k])));
           dp[d][k] = fma(k21, d0, fma(-k3, d1, fma(-0.1875, D3[0][k], 0.0625 * D3[2][k])));
         }
@@ -342,7 +347,28 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
         sm.set(q * NC + k, p_pack(du[q][0][k], du[q][DIM - 1][k]));
         sm.set((2 + q) * NC + k, p_pack(z[q][0][k], z[q][DIM - 1][k]));
       }
+    if (VAR == 2) {
+      const P4 hq = p_pack(p_const<float>(g.pg.h[0]), p_const<float>(g.pg.h[DIM - 1]));
+      float size[DIM][NC], u_[NC];
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        const P4 d0 = sm.get(k), d1 = sm.get(NC + k);
+        const P4 z0 = p_mul(hq, sm.get(2 * NC + k)), z1 = p_mul(hq, sm.get(3 * NC + k));
+        // d0/8 + 9 d1/16 - 3 z0/64 - 9 z1/64 and, mirrored, -d1/8 - 9 d0/16 + 3 z1/64 + 9 z0/64
+        um[k] = p_add(p_add(p_scale(d0, 0.125f), p_mulf(d1, 0.5625f)), p_neg(p_mulf(p_add(z0, p_mulf(z1, 3.0f)), 0.046875f)));
+        up[k] = p_sub(p_mulf(p_add(z1, p_mulf(z0, 3.0f)), 0.046875f), p_add(p_scale(d1, 0.125f), p_mulf(d0, 0.5625f)));
+        u_[k] = uc[k].h;
+        size[0][k] = fmaxf(fmaxf(fabsf(f_lane0(d0.h)), fabsf(f_lane0(d1.h))), fmaxf(fabsf(f_lane0(z0.h)), fabsf(f_lane0(z1.h))));
+        size[DIM - 1][k] =
+            fmaxf(fmaxf(fabsf(f_lane1(d0.h)), fabsf(f_lane1(d1.h))), fmaxf(fabsf(f_lane1(z0.h)), fabsf(f_lane1(z1.h))));
+      }
+      const float ir = f_rcp(u_[0]), ie = f_rcp(u_[NC - 1]);
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) small = small && p_rel2<NC>(size[d], ir, ie) <= 0x1p-12f;
+      small = small && u_[0] > 0.0f && u_[NC - 1] > 0.0f;
+    }
   }
+  if (!small) return false;
   EigP<NC, F2> e;
   if (SYS == SYS_EULER) {
     const P2 un = DIM == 2 ? pv : pu, ut = DIM == 2 ? pu : pv;
@@ -364,11 +390,12 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
       double* FSd = w.FS + (long long)d * 4 * NC * plane;
 #pragma unroll
       for (int k = 0; k < NC; ++k) {
-        const P2 a = d == 0 ? p_lane0(nm[k]) : p_lane1(nm[k]), b = d == 0 ? p_lane0(np[k]) : p_lane1(np[k]);
+        const P4 a4 = p_add(um[k], nm[k]), b4 = p_add(up[k], np[k]);
+        const P2 a = d == 0 ? p_lane0(a4) : p_lane1(a4), b = d == 0 ? p_lane0(b4) : p_lane1(b4);
         const double u1 = U[SYS == SYS_EULER && NC == 4 && d == 1 && (k == 1 || k == 2) ? 3 - k : k];
-        FSd[k * plane + p] = f.add(u1, f.add(um[d][k], f.add(d_from(a.h), d_from(a.l))));
+        FSd[k * plane + p] = f.add(u1, f.add(d_from(a.h), d_from(a.l)));
         FSd[(NC + k) * plane + p] = dm[d][k];
-        FSd[(2 * NC + k) * plane + p] = f.add(u1, f.add(up[d][k], f.add(d_from(b.h), d_from(b.l))));
+        FSd[(2 * NC + k) * plane + p] = f.add(u1, f.add(d_from(b.h), d_from(b.l)));
         FSd[(3 * NC + k) * plane + p] = dp[d][k];
       }
     }
@@ -968,7 +995,8 @@ __device__ __forceinline__ void update_body(const Grid& g, double* __restrict__ 
                                             double* __restrict__ Lout, double* __restrict__ Mout) {
   using T = Traits<DIM, SYS>;
   constexpr int NC = T::NC, NF = T::NF;
-  constexpr bool SRC = VAR != 0 && DIM == 2 && SYS == SYS_EULER;  // gravity source possible
+  // the gravity source, where it is possible (tested in the integer pipe)
+  const bool src = VAR != 0 && DIM == 2 && SYS == SYS_EULER && (dbl_bits(g.grav) << 1) != 0;
   const long long plane = g.plane;
   const long long p = HW_IDX(p_in, plane);
   const int i = (int)(p % g.nx), j = (int)(p / g.nx);
@@ -988,7 +1016,7 @@ __device__ __forceinline__ void update_body(const Grid& g, double* __restrict__ 
   for (int f = 0; f < NF; ++f) {
     // Eq. (euler2d-s): field f gains g (0, 0, S_f[rho], S_f[rho nu]) (read before S is overwritten)
     double src2 = 0.0, src3 = 0.0;
-    if (SRC && g.grav != 0.0) {
+    if (src) {
       src2 = g.grav * S[(f * NC + 0) * plane + p];
       src3 = g.grav * S[(f * NC + 2) * plane + p];
     }
@@ -1002,16 +1030,16 @@ __device__ __forceinline__ void update_body(const Grid& g, double* __restrict__ 
         // L = -(F_{i+1/2} - F_{i-1/2}) / dx [- (G_{j+1/2} - G_{j-1/2}) / dy] [+ source]
         double L = fu.mul(dF, mix);
         if (DIM == 2) L = fma(dG, miy, L);
-        if (SRC && k == 2) L = fu.add(L, src2);
-        if (SRC && k == 3) L = fu.add(L, src3);
+        if (src && k == 2) L = fu.add(L, src2);
+        if (src && k == 3) L = fu.add(L, src3);
         Lout[fk * plane + p] = L;
         Mout[fk * plane + p] = M;
         continue;
       }
       // b M + b dt L
       double v = stage == 0 ? M : fu.mul(bkr, M);
-      if (SRC && k == 2) v = fma(bdt, src2, v);
-      if (SRC && k == 3) v = fma(bdt, src3, v);
+      if (src && k == 2) v = fma(bdt, src2, v);
+      if (src && k == 3) v = fma(bdt, src3, v);
       if (DIM == 2) v = fma(cy, dG, v);
       v = fma(cx, dF, v);
       if (stage == 0) {

@@ -551,6 +551,16 @@ __device__ __forceinline__ bool p_cell(const PairSlots& sm, const EigP<NC, F2>& 
   return ok && p_finite<NC>(nt) && (!FACES || (p_finite<NC>(nm) && p_finite<NC>(np)));
 }
 
+// The square of a change's size beside a state with 1/rho = ir and 1/E = ie (the momentum's beside
+// sqrt(rho E))
+template <int NC>
+__device__ __forceinline__ float p_rel2(const float* x, float ir, float ie) {
+  const float a = x[0] * ir, b = x[NC - 1] * ie;
+  float m2 = x[1] * x[1];
+  if (NC == 4) m2 += x[2] * x[2];
+  return fmaxf(fmaxf(a * a, b * b), m2 * ir * ie);
+}
+
 // The Lax-Friedrichs flux of an Euler face whose two states are close, from the sums U = U^- + U^+,
 // D = D^- + D^+ and the differences dif = U^+ - U^-, hdif = h (D^+ - D^-).  With f homogeneous of
 // degree one,
@@ -573,13 +583,6 @@ __device__ __forceinline__ bool p_flux_pair(const double* U, const double* D, co
     d_[k] = p_from(D[k]).h;
   }
   const float rho = u_[0], gm1 = pg.gm1[0], ir = f_rcp(rho), ie = f_rcp(u_[E]);
-  // the square of a change's size beside the state (the momentum's beside sqrt(rho E))
-  auto rel2 = [&](const float* x) {
-    const float a = x[0] * ir, b = x[E] * ie;
-    float m2 = x[1] * x[1];
-    if (NC == 4) m2 += x[2] * x[2];
-    return fmaxf(fmaxf(a * a, b * b), m2 * ir * ie);
-  };
   float r[NC], s[NC];  // the differences and the differences of the derivatives (h and l overlap)
 #pragma unroll
   for (int k = 0; k < NC; ++k) {
@@ -587,8 +590,8 @@ __device__ __forceinline__ bool p_flux_pair(const double* U, const double* D, co
     s[k] = f_add(hdif[k].h, hdif[k].l);
   }
   // q is below 2^-32 of the fluxes, q' of the derivatives' fluxes
-  const float r2 = rel2(r), d2 = rel2(size);
-  if (!(r2 <= 0x1p-34f && d2 <= 0x1p-12f && r2 * rel2(s) <= 0x1p-64f * d2 && rho > 0.0f && u_[E] > 0.0f)) return false;
+  const float r2 = p_rel2<NC>(r, ir, ie), d2 = p_rel2<NC>(size, ir, ie);
+  if (!(r2 <= 0x1p-34f && d2 <= 0x1p-12f && r2 * p_rel2<NC>(s, ir, ie) <= 0x1p-64f * d2 && rho > 0.0f && u_[E] > 0.0f)) return false;
 #pragma unroll
   for (int k = 0; k < NC; ++k) s[k] *= ih.h;
   // first-order changes of the velocities and of the pressure, second-order ones, and their
