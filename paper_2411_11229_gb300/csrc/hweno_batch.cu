@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_stage(BatchArgs a) {
 // the 2D items, then of the 1D items), each kernel at the register budget of its own code path;
 // stream order replaces the grid barriers.
 template <int DIM>
-__global__ void __launch_bounds__(kThreads) k_batch_cells(BatchArgs a) {
+__global__ void __launch_bounds__(kThreads, 4) k_batch_cells(BatchArgs a) {
   __shared__ Leftover lo;
   __shared__ ulonglong2 slots[4 * Traits<DIM, SYS_EULER>::NC * kThreads];
   const PairSlots sm{slots + threadIdx.x};
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_cells(BatchArgs a) {
 }
 
 template <int DIM>
-__global__ void __launch_bounds__(kThreads, 3) k_batch_faces(BatchArgs a) {
+__global__ void __launch_bounds__(kThreads, 4) k_batch_faces(BatchArgs a) {
   __shared__ Leftover lo;
   __shared__ ulonglong2 slots[4 * Traits<DIM, SYS_EULER>::NC * kThreads];
   const PairSlots sm{slots + threadIdx.x};
