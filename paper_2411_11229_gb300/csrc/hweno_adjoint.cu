@@ -189,10 +189,10 @@ __global__ void __launch_bounds__(kThreads) k_adj_cell(Grid g, const double* __r
     if (k < g.plane) adj_cell<1>(g, S, muM, aw, 0, k);
     return;
   }
-  const unsigned int n = aw.count[0];
+  const long long n = min((long long)aw.count[0], 2 * g.plane);
   for (; k < n; k += (long long)gridDim.x * kThreads) {
     const unsigned int c = aw.cells[k];
-    adj_cell<DIM>(g, S, muM, aw, (int)(c & 1u), HW_IDX(c >> 1, g.plane));
+    if ((long long)(c >> 1) < g.plane) adj_cell<DIM>(g, S, muM, aw, (int)(c & 1u), HW_IDX(c >> 1, g.plane));
   }
 }
 
@@ -244,16 +244,16 @@ __device__ __forceinline__ void adj_face(const Grid& g, const double* __restrict
   double nuf[NC], nuh[NC];
   {
     const bool hasL = fa - 1 >= 0, hasR = fa <= n - 1;
-    const long long cL = dir == 0 ? (long long)line * g.nx + (fa - 1) : (long long)(fa - 1) * g.nx + line;
-    const long long cR = dir == 0 ? (long long)line * g.nx + fa : (long long)fa * g.nx + line;
+    // (an outer face has one cell inside: its address serves both loads)
+    const int aL = hasL ? fa - 1 : fa, aR = hasR ? fa : fa - 1;
+    const long long cL = HW_IDX(dir == 0 ? (long long)line * g.nx + aL : (long long)aL * g.nx + line, plane);
+    const long long cR = HW_IDX(dir == 0 ? (long long)line * g.nx + aR : (long long)aR * g.nx + line, plane);
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
-      const double rf = hasR ? muL[k * plane + HW_IDX(cR, plane)] : 0.0;
-      const double lf = hasL ? muL[k * plane + HW_IDX(cL, plane)] : 0.0;
-      const double rh = hasR ? muL[(fown * NC + k) * plane + HW_IDX(cR, plane)] : 0.0;
-      const double lh = hasL ? muL[(fown * NC + k) * plane + HW_IDX(cL, plane)] : 0.0;
-      nuf[k] = fu.sub(rf, lf);
-      nuh[k] = fu.sub(rh, lh);
+      const double rf = muL[k * plane + cR], lf = muL[k * plane + cL];
+      const double rh = muL[(fown * NC + k) * plane + cR], lh = muL[(fown * NC + k) * plane + cL];
+      nuf[k] = fu.sub(hasR ? rf : 0.0, hasL ? lf : 0.0);
+      nuh[k] = fu.sub(hasR ? rh : 0.0, hasL ? lh : 0.0);
     }
     if (dir == 1) {
       swap_frame<NC>(nuf);
@@ -421,10 +421,10 @@ __global__ void __launch_bounds__(kThreads) k_adj_face(Grid g, const double* __r
     if (k < nfx) adj_face<1>(g, S, muL, aw, alpha2, 0, k);
     return;
   }
-  const unsigned int n = aw.count[1];
+  const long long all = nfx + (long long)(g.ny + 1) * g.nx, n = min((long long)aw.count[1], all);
   for (; k < n; k += (long long)gridDim.x * kThreads) {
-    const long long f = HW_IDX(aw.faces[k], nfx + (long long)(g.ny + 1) * g.nx);
-    adj_face<DIM>(g, S, muL, aw, alpha2, f < nfx ? 0 : 1, f < nfx ? f : f - nfx);
+    const long long f = HW_IDX(aw.faces[k], all);
+    if (f < all) adj_face<DIM>(g, S, muL, aw, alpha2, f < nfx ? 0 : 1, f < nfx ? f : f - nfx);
   }
 }
 
@@ -723,17 +723,17 @@ __device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __res
     double Fb[NC], Hb2[NC];
     const double hih = g.hih[dir], ha = hih * alpha2[dir];
     const bool hasL = fa - 1 >= 0, hasR = fa <= n - 1;
-    const long long cL = dir == 0 ? (long long)line * g.nx + (fa - 1) : (long long)(fa - 1) * g.nx + line;
-    const long long cR = dir == 0 ? (long long)line * g.nx + fa : (long long)fa * g.nx + line;
+    // (an outer face has one cell inside: its address serves both loads)
+    const int aL = hasL ? fa - 1 : fa, aR = hasR ? fa : fa - 1;
+    const long long cL = HW_IDX(dir == 0 ? (long long)line * g.nx + aL : (long long)aL * g.nx + line, plane);
+    const long long cR = HW_IDX(dir == 0 ? (long long)line * g.nx + aR : (long long)aR * g.nx + line, plane);
     double nuf[NC], nuh[NC];
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
-      const double rf = hasR ? muL[k * plane + HW_IDX(cR, plane)] : 0.0;
-      const double lf = hasL ? muL[k * plane + HW_IDX(cL, plane)] : 0.0;
-      const double rh = hasR ? muL[(fown * NC + k) * plane + HW_IDX(cR, plane)] : 0.0;
-      const double lh = hasL ? muL[(fown * NC + k) * plane + HW_IDX(cL, plane)] : 0.0;
-      nuf[k] = fu.sub(rf, lf);
-      nuh[k] = fu.sub(rh, lh);
+      const double rf = muL[k * plane + cR], lf = muL[k * plane + cL];
+      const double rh = muL[(fown * NC + k) * plane + cR], lh = muL[(fown * NC + k) * plane + cL];
+      nuf[k] = fu.sub(hasR ? rf : 0.0, hasL ? lf : 0.0);
+      nuh[k] = fu.sub(hasR ? rh : 0.0, hasL ? lh : 0.0);
     }
     if (dir == 1) {
       swap_frame<NC>(nuf);
