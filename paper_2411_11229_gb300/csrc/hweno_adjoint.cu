@@ -38,17 +38,6 @@ struct AdjWork {
   unsigned int *cells, *faces;
 };
 
-// Appends v for the threads with add set; every thread of the warp calls it, at once per warp.
-__device__ __forceinline__ void list_append(unsigned int* count, unsigned int* list, unsigned int v, bool add) {
-  const unsigned int m = __ballot_sync(0xffffffffu, add);
-  if (m == 0u) return;
-  const int lane = threadIdx.x & 31, first = __ffs(m) - 1;
-  unsigned int at = 0u;
-  if (lane == first) at = atomicAdd(count, (unsigned int)__popc(m));
-  at = __shfl_sync(0xffffffffu, at, first) + __popc(m & ((1u << lane) - 1u));
-  if (add) list[at] = v;
-}
-
 template <int DIM>
 __device__ __forceinline__ long long nfaces_dir(const Grid& g, int dir) {
   return dir == 0 ? (long long)(g.nx + 1) * g.ny : (long long)(g.ny + 1) * g.nx;
@@ -601,10 +590,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_cell_pair(Grid g, const dou
                                                                const double* __restrict__ muM, AdjWork aw) {
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   extern __shared__ ulonglong2 adj_pair_slots[];
-  const bool left =
-      p < g.plane && !adj_cell_pair(g, S, muM, aw, HW_IDX(p, g.plane), PairSlots{adj_pair_slots + threadIdx.x});
-#pragma unroll
-  for (unsigned int d = 0; d < 2; ++d) list_append(aw.count, aw.cells, (unsigned int)p * 2u + d, left);
+  if (p < g.plane && !adj_cell_pair(g, S, muM, aw, HW_IDX(p, g.plane), PairSlots{adj_pair_slots + threadIdx.x})) {
+    const unsigned int k = atomicAdd(aw.count, 2u);
+    aw.cells[k] = (unsigned int)p * 2u;
+    aw.cells[k + 1] = (unsigned int)p * 2u + 1u;
+  }
 }
 
 // -------------------------------------------------------------------------------------------
@@ -867,8 +857,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_face_pair(Grid g, const dou
   const long long nfx = (long long)(g.nx + 1) * g.ny, nf = dir == 0 ? nfx : (long long)(g.ny + 1) * g.nx;
   const long long f = (long long)blockIdx.x * kThreads + threadIdx.x;
   extern __shared__ ulonglong2 adj_pair_slots[];
-  const bool left = f < nf && !adj_face_pair(g, S, muL, aw, alpha2, dir, f, PairSlots{adj_pair_slots + threadIdx.x});
-  list_append(aw.count + 1, aw.faces, (unsigned int)(f + (dir == 0 ? 0 : nfx)), left);
+  if (f < nf && !adj_face_pair(g, S, muL, aw, alpha2, dir, f, PairSlots{adj_pair_slots + threadIdx.x}))
+    aw.faces[atomicAdd(aw.count + 1, 1u)] = (unsigned int)(f + (dir == 0 ? 0 : nfx));
 }
 
 // -------------------------------------------------------------------------------------------

@@ -47,6 +47,7 @@ namespace {
 void set_plain_scheme(hweno_ctx* h, int bc) {
   h->var = 0;
   h->flags = 0;
+  h->lists = true;
   h->grav = 0.0;
   for (int sd = 0; sd < 4; ++sd) {
     h->side[sd] = bc;
@@ -211,6 +212,8 @@ int hweno_bind(hweno_t* h, double* state_dev, void* ws) {
   h->w.gstride = gstride_of(h);
   h->w.WS = l.WS ? reinterpret_cast<double*>(p) : nullptr;
   p += l.WS;
+  h->w.left_cells = l.LEFT ? reinterpret_cast<unsigned int*>(p) : nullptr;
+  h->w.left_faces = l.LEFT ? h->w.left_cells + 2 * h->nx * h->ny : nullptr;
   h->state = state_dev;
   h->ws = static_cast<unsigned char*>(ws);
   if (cudaMemsetAsync(scal_begin, 0, l.alpha + l.scal + l.status, h->stream) != cudaSuccess) return HWENO_ECUDA;
@@ -589,6 +592,7 @@ extern "C" int hweno_rhs_static(int dim, int system, int64_t nx, int64_t ny, dou
   // the same validation as hweno_create, on a handle that lives on this stack frame
   hweno_ctx h;
   set_plain_scheme(&h, bc);
+  h.lists = false;  // no scratch for them
   if (dim != 1 && dim != 2) return HWENO_EINVAL;
   if (system < HWENO_ADVECTION || system > HWENO_EULER) return HWENO_EINVAL;
   if (bc < HWENO_BC_PERIODIC || bc > HWENO_BC_REFLECTIVE) return HWENO_EINVAL;
@@ -659,6 +663,7 @@ extern "C" int hweno_rhs_static(int dim, int system, int64_t nx, int64_t ny, dou
   h.w.status = reinterpret_cast<unsigned int*>(p);
   h.w.astride = 2;
   h.w.FS = h.w.GFS = h.w.WS = nullptr;
+  h.w.left_cells = h.w.left_faces = nullptr;
   h.w.gstride = 0;
   // the array keeps the previous call's contents: clear the wavespeed slots and the status word
   if (cudaMemsetAsync(scal_begin, 0, l.alpha + l.scal + l.status, h.stream) != cudaSuccess) return HWENO_ECUDA;

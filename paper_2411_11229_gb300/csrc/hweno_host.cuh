@@ -33,13 +33,26 @@ inline unsigned blocks_for(long long n) { return (unsigned)((n + hw::kThreads - 
 template <int DIM, int SYS, int VAR>
 struct L {
   static void cell(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
-    hw::k_cell<DIM, SYS, VAR><<<blocks_for(g.plane), hw::kThreads, 0, st>>>(g, S, w, slot);
+    if (DIM == 2 && g.listed) {
+      hw::k_cell<2, SYS, VAR, true><<<blocks_for(g.plane), hw::kThreads, 0, st>>>(g, S, w, slot);
+      if (VAR == 2) left(g, S, w, slot, st);  // R2's faces need what is left of the cells
+    } else {
+      hw::k_cell<DIM, SYS, VAR, false><<<blocks_for(g.plane), hw::kThreads, 0, st>>>(g, S, w, slot);
+    }
+  }
+  static void left(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
+    hw::k_left<2, SYS, VAR><<<3 * hw::kSMs, hw::kThreads, 0, st>>>(g, S, w, slot);
   }
   static void face(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
     const long long nfx = (long long)(g.nx + 1) * g.ny;
     const long long nfy = DIM == 2 ? (long long)(g.ny + 1) * g.nx : 0;
     dim3 grid(blocks_for(nfx > nfy ? nfx : nfy), DIM);
-    hw::k_face<DIM, SYS, VAR><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
+    if (DIM == 2 && VAR != 2 && g.listed) {
+      hw::k_face<2, SYS, VAR, true><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
+      left(g, S, w, slot, st);
+    } else {
+      hw::k_face<DIM, SYS, VAR, false><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
+    }
   }
   static void update(const Grid& g, double* S, const Work& w, int mode, int stage, double a, double b,
                      double dt, int slot, double* Lo, double* Mo, cudaStream_t st) {
@@ -79,6 +92,7 @@ struct hweno_ctx {
   // extended scheme (hweno_create_ex); var = 0 for the scheme of the paper with one boundary
   // type, 1 with any extension, 2 with the per-cell characteristic decomposition (Euler)
   int var, flags;
+  bool lists;  // whether a large grid may list what is left to the FP64 weights (listed_of)
   int side[4];
   double grav;
   double fixed[4][4];
@@ -103,10 +117,25 @@ inline int np_of(const hweno_ctx* h) { return h->system == HWENO_EULER ? (h->dim
 
 // workspace sub-buffers in bytes, in layout order
 struct Layout {
-  size_t B, MD, NOD, PRIM, FX, FY, alpha, scal, status, FS, GFS, WS, total;
+  size_t B, MD, NOD, PRIM, FX, FY, alpha, scal, status, FS, GFS, WS, LEFT, total;
 };
 
 inline long long gstride_of(const hweno_ctx* h) { return h->nx > h->ny ? h->nx : h->ny; }
+
+inline size_t nfaces_of(const hweno_ctx* h) {
+  return (size_t)(h->nx + 1) * h->ny + (h->dim == 2 ? (size_t)(h->ny + 1) * h->nx : 0);
+}
+// Whether a grid lists what is left to the FP64 weights for a kernel of its own (k_left) instead of
+// taking it block by block.  The list runs in full warps while no block waits for it: 2D Euler with
+// fronts 1703 to 1269 us a stage at 1024^2 and 348 to 272 us at 384^2, Rayleigh-Taylor at 120x480 146 to
+// 122 us; with nothing to list the launch costs 4 us (1024^2 1082 to 1086 us, 256^2 99.6 to 103.7 us).
+// Below 2^15 cells that is 6 % and more of a smooth stage.  The weighted derivative takes the FP64
+// weights everywhere and lists nothing.
+constexpr long long kListMinCells = 1LL << 15;
+inline int listed_of(const hweno_ctx* h) {
+  return h->lists && h->dim == 2 && (long long)h->nx * h->ny >= kListMinCells && !(h->flags & HWENO_FLAG_V_WEIGHTED) &&
+         nfaces_of(h) < (size_t(1) << 32);
+}
 
 inline Layout layout_of(const hweno_ctx* h) {
   const size_t plane = (size_t)h->nx * h->ny;
@@ -124,7 +153,8 @@ inline Layout layout_of(const hweno_ctx* h) {
   l.FS = h->var == 2 ? align_up((size_t)h->dim * 4 * nc * plane * 8) : 0;
   l.GFS = h->var == 2 ? align_up((size_t)h->dim * 4 * nc * (size_t)gstride_of(h) * 8) : 0;
   l.WS = (h->var != 0 && (h->flags & HWENO_FLAG_ALPHA_LOCAL)) ? align_up((size_t)h->dim * plane * 8) : 0;
-  l.total = l.B + l.MD + l.NOD + l.PRIM + l.FX + l.FY + l.alpha + l.scal + l.status + l.FS + l.GFS + l.WS;
+  l.LEFT = listed_of(h) ? align_up((2 * plane + nfaces_of(h)) * sizeof(unsigned int)) : 0;
+  l.total = l.B + l.MD + l.NOD + l.PRIM + l.FX + l.FY + l.alpha + l.scal + l.status + l.FS + l.GFS + l.WS + l.LEFT;
   return l;
 }
 
@@ -151,6 +181,7 @@ inline Grid grid_of(const hweno_ctx* h) {
   g.bc = h->bc;
   g.flags = h->flags;
   g.pairs = pairs_of(h);
+  g.listed = listed_of(h);
   g.plane = (long long)h->nx * h->ny;
   g.dx = h->dx;
   g.dy = h->dy;
@@ -334,7 +365,7 @@ inline int stage(hweno_ctx* h, const double* S_in, double* S_out, int mode, int 
   if (ev[2]) cudaEventRecord(ev[2], h->stream);
   f.update(g, S_out, h->w, mode, st, a_k[st], b_k[st], dt, slot, Lo, Mo, h->stream);
   if (ev[3]) cudaEventRecord(ev[3], h->stream);
-  h->launches += 3;
+  h->launches += 3 + g.listed;
   return cuda_status();
 }
 

@@ -41,7 +41,8 @@ struct Work {
                               // direction d at alpha[s * astride + d]
   double* scal;               // [0] dt of the current step, [1] t, [2] t_end, [3] steps taken,
                               // [4..7] zero (read by fu_of; never written after creation)
-  unsigned int* status;       // bit 0: non-physical state met
+  unsigned int* status;       // [0] bit 0: non-physical state met; [2], [3] entries in left_cells and
+                              // left_faces (zero between stages)
   long long astride;          // distance between slots (2 for a single grid)
   // R2 only: face states of every cell, normal frame:
   // FS [DIM][4][NC][plane] = (u^- and v^- at the right face, u^+ and v^+ at the left face);
@@ -52,6 +53,9 @@ struct Work {
   long long gstride;
   // local LF coefficients only: the spectral radius of every cell per direction [DIM][plane]
   double* WS;
+  // listed grids only: cell * 2 + direction of the cells, x faces then y faces of the faces, that k_cell
+  // and k_face leave to k_left
+  unsigned int *left_cells, *left_faces;
 };
 
 
@@ -548,7 +552,9 @@ __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restric
 
 // The cells or faces of one block whose nonlinear weights are to be evaluated in FP64: the block's
 // threads take them in turn afterwards, so that a warp with a single one of them does not run the
-// FP64 path for its other lanes (an FP64 warp instruction costs the same with one lane active).
+// FP64 path for its other lanes (an FP64 warp instruction costs the same with one lane active).  A
+// block that has any keeps its place on the SM for one more pass of FP64 work in one or two warps;
+// listed grids append theirs to one list instead, which k_left takes in full warps.
 struct Leftover {
   int n;
   unsigned short item[2 * kThreads];
@@ -556,11 +562,20 @@ struct Leftover {
 
 // The cells p0 .. p0 + kThreads - 1 of a block, one per thread; every thread of the block calls it.
 // reused: the block calls it again with the same list.
-template <int DIM, int SYS, int VAR>
+template <int DIM, int SYS, int VAR, bool LISTED>
 __device__ __forceinline__ void cell_tile(const Grid& g, const double* __restrict__ S, const Work& w, long long p0,
                                           double& wsx, double& wsy, Leftover& lo, const PairSlots& sm,
                                           bool reused) {
   const long long p = p0 + threadIdx.x;
+  if (LISTED) {
+    // (one atomic per thread: collected by warp, the kernel takes 3 % longer with nothing to append)
+    if (p < g.plane && !cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm)) {
+      const unsigned int k = atomicAdd(w.status + 2, (unsigned int)DIM);
+#pragma unroll
+      for (unsigned int d = 0; d < DIM; ++d) w.left_cells[k + d] = (unsigned int)p * 2u + d;
+    }
+    return;
+  }
   if (DIM == 1 && !g.pairs) {
     if (p < g.plane) {
       cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm);
@@ -587,13 +602,13 @@ __device__ __forceinline__ void cell_tile(const Grid& g, const double* __restric
 
 // Bound by the FP64 pipe (85 % busy): 123 FP64 instructions per 2D Euler cell against 545 with the FP64
 // weights; 1024^2 0.24 ms per launch against 0.97 ms.
-template <int DIM, int SYS, int VAR>
+template <int DIM, int SYS, int VAR, bool LISTED>
 __global__ void __launch_bounds__(kThreads, 4) k_cell(Grid g, const double* __restrict__ S, Work w, int slot) {
   __shared__ Leftover lo;
   __shared__ ulonglong2 slots[4 * Traits<DIM, SYS>::NC * kThreads];
   double wsx = 0.0, wsy = 0.0;
-  cell_tile<DIM, SYS, VAR>(g, S, w, (long long)blockIdx.x * kThreads, wsx, wsy, lo, PairSlots{slots + threadIdx.x},
-                           false);
+  cell_tile<DIM, SYS, VAR, LISTED>(g, S, w, (long long)blockIdx.x * kThreads, wsx, wsy, lo,
+                                   PairSlots{slots + threadIdx.x}, false);
   block_max2(wsx, wsy, w.alpha + slot * w.astride);
 }
 
@@ -947,11 +962,16 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
 
 // The faces f0 .. f0 + kThreads - 1 (of nf) of direction dir, one per thread; every thread of the
 // block calls it.  reused: as cell_tile.
-template <int DIM, int SYS, int VAR>
+template <int DIM, int SYS, int VAR, bool LISTED>
 __device__ __forceinline__ void face_tile(const Grid& g, const double* __restrict__ S, const Work& w, int dir,
                                           long long f0, long long nf, double alpha, Leftover& lo,
                                           const PairSlots& sm, bool reused) {
   const long long f = f0 + threadIdx.x;
+  if (LISTED && VAR != 2) {
+    if (f < nf && !face_body<DIM, SYS, VAR, true>(g, S, w, dir, f, alpha, sm))
+      w.left_faces[atomicAdd(w.status + 3, 1u)] = (unsigned int)(f + (dir == 0 ? 0 : (long long)(g.nx + 1) * g.ny));
+    return;
+  }
   // R2: only the fluxes (k_cell formed the face states); the weighted derivative needs the weights
   // themselves
   if (VAR == 2 || !g.pairs || (VAR && (g.flags & FLAG_V_WEIGHTED))) {
@@ -973,7 +993,7 @@ __device__ __forceinline__ void face_tile(const Grid& g, const double* __restric
 // per SM (128 registers) cover it better than three or five (2D Euler 2048^2 with k_cell likewise: 4.70
 // against 4.75 and 4.94 ms per stage, before the pairs' loops).  2D Euler 1024^2: 0.70 ms per launch
 // against 2.33 ms with the FP64 weights.
-template <int DIM, int SYS, int VAR>
+template <int DIM, int SYS, int VAR, bool LISTED>
 __global__ void __launch_bounds__(kThreads, 4) k_face(Grid g, const double* __restrict__ S, Work w, int slot) {
   __shared__ Leftover lo;
   constexpr bool kSlots = SYS == SYS_EULER && VAR != 2;  // scalar laws and R2's faces use none
@@ -981,9 +1001,32 @@ __global__ void __launch_bounds__(kThreads, 4) k_face(Grid g, const double* __re
   const int dir = blockIdx.y;
   const int n = dir == 0 ? g.nx : g.ny;
   const int nlines = dir == 0 ? g.ny : g.nx;
-  face_tile<DIM, SYS, VAR>(g, S, w, dir, (long long)blockIdx.x * kThreads, (long long)(n + 1) * nlines,
-                           __longlong_as_double((long long)w.alpha[slot * w.astride + dir]), lo,
-                           PairSlots{slots + (kSlots ? threadIdx.x : 0)}, false);
+  face_tile<DIM, SYS, VAR, LISTED>(g, S, w, dir, (long long)blockIdx.x * kThreads, (long long)(n + 1) * nlines,
+                                   __longlong_as_double((long long)w.alpha[slot * w.astride + dir]), lo,
+                                   PairSlots{slots + (kSlots ? threadIdx.x : 0)}, false);
+}
+
+// The listed cells and faces of a stage with the FP64 weights, in full warps (faces first, then cells): a
+// fixed grid, three blocks of 128 per SM as the FP64 path's registers allow.  It is bound by the FP64
+// pipe (about 560 instructions a face) and idle when the lists are empty.
+template <int DIM, int SYS, int VAR>
+__global__ void __launch_bounds__(kThreads, 3) k_left(Grid g, const double* __restrict__ S, Work w, int slot) {
+  const long long nfx = (long long)(g.nx + 1) * g.ny, all = nfx + (DIM == 2 ? (long long)(g.ny + 1) * g.nx : 0);
+  const long long nf = min((long long)w.status[3], all), nfw = (nf + 31) / 32 * 32;
+  const long long nc = min((long long)w.status[2], DIM * g.plane);
+  const PairSlots none{nullptr};
+  for (long long k = (long long)blockIdx.x * kThreads + threadIdx.x; k < nfw + nc; k += (long long)gridDim.x * kThreads) {
+    if (k < nf) {
+      const long long f = HW_IDX(w.left_faces[k], all);
+      const int dir = f < nfx ? 0 : 1;
+      if (f < all)
+        face_body<DIM, SYS, VAR, false>(g, S, w, dir, f - (dir == 0 ? 0 : nfx),
+                                        __longlong_as_double((long long)w.alpha[slot * w.astride + dir]), none);
+    } else if (k >= nfw) {
+      const unsigned int c = w.left_cells[k - nfw];
+      if ((long long)(c >> 1) < g.plane) cell_limiter<DIM, SYS, VAR>(g, S, w, HW_IDX(c >> 1, g.plane), (int)(c & 1u));
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1077,6 +1120,7 @@ __global__ void __launch_bounds__(kThreads) k_update(Grid g, double* __restrict_
                                                       double a_k, double b_k, double dt_fixed, int slot,
                                                       double* __restrict__ Lout, double* __restrict__ Mout) {
   __shared__ double s_dt;
+  if (g.listed && blockIdx.x == 0 && threadIdx.x == 0) w.status[2] = w.status[3] = 0u;
   if (mode == 0) {
     if (threadIdx.x == 0) {
       const double dt = stage_dt<DIM>(g, w, stage, dt_fixed, slot);

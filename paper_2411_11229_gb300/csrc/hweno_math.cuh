@@ -41,6 +41,7 @@ struct Grid {
   int bc;
   int flags;    // FLAG_* (read by the extended kernels only)
   int pairs;    // whether the nonlinear part is taken in pairs where it may be (see hweno_host.cuh)
+  int listed;   // whether what is left to the FP64 weights goes to the grid's list (see hweno_host.cuh)
   long long plane;  // nx * ny
   double dx, dy, inv_dx, inv_dy;
   double gamma, gm1;
