@@ -49,6 +49,25 @@ def test_steps_euler(n, bc):
     _same(a, b)
 
 
+# four warps to a block's cells: 28 of them at most, up to 152 blocks
+@pytest.mark.parametrize("n", [27, 28, 29, 56, 57, 59, 4255, 4256, 4257])
+@pytest.mark.parametrize("system,bc", [("advection", "periodic"), ("advection", "transmissive"),
+                                       ("burgers", "periodic"), ("burgers", "transmissive"), ("euler", "periodic"),
+                                       ("euler", "transmissive"), ("euler", "reflective")])
+def test_steps_four_warps(system, n, bc):
+    if system == "euler":
+        S, dx = W.euler1d_random(n, seed=n, kind="smooth" if n % 2 else "jumps")
+    else:
+        S, dx, _ = W.scalar_random(1, n, 1, seed=n, kind="smooth" if n % 2 else "jumps")
+    a, b = _pair(system, n, bc, S, dx)
+    for s in (a, b):
+        s.set_time(0.0, 0.0)
+        s.step(0.0, 3)
+        s.step(1e-4 * dx, 1)
+        s.step(0.0, 2)
+    _same(a, b)
+
+
 @pytest.mark.parametrize("system", ["advection", "burgers"])
 @pytest.mark.parametrize("n", [40, 124, 125, 161, 3001])
 def test_steps_scalar(system, n):
