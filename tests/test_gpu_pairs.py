@@ -136,3 +136,40 @@ def test_adjoint_scales_with_its_seeds(nx, ny, bc, kind):
         err = np.abs(_planes(out[k]) - _planes(ref)).max(axis=1) / np.abs(_planes(ref)).max(axis=1)
         assert (err <= 1e-10).all(), (k, err)
     assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+
+
+@pytest.mark.parametrize("kind", ["none", "corner", "all"])
+@pytest.mark.parametrize("system,nx,ny,bc,flags", [
+    ("euler", 181, 181, "periodic", 0), ("euler", 128, 256, "periodic", 0), ("euler", 1001, 33, "reflective", 0),
+    ("euler", 33, 1001, "transmissive", 4), ("burgers", 256, 129, "periodic", 0)])
+def test_left_to_the_fp64_weights(system, nx, ny, bc, flags, kind):
+    """Grids on both sides of the size from which the cells and faces of the FP64 weights go through the
+    grid's list (2^15 cells), with none, some and every one of them in it; again on a handle whose list
+    has been used."""
+    if system == "euler":
+        S, dx, dy = W.euler2d_random(nx, ny, seed=2, kind="smooth")
+        mean = S[0].mean(axis=(1, 2), keepdims=True)
+    else:
+        S, dx, dy = W.scalar_random(2, nx, ny, seed=2, kind="smooth")
+        mean = 0.3 + 0 * S[0].mean(axis=(1, 2), keepdims=True)
+    amp = 1e-3 if kind != "all" else 0.05
+    S[0] = mean + amp * (S[0] - mean)
+    S[1:] *= amp
+    if kind == "corner":
+        S[0, 0, : ny // 3, : nx // 4] *= 1.5
+    if kind == "all":
+        r = np.random.default_rng(7)
+        S[0] *= 1.0 + 0.1 * r.uniform(-1.0, 1.0, size=S[0, :1].shape)
+    cfg = O.make_cfg(2, getattr(O, system.upper()), nx, ny, dx=dx, dy=dy, bc=getattr(O, "BC_" + bc.upper()),
+                     flags=flags)
+    s = Solver(2, system, nx, ny, dx=dx, dy=dy, bc=bc, flags=flags)
+    Le, Me = O.rhs_ext(cfg, S)[:2]
+    Lo, Mo = O.rhs(cfg, S)
+    for _ in range(2):
+        s.set_state(S)
+        L, M = s.rhs()
+        _check(L.cpu().numpy(), Le, Lo)
+        _check(M.cpu().numpy(), Me, Mo)
+        s.set_time(0.0, 0.0)
+        s.step(0.0, 2)
+    s.sync()
