@@ -160,7 +160,8 @@ int hweno_rhs(hweno_t *h, const double *S_dev, double *L_dev, double *M_dev);
  * has dt = 0 and leaves the state unchanged.  No host synchronisation. */
 int hweno_step(hweno_t *h, double dt);
 
-/* nsteps calls of hweno_step(h, dt). */
+/* nsteps calls of hweno_step(h, dt).  1D grids of the plain scheme up to 18848 cells (152 SMs x 124) take
+ * them in one cooperative launch, if the device can hold it; every other grid stage by stage. */
 int hweno_steps(hweno_t *h, double dt, int nsteps);
 
 /* Device time and end time used by CFL steps (t_end <= 0: no clamp); resets the count of steps
@@ -213,7 +214,8 @@ int hweno_pipeline(hweno_t *h, int count, const double *const *host_in, double *
                    int depth, void *slot_mem);
 
 /* Per-kernel timing (tracing aid).  When on, every stage records CUDA events on the handle's
- * stream around its three launches (cell, face, update kernels).  hweno_kernel_times()
+ * stream around its launches (cell; face, with the kernel of what is left to the FP64 weights; update).
+ * A small 1D grid then takes its steps by stages, not in its one launch.  hweno_kernel_times()
  * synchronises, returns the summed milliseconds and launch counts per kernel kind in
  * ms3[0..2], n3[0..2] (cell, face, update) since the previous query, and resets them. */
 int hweno_set_profiling(hweno_t *h, int on);
@@ -231,7 +233,7 @@ const char *hweno_strerror(int status);
  * first one recorded, and the access redirected to element 0 of its array.  Synchronises the
  * device and returns the number of such indices since the previous call (then clears it); *where
  * (may be NULL) receives the first one's source line plus 100000 x its translation unit (0: entry
- * points and stage kernels, 1: batched, 2: adjoint).  Returns -1 in a normal build, HWENO_ECUDA if
+ * points and stage kernels, 1: batched, 2: adjoint, 3: steps of small 1D grids).  Returns -1 in a normal build, HWENO_ECUDA if
  * the synchronisation fails. */
 long long hweno_bounds_status(int *where);
 

@@ -38,11 +38,6 @@ struct AdjWork {
   unsigned int *cells, *faces;
 };
 
-template <int DIM>
-__device__ __forceinline__ long long nfaces_dir(const Grid& g, int dir) {
-  return dir == 0 ? (long long)(g.nx + 1) * g.ny : (long long)(g.ny + 1) * g.nx;
-}
-
 // -------------------------------------------------------------------------------------------
 template <int DIM>
 __device__ __forceinline__ void adj_cell(const Grid& g, const double* __restrict__ S, const double* __restrict__ muM,

@@ -199,14 +199,12 @@ inline Grid grid_of(const hweno_ctx* h) {
   g.cfl = h->cfl;
   // folded constants (see hw::Grid)
   const double g1 = g.g1;
+  // (p0 - gamma1 (p1 + p2)) / gamma1 on (um, u0, up, hvm, hvp) at the right face x_{i+1/2} and, mirrored,
+  // at the left face x_{i-1/2}
   const double cr[5] = {(-0.125 + 0.5 * g1) / g1, (0.5625 - 2.0 * g1) / g1, (0.5625 - 0.5 * g1) / g1,
                         -0.046875 / g1, -0.140625 / g1};
   const double cl[5] = {(0.5625 - 0.5 * g1) / g1, (0.5625 - 2.0 * g1) / g1, (-0.125 + 0.5 * g1) / g1,
                         0.140625 / g1, 0.046875 / g1};
-  for (int k = 0; k < 5; ++k) {
-    g.cr[k] = cr[k];
-    g.cl[k] = cl[k];
-  }
   // the centre-value-free forms: right face on (d01, d12, hvm, hvp) of the stencil {i-1, i, i+1};
   // left face (mirror) on (d_{i,i+1} of its own stencil's first pair, second pair, h v_{i-1}, h v_{i+1})
   const double dm[4] = {-cr[0], cr[2], cr[3], cr[4]};

@@ -1,6 +1,7 @@
 // Stage kernels of the HWENO-I scheme (Xie, Tao, Jiao, Zhang, arXiv 2411.11229) for sm_103a.
 //
-// One Runge-Kutta stage is three launches over the grid:
+// One Runge-Kutta stage is three launches over the grid, and on 2D grids from 2^15 cells a fourth (k_left)
+// for the cells and faces whose nonlinear part needs the FP64 weights:
 //   k_cell   per cell : wavespeed (LF alpha of the stage input), nodal fluxes f, h = f'(u) v (and
 //                       the mixed-flux nodal values in 2D) for the D-terms (Eqs. Cd-1, DfDh, mixed),
 //                       Euler primitives for the Roe averages, and the modified derivative v~

@@ -51,11 +51,9 @@ struct Grid {
   double eps;       // epsilon of Eq. (nonlinear)
   double cfl;
   // Folded constants (computed on the host from the linear weights and the spacings):
-  //   cr, cl: coefficients of (p0 - gamma1 (p1 + p2)) / gamma1 on (um, u0, up, hvm, hvp) at the
-  //           right face x_{i+1/2} and, mirrored, at the left face x_{i-1/2};
   //   G = gamma0 / gamma1;  limiter: cdu = (3/4 - d1)/d1, Gd = d0 / d1;
   //   per direction: h, 1/h, ch*h, ef/h, eg/h (D-terms), 1/(2h).
-  double cr[5], cl[5], G;
+  double G;
   double cdu, Gd;
   // The arithmetic with the derivatives entering unscaled (v, not h v), per direction: the h of
   // every derivative term folded into its coefficient (the forward and the adjoint kernels).
@@ -607,11 +605,6 @@ __device__ __forceinline__ int bc_map_ext(int k, int n, int lo, int hi, bool& re
     return k < 0 ? 0 : n - 1;
   }
   return bc_map(k, n, t, refl);
-}
-
-__device__ __forceinline__ int bc_index(int k, int n, int bc) {
-  bool refl;
-  return bc_map(k, n, bc, refl);
 }
 
 // -x when b, else x: a flip of the sign bit in the integer pipe, so that a data-dependent sign
