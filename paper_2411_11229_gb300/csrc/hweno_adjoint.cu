@@ -17,7 +17,7 @@
 // Contributions are stored per face / per cell and gathered (no atomics: deterministic).
 // In 2D, k_adj_cell_pair and k_adj_face_pair form the same contributions with the transposes of the
 // nonlinear part in pairs (hweno_adjoint_pair.cuh) and list the cells and faces that need the FP64 weights
-// for k_adj_cell and k_adj_face.  1D grids are too small to fill the FP64 pipe and keep the FP64 kernels.
+// for k_adj_cell and k_adj_face.  1D grids, and 2D ones up to kAdjPairMinCells, are too small to fill the FP64 pipe and keep the FP64 kernels.
 #include <cmath>
 #include "hweno_adjoint.cuh"
 #include "hweno_adjoint_pair.cuh"
@@ -164,7 +164,7 @@ __device__ __forceinline__ void adj_cell(const Grid& g, const double* __restrict
   }
 }
 
-// 1D: every cell; 2D: the cells of the list
+// 1D: every cell; 2D: the cells of the list, or every one where there is no list
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_adj_cell(Grid g, const double* __restrict__ S, const double* __restrict__ muM,
                                                        AdjWork aw) {
@@ -173,9 +173,9 @@ __global__ void __launch_bounds__(kThreads) k_adj_cell(Grid g, const double* __r
     if (k < g.plane) adj_cell<1>(g, S, muM, aw, 0, k);
     return;
   }
-  const long long n = min((long long)aw.count[0], 2 * g.plane);
+  const long long n = aw.cells ? min((long long)aw.count[0], 2 * g.plane) : 2 * g.plane;
   for (; k < n; k += (long long)gridDim.x * kThreads) {
-    const unsigned int c = aw.cells[k];
+    const unsigned int c = aw.cells ? aw.cells[k] : (unsigned int)k;
     if ((long long)(c >> 1) < g.plane) adj_cell<DIM>(g, S, muM, aw, (int)(c & 1u), HW_IDX(c >> 1, g.plane));
   }
 }
@@ -395,7 +395,7 @@ __device__ __forceinline__ void adj_face(const Grid& g, const double* __restrict
   }
 }
 
-// 1D: every face; 2D: the faces of the list
+// 1D: every face; 2D: the faces of the list, or every one where there is no list
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_adj_face(Grid g, const double* __restrict__ S, const double* __restrict__ muL,
                                                        AdjWork aw, const double* __restrict__ alpha2) {
@@ -405,9 +405,10 @@ __global__ void __launch_bounds__(kThreads) k_adj_face(Grid g, const double* __r
     if (k < nfx) adj_face<1>(g, S, muL, aw, alpha2, 0, k);
     return;
   }
-  const long long all = nfx + (long long)(g.ny + 1) * g.nx, n = min((long long)aw.count[1], all);
+  const long long all = nfx + (long long)(g.ny + 1) * g.nx;
+  const long long n = aw.faces ? min((long long)aw.count[1], all) : all;
   for (; k < n; k += (long long)gridDim.x * kThreads) {
-    const long long f = HW_IDX(aw.faces[k], all);
+    const long long f = HW_IDX(aw.faces ? (long long)aw.faces[k] : k, all);
     if (f < all) adj_face<DIM>(g, S, muL, aw, alpha2, f < nfx ? 0 : 1, f < nfx ? f : f - nfx);
   }
 }
@@ -1123,6 +1124,12 @@ AdjPtrs adj_ptrs(const hweno_ctx* h, void* ws) {
   return a;
 }
 
+// From this many cells on a 2D grid's VJP takes the pairs: below it there is at most one warp of faces to a
+// scheduler, whose FP64 pipe waits for that warp's chain of instructions, the longer one in pairs, and the
+// kernels of the lists find little or nothing to do.  One step forward and back at 46x146 1.23 ms in FP64,
+// 1.50 in pairs; at 128^2 1.49 and 1.51, at 160^2 1.96 and 1.64.
+constexpr long long kAdjPairMinCells = hw::kSMs * 4LL * 32 / 2;
+
 template <int DIM>
 int stage_vjp(const hweno_ctx* h, const Grid& g, const double* S, const double* alpha2, const double* muM,
               const double* muL, const hw::AdjWork& aw, double* lam) {
@@ -1152,11 +1159,16 @@ int stage_vjp(const hweno_ctx* h, const Grid& g, const double* S, const double* 
         cudaFuncSetAttribute(hw::k_adj_cell_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_sm) !=
             cudaSuccess)
       return HWENO_ECUDA;
-    if (cudaMemsetAsync(aw.count, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) return HWENO_ECUDA;
-    hw::k_adj_cell_pair<<<bc, hw::kThreads, pair_sm, st>>>(g, S, muM, aw);
-    hw::k_adj_face_pair<<<dim3(bf, 2), hw::kThreads, pair_sm, st>>>(g, S, muL, aw, alpha2);
-    hw::k_adj_cell<DIM><<<bl < 2 * bc ? bl : 2 * bc, hw::kThreads, cell_sm, st>>>(g, S, muM, aw);
-    hw::k_adj_face<DIM><<<bl < 2 * bf ? bl : 2 * bf, hw::kThreads, face_sm, st>>>(g, S, muL, aw, alpha2);
+    hw::AdjWork fw = aw;
+    if (g.plane >= kAdjPairMinCells) {
+      if (cudaMemsetAsync(aw.count, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) return HWENO_ECUDA;
+      hw::k_adj_cell_pair<<<bc, hw::kThreads, pair_sm, st>>>(g, S, muM, aw);
+      hw::k_adj_face_pair<<<dim3(bf, 2), hw::kThreads, pair_sm, st>>>(g, S, muL, aw, alpha2);
+    } else {
+      fw.cells = fw.faces = nullptr;
+    }
+    hw::k_adj_cell<DIM><<<bl < 2 * bc ? bl : 2 * bc, hw::kThreads, cell_sm, st>>>(g, S, muM, fw);
+    hw::k_adj_face<DIM><<<bl < 2 * bf ? bl : 2 * bf, hw::kThreads, face_sm, st>>>(g, S, muL, fw, alpha2);
   }
   hw::k_adj_gather<DIM><<<bc, hw::kThreads, 0, st>>>(g, S, muM, muL, aw, lam);
   return cudaGetLastError() == cudaSuccess ? HWENO_OK : HWENO_ECUDA;

@@ -106,7 +106,10 @@ def test_constant_state_stays_constant():
 
 
 @pytest.mark.parametrize("kind", ["smooth", "jumps"])
-@pytest.mark.parametrize("nx,ny,bc", [(67, 41, "periodic"), (5, 130, "transmissive"), (40, 33, "reflective")])
+@pytest.mark.parametrize("nx,ny,bc", [(67, 41, "periodic"), (5, 130, "transmissive"), (40, 33, "reflective"),
+                                      # both sides of the size from which the pairs are used (9728 cells)
+                                      (97, 100, "periodic"), (128, 76, "periodic"), (101, 97, "reflective"),
+                                      (13, 801, "transmissive"), (801, 13, "reflective")])
 def test_adjoint_scales_with_its_seeds(nx, ny, bc, kind):
     """The stage VJP against the oracle's (1e-10, the bar of the adjoint tests), and exactly linear under
     powers of two of any size: the pairs take each thread's seeds relative to their largest."""
