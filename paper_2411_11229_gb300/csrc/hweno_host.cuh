@@ -125,6 +125,21 @@ inline long long gstride_of(const hweno_ctx* h) { return h->nx > h->ny ? h->nx :
 inline size_t nfaces_of(const hweno_ctx* h) {
   return (size_t)(h->nx + 1) * h->ny + (h->dim == 2 ? (size_t)(h->ny + 1) * h->nx : 0);
 }
+// Cells of a 1D grid that one block of each SM can hold (hweno_line.cu)
+constexpr long long kLineMaxCells = hw::kSMs * (hw::kThreads - 4LL);
+
+// The nonlinear part in pairs (hweno_pair.cuh) trades FP64 instructions for several times as many FP32
+// ones, which pays where the FP64 pipe is kept busy.  A grid of at most one warp of cells per scheduler
+// leaves it idle and waits for each thread's chain of instructions instead, which is the longer one in
+// pairs: one evaluation of 1D Euler at 2048 cells 43 us in FP64, 53 us in pairs; of 2D Euler at 48^2
+// 62 and 74 us (with fronts 60 and 82), at 96x170 84 and 80 (83 and 98), at 128x200 123 and 88 (123 and
+// 111).  A scalar law's chain is short: at 182x181 40 and 46 us, at 256^2 58 and 48.
+constexpr long long kPairMinCells = hw::kSMs * 4LL * 32;
+inline int pairs_of(const hweno_ctx* h) {
+  if (h->dim == 1) return h->nx > kLineMaxCells;
+  return (long long)h->nx * h->ny > kPairMinCells * (h->system == hw::SYS_EULER ? 1 : 2);
+}
+
 // Whether a grid lists what is left to the FP64 weights for a kernel of its own (k_left) instead of
 // taking it block by block.  The list runs in full warps while no block waits for it: 2D Euler with
 // fronts 1703 to 1269 us a stage at 1024^2 and 348 to 272 us at 384^2, Rayleigh-Taylor at 120x480 146 to
@@ -133,7 +148,7 @@ inline size_t nfaces_of(const hweno_ctx* h) {
 // weights everywhere and lists nothing.
 constexpr long long kListMinCells = 1LL << 15;
 inline int listed_of(const hweno_ctx* h) {
-  return h->lists && h->dim == 2 && (long long)h->nx * h->ny >= kListMinCells && !(h->flags & HWENO_FLAG_V_WEIGHTED) &&
+  return h->lists && h->dim == 2 && pairs_of(h) && (long long)h->nx * h->ny >= kListMinCells && !(h->flags & HWENO_FLAG_V_WEIGHTED) &&
          nfaces_of(h) < (size_t(1) << 32);
 }
 
@@ -163,16 +178,6 @@ inline void to_pair(double x, float* p) {
   p[0] = (float)x;
   p[1] = (float)(x - (double)p[0]);
 }
-
-// Cells of a 1D grid that one block of each SM can hold (hweno_line.cu)
-constexpr long long kLineMaxCells = hw::kSMs * (hw::kThreads - 4LL);
-
-// The nonlinear part in pairs (hweno_pair.cuh) trades FP64 instructions for several times as many FP32
-// ones, which pays where the FP64 pipe is kept busy.  A 1D grid of at most one warp per scheduler
-// leaves it idle and waits for each thread's chain of instructions instead, which is the longer one in
-// pairs: one stage of 2048 cells in the stage kernels 43 us in FP64, 53 us in pairs.  A 2D grid of 64^2
-// cells (128 warps of cells, 260 of faces) already gains: 64 us in FP64, 48 us in pairs.
-inline int pairs_of(const hweno_ctx* h) { return h->dim == 2 || h->nx > kLineMaxCells; }
 
 inline Grid grid_of(const hweno_ctx* h) {
   Grid g;

@@ -521,12 +521,13 @@ __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restric
     }
     // modified derivatives (Eq. limiter), one per direction; the weighted derivative of R2 needs the
     // weights themselves
-    if (DIM == 1 && !g.pairs) {
+    if (!g.pairs) {
       if (SYS == SYS_EULER && VAR != 2) {
         double* P = reinterpret_cast<double*>(w.PRIM);
         P[p] = sqrt_fast(U[0], f);
         P[plane + p] = u;
-        P[2 * plane + p] = f.mul(f.add(U[NC - 1], pr), ir);
+        if (DIM == 2) P[2 * plane + p] = v;
+        P[DIM * plane + plane + p] = f.mul(f.add(U[NC - 1], pr), ir);
       }
       return false;
     }
@@ -577,10 +578,11 @@ __device__ __forceinline__ void cell_tile(const Grid& g, const double* __restric
     }
     return;
   }
-  if (DIM == 1 && !g.pairs) {
+  if (!g.pairs) {
     if (p < g.plane) {
       cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm);
-      cell_limiter<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), 0);
+#pragma unroll 1
+      for (int d = 0; d < DIM; ++d) cell_limiter<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), d);
     }
     return;
   }
@@ -854,14 +856,15 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const double* U = Uq[1 + q];
-          if (DIM == 1 && !g.pairs) {
+          if (!g.pairs) {
             const double* P = reinterpret_cast<const double*>(w.PRIM);
             const bool fx = VAR && fixed[1 + q];
             const double* F = g.fixP[fside[1 + q]];
+            const int kn = DIM == 2 && dir == 1 ? 2 : 1;  // the normal velocity
             sq[q] = fx ? F[0] : P[pc[1 + q]];
-            uq[q] = neg_if(fx ? F[1] : P[plane + pc[1 + q]], refl[1 + q]);
-            Hq[q] = fx ? F[2] : P[2 * plane + pc[1 + q]];
-            vq[q] = 0.0;
+            uq[q] = neg_if(fx ? F[kn] : P[kn * plane + pc[1 + q]], refl[1 + q]);
+            vq[q] = DIM == 1 ? 0.0 : (fx ? F[3 - kn] : P[(3 - kn) * plane + pc[1 + q]]);
+            Hq[q] = fx ? F[DIM + 1] : P[(DIM + 1) * plane + pc[1 + q]];
             continue;
           }
           const double ir = rcp(U[0], fu);
