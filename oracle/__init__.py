@@ -109,6 +109,7 @@ def lib():
             L.oracle_count_flops.argtypes = [CP, ctypes.POINTER(ctypes.c_longlong)]
             L.oracle_count_stencil.argtypes = [ctypes.POINTER(ctypes.c_longlong)]
             L.oracle_stage_vjp.argtypes = [CP, _P, ctypes.c_double, ctypes.c_double, _P, _P, _P]
+            L.oracle_stage_vjp_ext.argtypes = [CP, _P, ctypes.c_double, ctypes.c_double, _P, _P, _P]
             L.oracle_stage_jvp.argtypes = [CP, _P, ctypes.c_double, ctypes.c_double, _P, _P, _P]
             L.oracle_steps_record.argtypes = [CP, _P, ctypes.c_int, ctypes.c_double, _P, _P]
             L.oracle_steps_replay.argtypes = [CP, _P, ctypes.c_int, _P, _P]
@@ -270,6 +271,15 @@ def stage_vjp(cfg: Cfg, S, alpha, muM, muL):
     lam = np.zeros_like(S)
     _check(lib().oracle_stage_vjp(ctypes.byref(cfg), _ptr(S), float(alpha[0]), float(alpha[1]), _ptr(muM),
                                   _ptr(muL), _ptr(lam)))
+    return lam
+
+
+def stage_vjp_ext(cfg: Cfg, S, alpha, muM, muL):
+    """stage_vjp in long double (the adjoint of the same formulas), rounded to double once."""
+    S, muM, muL = (np.ascontiguousarray(a, dtype=np.float64) for a in (S, muM, muL))
+    lam = np.zeros_like(S)
+    _check(lib().oracle_stage_vjp_ext(ctypes.byref(cfg), _ptr(S), float(alpha[0]), float(alpha[1]), _ptr(muM),
+                                      _ptr(muL), _ptr(lam)))
     return lam
 
 

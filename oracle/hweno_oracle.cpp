@@ -1016,16 +1016,18 @@ inline Counted sqrt(const Counted& a) {
 // derivatives); one reverse sweep gives the gradient of a weighted sum of outputs.  The tape is
 // kept per face or per cell (the operator is local), so its size stays small.
 // Forward mode: `Dual` carries one directional derivative through the same code.
+// Both in a scalar T: double, or long double for the extended-precision evaluation.
+template <class T>
 struct Tape {
   std::vector<int> a, b;
-  std::vector<double> da, db;
+  std::vector<T> da, db;
   void clear() {
     a.clear();
     b.clear();
     da.clear();
     db.clear();
   }
-  int push(int ia, double pa, int ib, double pb) {
+  int push(int ia, T pa, int ib, T pb) {
     a.push_back(ia);
     b.push_back(ib);
     da.push_back(pa);
@@ -1034,43 +1036,48 @@ struct Tape {
   }
   size_t size() const { return a.size(); }
 };
-inline Tape& tape() {
-  static thread_local Tape t;
+template <class T>
+inline Tape<T>& tape() {
+  static thread_local Tape<T> t;
   return t;
 }
 
+template <class T>
 struct Adj {
-  double v;
+  T v;
   int id;  // tape index, -1 for a constant
   Adj() : v(0.0), id(-1) {}
-  Adj(double x) : v(x), id(-1) {}
-  Adj(double x, int i) : v(x), id(i) {}
+  Adj(T x) : v(x), id(-1) {}
+  Adj(T x, int i) : v(x), id(i) {}
+  static Adj var(T x) { return Adj(x, tape<T>().push(-1, 0.0, -1, 0.0)); }
+  static Adj node(T v, int ia, T pa, int ib, T pb) {
+    if (ia < 0 && ib < 0) return Adj(v);
+    return Adj(v, tape<T>().push(ia, pa, ib, pb));
+  }
+  friend Adj operator+(const Adj& x, const Adj& y) { return node(x.v + y.v, x.id, 1.0, y.id, 1.0); }
+  friend Adj operator-(const Adj& x, const Adj& y) { return node(x.v - y.v, x.id, 1.0, y.id, -1.0); }
+  friend Adj operator*(const Adj& x, const Adj& y) { return node(x.v * y.v, x.id, y.v, y.id, x.v); }
+  friend Adj operator/(const Adj& x, const Adj& y) {
+    const T q = x.v / y.v;
+    return node(q, x.id, T(1.0) / y.v, y.id, -q / y.v);
+  }
+  friend Adj operator-(const Adj& x) { return node(-x.v, x.id, -1.0, -1, 0.0); }
+  friend bool operator>(const Adj& x, const Adj& y) { return x.v > y.v; }
+  friend Adj fabs(const Adj& x) {
+    return node(std::fabs(x.v), x.id, x.v > 0 ? 1.0 : (x.v < 0 ? -1.0 : 0.0), -1, 0.0);
+  }
+  friend Adj sqrt(const Adj& x) {
+    const T r = std::sqrt(x.v);
+    return node(r, x.id, T(0.5) / r, -1, 0.0);
+  }
 };
-inline Adj adj_var(double x) { return Adj(x, tape().push(-1, 0.0, -1, 0.0)); }
-inline Adj adj_node(double v, int ia, double pa, int ib, double pb) {
-  if (ia < 0 && ib < 0) return Adj(v);
-  return Adj(v, tape().push(ia, pa, ib, pb));
-}
-inline Adj operator+(const Adj& x, const Adj& y) { return adj_node(x.v + y.v, x.id, 1.0, y.id, 1.0); }
-inline Adj operator-(const Adj& x, const Adj& y) { return adj_node(x.v - y.v, x.id, 1.0, y.id, -1.0); }
-inline Adj operator*(const Adj& x, const Adj& y) { return adj_node(x.v * y.v, x.id, y.v, y.id, x.v); }
-inline Adj operator/(const Adj& x, const Adj& y) {
-  const double q = x.v / y.v;
-  return adj_node(q, x.id, 1.0 / y.v, y.id, -q / y.v);
-}
-inline Adj operator-(const Adj& x) { return adj_node(-x.v, x.id, -1.0, -1, 0.0); }
-inline bool operator>(const Adj& x, const Adj& y) { return x.v > y.v; }
-inline Adj fabs(const Adj& x) { return adj_node(std::fabs(x.v), x.id, x.v > 0 ? 1.0 : (x.v < 0 ? -1.0 : 0.0), -1, 0.0); }
-inline Adj sqrt(const Adj& x) {
-  const double r = std::sqrt(x.v);
-  return adj_node(r, x.id, 0.5 / r, -1, 0.0);
-}
 
 // reverse sweep: adjoint of every tape entry from the seeds already placed in g
-inline void adj_sweep(std::vector<double>& g) {
-  const Tape& t = tape();
+template <class T>
+inline void adj_sweep(std::vector<T>& g) {
+  const Tape<T>& t = tape<T>();
   for (int i = (int)t.size() - 1; i >= 0; --i) {
-    const double gi = g[i];
+    const T gi = g[i];
     if (gi == 0.0) continue;
     if (t.a[i] >= 0) g[t.a[i]] += t.da[i] * gi;
     if (t.b[i] >= 0) g[t.b[i]] += t.db[i] * gi;
@@ -1100,9 +1107,9 @@ inline Dual sqrt(const Dual& x) {
 
 // Vector-Jacobian product of one stage operator at S with alpha fixed:
 // lam = (dM/dS)^T muM + (dL/dS)^T muL (all arrays in the state layout).
-inline void stage_vjp(const Cfg& c, const double* S, double ax, double ay, const double* muM, const double* muL,
-                      double* lam) {
-  Operator<Adj> op(c);
+template <class T>
+inline void stage_vjp(const Cfg& c, const double* S, double ax, double ay, const double* muM, const double* muL, T* lam) {
+  Operator<Adj<T>> op(c);
   const int m = ncomp(c), nf = nfield(c);
   const int nx = c.nx, ny = c.dim == 2 ? c.ny : 1;
   const size_t plane = (size_t)nx * ny;
@@ -1128,10 +1135,10 @@ inline void stage_vjp(const Cfg& c, const double* S, double ax, double ay, const
   if (c.grav != 0.0)
     for (int f = 0; f < nf; ++f)
       for (size_t p = 0; p < plane; ++p) {
-        lam[((size_t)f * m + 0) * plane + p] += c.grav * muL[((size_t)f * m + 2) * plane + p];
-        lam[((size_t)f * m + 2) * plane + p] += c.grav * muL[((size_t)f * m + 3) * plane + p];
+        lam[((size_t)f * m + 0) * plane + p] += T(c.grav) * muL[((size_t)f * m + 2) * plane + p];
+        lam[((size_t)f * m + 2) * plane + p] += T(c.grav) * muL[((size_t)f * m + 3) * plane + p];
       }
-  std::vector<double> g;
+  std::vector<T> g;
   for (int dir = 0; dir < c.dim; ++dir) {
     const double h = dir == 0 ? c.dx : c.dy;
     const double alpha = dir == 0 ? ax : ay;
@@ -1150,8 +1157,8 @@ inline void stage_vjp(const Cfg& c, const double* S, double ax, double ay, const
       };
       // faces a+1/2: the fluxes enter L of cells a (-1/h) and a+1 (+1/h)
       for (int a = -1; a < nalong; ++a) {
-        tape().clear();
-        Adj Uc[4][4], Dc[4][4], Oc[4][4];
+        tape<T>().clear();
+        Adj<T> Uc[4][4], Dc[4][4], Oc[4][4];
         size_t iu[4][4], id[4][4], io[4][4];
         double su[4][4], sd[4][4], so[4][4];
         for (int q = 0; q < 4; ++q) {
@@ -1160,19 +1167,19 @@ inline void stage_vjp(const Cfg& c, const double* S, double ax, double ay, const
           for (int k = 0; k < m; ++k) {
             su[q][k] = source(0, k, jj, ii, &iu[q][k], &vu);
             sd[q][k] = source(own, k, jj, ii, &id[q][k], &vd);
-            Uc[q][k] = adj_var(vu);
-            Dc[q][k] = adj_var(vd);
+            Uc[q][k] = Adj<T>::var(vu);
+            Dc[q][k] = Adj<T>::var(vd);
             if (c.dim == 2) {
               so[q][k] = source(other, k, jj, ii, &io[q][k], &vo);
-              Oc[q][k] = adj_var(vo);
+              Oc[q][k] = Adj<T>::var(vo);
             }
           }
         }
-        Adj fh[4], hh[4], mx[4];
-        op.face_flux(dir, Uc, Dc, Oc, Adj(alpha), fh, hh, mx);
-        g.assign(tape().size(), 0.0);
+        Adj<T> fh[4], hh[4], mx[4];
+        op.face_flux(dir, Uc, Dc, Oc, Adj<T>(alpha), fh, hh, mx);
+        g.assign(tape<T>().size(), 0.0);
         for (int k = 0; k < m; ++k) {
-          auto nu = [&](int f) { return (mu_at(muL, f, k, a + 1) - mu_at(muL, f, k, a)) / h; };
+          auto nu = [&](int f) { return (T(mu_at(muL, f, k, a + 1)) - mu_at(muL, f, k, a)) / h; };
           if (fh[k].id >= 0) g[fh[k].id] += nu(0);
           if (hh[k].id >= 0) g[hh[k].id] += nu(own);
           if (c.dim == 2 && mx[k].id >= 0) g[mx[k].id] += nu(other);
@@ -1187,8 +1194,8 @@ inline void stage_vjp(const Cfg& c, const double* S, double ax, double ay, const
       }
       // modified derivative of every cell on the line
       for (int a = 0; a < nalong; ++a) {
-        tape().clear();
-        Adj Uc[3][4], Dc[3][4], Dt[4];
+        tape<T>().clear();
+        Adj<T> Uc[3][4], Dc[3][4], Dt[4];
         size_t iu[3][4], id[3][4];
         double su[3][4], sd[3][4];
         for (int q = 0; q < 3; ++q) {
@@ -1197,12 +1204,12 @@ inline void stage_vjp(const Cfg& c, const double* S, double ax, double ay, const
           for (int k = 0; k < m; ++k) {
             su[q][k] = source(0, k, jj, ii, &iu[q][k], &vu);
             sd[q][k] = source(own, k, jj, ii, &id[q][k], &vd);
-            Uc[q][k] = adj_var(vu);
-            Dc[q][k] = adj_var(vd);
+            Uc[q][k] = Adj<T>::var(vu);
+            Dc[q][k] = Adj<T>::var(vd);
           }
         }
         op.modified_derivative(dir, Uc, Dc, Dt);
-        g.assign(tape().size(), 0.0);
+        g.assign(tape<T>().size(), 0.0);
         for (int k = 0; k < m; ++k)
           if (Dt[k].id >= 0) g[Dt[k].id] += mu_at(muM, own, k, a);
         adj_sweep(g);
@@ -1214,7 +1221,7 @@ inline void stage_vjp(const Cfg& c, const double* S, double ax, double ay, const
       }
     }
   }
-  tape().clear();
+  tape<T>().clear();
 }
 
 // Jacobian-vector products of one stage operator at S along delta with alpha fixed.
@@ -1575,6 +1582,16 @@ int oracle_stage_vjp(const oracle_cfg* c, const double* S, double ax, double ay,
                      const double* muL, double* lam) {
   if (check_cfg(c)) return -1;
   hwo::stage_vjp(*c, S, ax, ay, muM, muL, lam);
+  return 0;
+}
+
+// the same in long double, rounded to double once at the end
+int oracle_stage_vjp_ext(const oracle_cfg* c, const double* S, double ax, double ay, const double* muM,
+                         const double* muL, double* lam) {
+  if (check_cfg(c)) return -1;
+  std::vector<long double> l(state_len(c));
+  hwo::stage_vjp(*c, S, ax, ay, muM, muL, l.data());
+  for (size_t p = 0; p < l.size(); ++p) lam[p] = (double)l[p];
   return 0;
 }
 
