@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdint>
@@ -280,6 +281,8 @@ inline Grid grid_of(const hweno_ctx* h) {
   to_pair(g.Gd + 2.0, g.pg.id1);
   g.pg.G = (float)g.G;
   g.pg.Gd = (float)g.Gd;
+  g.pg.hexp = 0;
+  for (int d = 0; d < h->dim; ++d) g.pg.hexp = std::max(g.pg.hexp, std::ilogb(hs[d]));
   g.grav = h->grav;
   for (int sd = 0; sd < 4; ++sd) {
     g.side[sd] = h->side[sd];

@@ -310,6 +310,7 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
                                                   P2 pc2, const PairSlots& sm, const FU& f) {
   constexpr int NC = Traits<DIM, SYS>::NC;
   const long long plane = g.plane;
+  if (SYS == SYS_EULER && !p_units(U[0], U[NC - 1], g.pg.hexp)) return false;
   // FP64: p_0'(x_i) = 3/4 (u_{i+1} - u_{i-1})/h - (v_{i-1} + v_{i+1})/4 and (R2) the derivatives at the two
   // faces; the linear parts of R2's values less the centre value in pairs, which hold them to the last
   // bit of the states where the stencil's differences are small beside these
@@ -370,7 +371,6 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
       const float ir = f_rcp(u_[0]), ie = f_rcp(u_[NC - 1]);
 #pragma unroll
       for (int d = 0; d < DIM; ++d) small = small && p_rel2<NC>(size[d], ir, ie) <= 0x1p-12f;
-      small = small && u_[0] > 0.0f && u_[NC - 1] > 0.0f;
     }
   }
   if (!small) return false;
@@ -784,6 +784,9 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
       if (VAR && fixed[q]) load_fixed<NC, SYS>(g, fside[q], dir, Uq[q], Zq[q]);
     }
     if (PAIR) {
+      if (SYS == SYS_EULER &&
+          !(p_units(Uq[1][0], Uq[1][NC - 1], g.pg.hexp) && p_units(Uq[2][0], Uq[2][NC - 1], g.pg.hexp)))
+        return false;
       double dU[3][NC];
 #pragma unroll
       for (int q = 0; q < 3; ++q)
@@ -901,7 +904,7 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
       hdif[k] = p_mul(h, p_from(fu.sub(Dp[k], Dm[k])));
       size[k] = p_from(Ds[k]).h * h.h;
     }
-    if (p_flux_pair<NC>(Us, Ds, dif, hdif, size, alpha, ih, g.pg, fu, vf, vh)) {
+    if (p_units(Us[0], Us[NC - 1], g.pg.hexp) && p_flux_pair<NC>(Us, Ds, dif, hdif, size, alpha, ih, g.pg, fu, vf, vh)) {
       Phys<DIM, SYS>::flux_jvp(Us, Ds, FS, HS, a_adv, g.gm1, fu);
       summed = true;
     }

@@ -30,9 +30,11 @@ struct Traits {
 };
 
 // Constants of the pair arithmetic (hweno_pair.cuh), each as hi + lo of two FP32 numbers: the mesh
-// sizes and their inverses, gamma - 1, eps, 1/gamma1 and 1/d1; G = gamma0/gamma1, Gd = d0/d1.
+// sizes and their inverses, gamma - 1, eps, 1/gamma1 and 1/d1; G = gamma0/gamma1, Gd = d0/d1; hexp: the
+// exponent of the larger mesh size, not below 0 (p_units).
 struct PairGrid {
   float h[2][2], ih[2][2], gm1[2], eps[2], ig1[2], id1[2], G, Gd;
+  int hexp;
 };
 
 // Parameters shared by all kernels of one grid.

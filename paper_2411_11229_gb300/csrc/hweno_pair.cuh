@@ -552,13 +552,24 @@ __device__ __forceinline__ bool p_cell(const PairSlots& sm, const EigP<NC, F2>& 
 }
 
 // The square of a change's size beside a state with 1/rho = ir and 1/E = ie (the momentum's beside
-// sqrt(rho E))
+// sqrt(rho E)); each factor beside the state, so that no square leaves the FP32 range before it is compared
 template <int NC>
 __device__ __forceinline__ float p_rel2(const float* x, float ir, float ie) {
   const float a = x[0] * ir, b = x[NC - 1] * ie;
-  float m2 = x[1] * x[1];
-  if (NC == 4) m2 += x[2] * x[2];
-  return fmaxf(fmaxf(a * a, b * b), m2 * ir * ie);
+  float m2 = (x[1] * ir) * (x[1] * ie);
+  if (NC == 4) m2 += (x[2] * ir) * (x[2] * ie);
+  return fmaxf(fmaxf(a * a, b * b), m2);
+}
+
+// Whether pairs hold an Euler state with density rho and energy E, its fluxes and their derivatives on the
+// mesh to the last bit: what d_from leaves out is below 2^-126, and has to stay below 2^-53 (here
+// 2^-62) of the smallest of rho, E, rho c, E c and of these over h (rho c^2 ~ E); the upper bounds keep
+// 1/rho^2 and the products of p_flux_pair inside FP32.  Not true for rho <= 0, E <= 0, infinities and NaN.
+// On the exponents, in the integer pipe (hexp: the larger mesh size's, not below 0).
+__device__ __forceinline__ bool p_units(double rho, double E, int hexp) {
+  const int a = (__double2hiint(rho) >> 20) - 1023, b = (__double2hiint(E) >> 20) - 1023;
+  const int low = min(min(2 * a, 2 * b), min(a + b, 3 * b - a));
+  return a >= -50 && a <= 40 && b >= -50 && b <= 60 && b - a >= -40 && b - a <= 60 && low - 2 * hexp >= -128;
 }
 
 // The Lax-Friedrichs flux of an Euler face whose two states are close, from the sums U = U^- + U^+,
