@@ -581,7 +581,8 @@ __device__ __forceinline__ bool p_units(double rho, double E, int hexp) {
 // carries them; where the differences are larger, or where the pairs' noise in them (2^-48 of size,
 // what they were formed from) would show beside the rounding of the states, the FP64 code takes both
 // states.
-// Returns vf and vh: minus half of alpha times the differences plus half of q and q'.
+// Returns vf and vh: minus half of alpha times the differences plus half of q and q'; false where any of
+// these is not held by FP32.
 template <int NC>
 __device__ __forceinline__ bool p_flux_pair(const double* U, const double* D, const P2* dif, const P2* hdif,
                                             const float* size, double alpha, P2 ih, const PairGrid& pg, const FU& f,
@@ -602,7 +603,7 @@ __device__ __forceinline__ bool p_flux_pair(const double* U, const double* D, co
   }
   // q is below 2^-32 of the fluxes, q' of the derivatives' fluxes
   const float r2 = p_rel2<NC>(r, ir, ie), d2 = p_rel2<NC>(size, ir, ie);
-  if (!(r2 <= 0x1p-34f && d2 <= 0x1p-12f && r2 * p_rel2<NC>(s, ir, ie) <= 0x1p-64f * d2 && rho > 0.0f && u_[E] > 0.0f)) return false;
+  if (!(r2 <= 0x1p-34f && d2 <= 0x1p-12f && r2 * p_rel2<NC>(s, ir, ie) <= 0x1p-64f * d2)) return false;
 #pragma unroll
   for (int k = 0; k < NC; ++k) s[k] *= ih.h;
   // first-order changes of the velocities and of the pressure, second-order ones, and their
@@ -640,15 +641,18 @@ __device__ __forceinline__ bool p_flux_pair(const double* U, const double* D, co
   q[E] = (r[E] + p1) * du - hp * a * ir + p2 * u;
   t[E] = (s[E] + p1t) * du + (r[E] + p1) * dut - (hpt * a + hp * at) * ir - hp * a * irt + p2t * u + p2 * ut;
   const P2 ma = p_scale(p_from(alpha), -0.5f);
+  // an alpha outside the FP32 range (a NaN here, which d_from would make a number), or a product with it
+  float big = fabsf(ma.h);
 #pragma unroll
   for (int k = 0; k < NC; ++k) {
     P2 x = p_mul(ma, dif[k]), y = p_mul(p_mul(ma, hdif[k]), ih);
     x.l += 0.5f * q[k];
     y.l += 0.5f * t[k];
+    big = f_add(big, f_add(f_add(fabsf(x.h), fabsf(x.l)), f_add(fabsf(y.h), fabsf(y.l))));
     vf[k] = f.add(d_from(x.h), d_from(x.l));
     vh[k] = f.add(d_from(y.h), d_from(y.l));
   }
-  return true;
+  return big < kPairMax;
 }
 
 }  // namespace hw

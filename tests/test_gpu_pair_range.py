@@ -61,3 +61,18 @@ def test_euler_units(rho, vel, kind, nx, ny, flags):
     S, dx, dy = _flow(nx, ny, kind)
     S = S * (rho * np.array([1.0, vel, vel, vel * vel])).reshape(1, 4, 1, 1)
     _check(O.make_cfg(2, O.EULER, nx, ny, dx=dx, dy=dy, flags=flags), S, flags=flags)
+
+
+@pytest.mark.parametrize("flags", [0, O.FLAG_R2])
+@pytest.mark.parametrize("nx,ny", SIZES)
+@pytest.mark.parametrize("energy", [1e30, 1e70, 1e80, 1e160])
+def test_one_cell_of_any_wavespeed(energy, nx, ny, flags):
+    """A smooth flow but for one cell whose wavespeed (the Lax-Friedrichs coefficient of every face) goes
+    through the end of the FP32 range: the cells out of its reach, where the dissipation is that
+    coefficient times the small jumps of a smooth flow."""
+    S, dx, dy = _flow(nx, ny, "smooth")
+    S[0, 3, ny // 2, nx // 2] = energy
+    far = np.ones((ny, nx), bool)
+    far[ny // 2 - 4: ny // 2 + 5, :] = False
+    far[:, nx // 2 - 4: nx // 2 + 5] = False
+    _check(O.make_cfg(2, O.EULER, nx, ny, dx=dx, dy=dy, flags=flags), S, far, flags=flags)
