@@ -1160,7 +1160,7 @@ int stage_vjp(const hweno_ctx* h, const Grid& g, const double* S, const double* 
             cudaSuccess)
       return HWENO_ECUDA;
     hw::AdjWork fw = aw;
-    if (g.plane >= kAdjPairMinCells) {
+    if (g.plane >= kAdjPairMinCells && pair_mesh(h)) {
       if (cudaMemsetAsync(aw.count, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) return HWENO_ECUDA;
       hw::k_adj_cell_pair<<<bc, hw::kThreads, pair_sm, st>>>(g, S, muM, aw);
       hw::k_adj_face_pair<<<dim3(bf, 2), hw::kThreads, pair_sm, st>>>(g, S, muL, aw, alpha2);

@@ -464,7 +464,7 @@ int hweno_batch_bind(hweno_batch_t* b, double* state_dev, void* ws) {
     h.w.alpha = b->alpha + 2 * i;
     h.w.astride = 2 * b->n;
     hi[i].g = grid_of(&h);
-    hi[i].g.pairs = 1;  // many instances share the FP64 pipe
+    hi[i].g.pairs = pair_mesh(&h);  // many instances share the FP64 pipe
     hi[i].w = h.w;
     hi[i].S = h.state;
     hi[i].dim = h.dim;

@@ -136,7 +136,13 @@ constexpr long long kLineMaxCells = hw::kSMs * (hw::kThreads - 4LL);
 // 62 and 74 us (with fronts 60 and 82), at 96x170 84 and 80 (83 and 98), at 128x200 123 and 88 (123 and
 // 111).  A scalar law's chain is short: at 182x181 40 and 46 us, at 256^2 58 and 48.
 constexpr long long kPairMinCells = hw::kSMs * 4LL * 32;
+// Mesh sizes whose pairs (and those of their inverses and of the derivatives on them) have all of their 48
+// bits inside the FP32 range: 2^-64 to 2^64.  At 1e-36 the second half of h is an FP32 denormal.
+inline bool pair_mesh(const hweno_ctx* h) {
+  return std::abs(std::ilogb(h->dx)) <= 64 && (h->dim == 1 || std::abs(std::ilogb(h->dy)) <= 64);
+}
 inline int pairs_of(const hweno_ctx* h) {
+  if (!pair_mesh(h)) return 0;
   if (h->dim == 1) return h->nx > kLineMaxCells;
   return (long long)h->nx * h->ny > kPairMinCells * (h->system == hw::SYS_EULER ? 1 : 2);
 }

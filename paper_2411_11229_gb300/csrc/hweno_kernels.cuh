@@ -891,7 +891,7 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
         r1_face_states<NC, SYS, false>(Uq, Zq, e, g, dir, Um, Up, Dm, Dp, fu);
     }
   }
-  if (VAR == 2) {
+  if (VAR == 2 && g.pairs) {
     double Us[NC], Ds[NC];
     P2 dif[NC], hdif[NC];
     float size[NC];

@@ -65,6 +65,17 @@ def test_euler_units(rho, vel, kind, nx, ny, flags):
 
 @pytest.mark.parametrize("flags", [0, O.FLAG_R2])
 @pytest.mark.parametrize("nx,ny", SIZES)
+@pytest.mark.parametrize("length", [1e-36, 1e-30, 1e-20, 1e-9, 1e9, 1e20, 1e30, 1e36])
+def test_mesh_sizes(length, nx, ny, flags):
+    """The same flow on a domain scaled by length."""
+    S, dx, dy = _flow(nx, ny, "smooth")
+    S[1:] /= length
+    cfg = O.make_cfg(2, O.EULER, nx, ny, dx=dx * length, dy=dy * length, flags=flags)
+    _check(cfg, S, flags=flags)
+
+
+@pytest.mark.parametrize("flags", [0, O.FLAG_R2])
+@pytest.mark.parametrize("nx,ny", SIZES)
 @pytest.mark.parametrize("energy", [1e30, 1e70, 1e80, 1e160])
 def test_one_cell_of_any_wavespeed(energy, nx, ny, flags):
     """A smooth flow but for one cell whose wavespeed (the Lax-Friedrichs coefficient of every face) goes
