@@ -440,6 +440,7 @@ __device__ __forceinline__ bool adj_cell_pair(const Grid& g, const double* __res
     double Uc[NC];
 #pragma unroll
     for (int k = 0; k < NC; ++k) Uc[k] = S[k * plane + p];
+    if (!p_units(Uc[0], Uc[NC - 1], g.pg.hexp)) return false;
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
       const int n = d == 0 ? g.nx : g.ny, a0 = d == 0 ? i : j, fld = d == 0 ? 1 : 2;
@@ -634,6 +635,7 @@ __device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __res
       mirror_U<NC>(U[q], refl[q]);
       mirror_D<NC>(Z[q], refl[q]);
     }
+    if (!(p_units(U[1][0], U[1][NC - 1], g.pg.hexp) && p_units(U[2][0], U[2][NC - 1], g.pg.hexp))) return false;
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
       const double a = fu.sub(U[1][k], U[0][k]), b = fu.sub(U[2][k], U[1][k]), c = fu.sub(U[3][k], U[2][k]);
