@@ -1133,7 +1133,7 @@ AdjPtrs adj_ptrs(const hweno_ctx* h, void* ws) {
 constexpr long long kAdjPairMinCells = hw::kSMs * 4LL * 32 / 2;
 
 template <int DIM>
-int stage_vjp(const hweno_ctx* h, const Grid& g, const double* S, const double* alpha2, const double* muM,
+int stage_vjp(hweno_ctx* h, const Grid& g, const double* S, const double* alpha2, const double* muM,
               const double* muL, const hw::AdjWork& aw, double* lam) {
   const cudaStream_t st = h->stream;
   const unsigned bc = blocks_for(g.plane);
@@ -1166,6 +1166,7 @@ int stage_vjp(const hweno_ctx* h, const Grid& g, const double* S, const double* 
       if (cudaMemsetAsync(aw.count, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) return HWENO_ECUDA;
       hw::k_adj_cell_pair<<<bc, hw::kThreads, pair_sm, st>>>(g, S, muM, aw);
       hw::k_adj_face_pair<<<dim3(bf, 2), hw::kThreads, pair_sm, st>>>(g, S, muL, aw, alpha2);
+      h->launches += 2;
     } else {
       fw.cells = fw.faces = nullptr;
     }
@@ -1173,6 +1174,7 @@ int stage_vjp(const hweno_ctx* h, const Grid& g, const double* S, const double* 
     hw::k_adj_face<DIM><<<bl < 2 * bf ? bl : 2 * bf, hw::kThreads, face_sm, st>>>(g, S, muL, fw, alpha2);
   }
   hw::k_adj_gather<DIM><<<bc, hw::kThreads, 0, st>>>(g, S, muM, muL, aw, lam);
+  h->launches += 3;
   return cudaGetLastError() == cudaSuccess ? HWENO_OK : HWENO_ECUDA;
 }
 
@@ -1208,7 +1210,7 @@ int adjoint_from_stages(hweno_t* h, const AdjPtrs& a, const double* Sn, const do
   hw::k_rk_first<<<rk_blocks(h), 256, 0, h->stream>>>(rk_n(h), a.muM, a.muL, dt, a.lam1, a.lamB);
   if ((rc = launch_status())) return rc;
   if ((rc = vjp(Sn, 0, a.muM, a.muL, lam_out))) return rc;
-  h->launches += (h->dim == 1 ? 9 : 15) + 3;
+  h->launches += 3;
   return HWENO_OK;
 }
 
@@ -1298,7 +1300,6 @@ int hweno_stage_vjp(hweno_t* h, const double* S, const double* alpha2, const dou
   if ((uintptr_t)adj_ws & 255) return HWENO_EINVAL;
   const AdjPtrs a = adj_ptrs(h, adj_ws);
   const Grid g = grid_of(h);
-  h->launches += h->dim == 1 ? 3 : 5;
   return h->dim == 1 ? stage_vjp<1>(h, g, S, alpha2, muM, muL, a.aw, lam)
                      : stage_vjp<2>(h, g, S, alpha2, muM, muL, a.aw, lam);
 }

@@ -1,7 +1,8 @@
 """The stage VJP against the exact value of the adjoint formulas (the oracle's reverse mode in long double),
 on both sides of the size from which a 2D VJP takes the nonlinear part in pairs (9728 cells): per plane no
 further from it than three times the FP64 oracle plus 1e-14, the bars of the extended-precision tests.
-Also gradients of 1D rollouts from checkpoints and from kept stage inputs."""
+Also the number of kernels that a VJP launches, and gradients of 1D rollouts from checkpoints and from
+kept stage inputs."""
 import ctypes
 
 import numpy as np
@@ -62,6 +63,30 @@ def test_stage_vjp(nx, ny, amp, units, par):
     scale = np.abs(ref).max(axis=1)
     err, own = np.abs(got - ref).max(axis=1) / scale, np.abs(own - ref).max(axis=1) / scale
     assert (err <= 3.0 * own + 1e-14).all(), (err, own)
+
+
+@pytest.mark.parametrize("dim,nx,ny,kernels", [(1, 300, 1, 3), (2, 40, 33, 3), (2, 97, 100, 3), (2, 128, 76, 5),
+                                               (2, 101, 97, 5)])
+def test_launch_counts(dim, nx, ny, kernels):
+    """Three kernels a VJP; five where the pairs' kernels come before those of their lists (from 9728
+    cells).  A step's adjoint is three VJPs and three passes over the state."""
+    if dim == 2:
+        S, dx, dy = W.euler2d_random(nx, ny, seed=1, kind="smooth")
+    else:
+        S, dx = W.euler1d_random(nx, seed=1, kind="smooth")
+        dy = dx
+    s = Solver(dim, "euler", nx, ny, dx=dx, dy=dy)
+    s.set_state(S)
+    r = np.random.default_rng(0)
+    n0 = s.launch_count()
+    _vjp(s, S, (2.0, 2.0), r.normal(size=S.shape), r.normal(size=S.shape))
+    n1 = s.launch_count()
+    assert n1 - n0 == kernels
+    Sd = s.state.clone()
+    al = torch.full((6,), 2.0, dtype=torch.float64, device="cuda")
+    s.adjoint_step_stages(Sd, Sd, Sd, 1e-4, al, torch.ones_like(Sd))
+    assert s.launch_count() - n1 == 3 * kernels + 3
+    torch.cuda.synchronize()
 
 
 # four warps to a block's cells, one block; 152 blocks; a thread to a cell; stage kernels
