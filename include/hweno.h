@@ -274,7 +274,9 @@ int hweno_step_replay(hweno_t *h, double dt, const double *alpha6_dev);
  * and adj_ws_dev (hweno_adjoint_workspace_bytes, 256-byte aligned).  S_n, lam_in and lam_out must
  * not alias each other.  All three boundary types of hweno_create (a reflective wall reads its
  * mirrored neighbours through the sign tables, and their adjoints go back through the same
- * tables).  EINVAL for scalar systems, handles of hweno_create_ex with extensions, or dt <= 0. */
+ * tables).  EINVAL for scalar systems, handles of hweno_create_ex with extensions, or dt <= 0; ESTATE:
+ * no workspace bound (so for hweno_adjoint_step_stages and hweno_stage_vjp: their kernels read its
+ * scalars). */
 int hweno_adjoint_step(hweno_t *h, const double *S_n_dev, double dt, const double *alpha6_dev,
                        const double *lam_in_dev, double *lam_out_dev, void *adj_ws_dev);
 

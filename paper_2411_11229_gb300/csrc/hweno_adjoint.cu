@@ -1241,6 +1241,7 @@ int hweno_adjoint_step_stages(hweno_t* h, const double* Sn, const double* S1, co
   if (!h || !Sn || !S1 || !S2 || !alpha6 || !lam_in || !lam_out || !adj_ws) return HWENO_EINVAL;
   if (h->system != HWENO_EULER || h->var != 0) return HWENO_EINVAL;
   if (!(dt > 0.0) || ((uintptr_t)adj_ws & 255)) return HWENO_EINVAL;
+  if (!h->ws) return HWENO_ESTATE;  // the kernels read the bound workspace's scalars
   return adjoint_from_stages(h, adj_ptrs(h, adj_ws), Sn, S1, S2, dt, alpha6, lam_in, lam_out);
 }
 
@@ -1298,6 +1299,7 @@ int hweno_stage_vjp(hweno_t* h, const double* S, const double* alpha2, const dou
   if (!h || !S || !alpha2 || !muM || !muL || !lam || !adj_ws) return HWENO_EINVAL;
   if (h->system != HWENO_EULER || h->var != 0) return HWENO_EINVAL;
   if ((uintptr_t)adj_ws & 255) return HWENO_EINVAL;
+  if (!h->ws) return HWENO_ESTATE;
   const AdjPtrs a = adj_ptrs(h, adj_ws);
   const Grid g = grid_of(h);
   return h->dim == 1 ? stage_vjp<1>(h, g, S, alpha2, muM, muL, a.aw, lam)
