@@ -159,6 +159,9 @@ inline int listed_of(const hweno_ctx* h) {
          nfaces_of(h) < (size_t(1) << 32);
 }
 
+// Words of Work::alpha: four slots of two directions, then what hweno_line.cu keeps behind them
+constexpr int kAlphaWords = 8 + 9;
+
 inline Layout layout_of(const hweno_ctx* h) {
   const size_t plane = (size_t)h->nx * h->ny;
   const size_t nc = nc_of(h), nf = nf_of(h);
@@ -169,7 +172,7 @@ inline Layout layout_of(const hweno_ctx* h) {
   l.PRIM = align_up((size_t)np_of(h) * plane * 8 + 8);
   l.FX = align_up(nf * nc * (size_t)h->ny * (h->nx + 1) * 8);
   l.FY = h->dim == 2 ? align_up(nf * nc * (size_t)(h->ny + 1) * h->nx * 8) : 0;
-  l.alpha = align_up(8 * 8);
+  l.alpha = align_up(kAlphaWords * 8);
   l.scal = align_up(8 * 8);
   l.status = align_up(16);
   l.FS = h->var == 2 ? align_up((size_t)h->dim * 4 * nc * plane * 8) : 0;

@@ -31,6 +31,7 @@ namespace hw {
 // alpha[0..7]: [8] the number of launches, [9 + 4 set + slot] the slots of a set, all zero between
 // launches of that set
 constexpr int kLineToggle = 8, kLineSlots = 9;
+static_assert(kLineSlots + 2 * 4 <= hwh::kAlphaWords, "the layout holds both sets");
 
 struct LineArgs {
   int nsteps;
