@@ -49,7 +49,7 @@ __device__ __forceinline__ void batch_cells(const BatchInst& I, long long p0, in
   double wsx = 0.0, wsy = 0.0;
   for (int t = 0; t < tpi; ++t) {
     double a = 0.0, b = 0.0;
-    cell_tile<DIM, SYS_EULER, 0, false>(I.g, I.S, I.w, p0 + (long long)t * kThreads, a, b, lo, sm,
+    cell_tile<DIM, SYS_EULER, 0, MODE_BLOCK>(I.g, I.S, I.w, p0 + (long long)t * kThreads, a, b, lo, sm,
                                  true);
     wsx = speed_bits(a) > speed_bits(wsx) ? a : wsx;
     wsy = speed_bits(b) > speed_bits(wsy) ? b : wsy;
@@ -64,7 +64,7 @@ __device__ __forceinline__ void batch_faces(const BatchInst& I, int dir, long lo
   const long long nf = dir == 0 ? (long long)(I.g.nx + 1) * I.g.ny : (long long)(I.g.ny + 1) * I.g.nx;
   const double alpha = __longlong_as_double((long long)I.w.alpha[slot * I.w.astride + dir]);
   for (int t = 0; t < tpi; ++t)
-    face_tile<DIM, SYS_EULER, 0, false>(I.g, I.S, I.w, dir, f0 + (long long)t * kThreads, nf, alpha, lo,
+    face_tile<DIM, SYS_EULER, 0, MODE_BLOCK>(I.g, I.S, I.w, dir, f0 + (long long)t * kThreads, nf, alpha, lo,
                                  sm, true);
 }
 
@@ -464,7 +464,7 @@ int hweno_batch_bind(hweno_batch_t* b, double* state_dev, void* ws) {
     h.w.alpha = b->alpha + 2 * i;
     h.w.astride = 2 * b->n;
     hi[i].g = grid_of(&h);
-    hi[i].g.pairs = pair_mesh(&h);  // many instances share the FP64 pipe
+    hi[i].g.pairs = hi[i].g.face_pairs = pair_mesh(&h);  // many instances share the FP64 pipe
     hi[i].w = h.w;
     hi[i].S = h.state;
     hi[i].dim = h.dim;

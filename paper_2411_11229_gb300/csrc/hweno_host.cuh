@@ -34,11 +34,14 @@ inline unsigned blocks_for(long long n) { return (unsigned)((n + hw::kThreads - 
 template <int DIM, int SYS, int VAR>
 struct L {
   static void cell(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
-    if (DIM == 2 && g.listed) {
-      hw::k_cell<2, SYS, VAR, true><<<blocks_for(g.plane), hw::kThreads, 0, st>>>(g, S, w, slot);
+    const unsigned nb = blocks_for(g.plane);
+    if (!g.pairs) {
+      hw::k_cell<DIM, SYS, VAR, hw::MODE_FP64><<<nb, hw::kThreads, 0, st>>>(g, S, w, slot);
+    } else if (DIM == 2 && g.listed) {
+      hw::k_cell<2, SYS, VAR, hw::MODE_LISTED><<<nb, hw::kThreads, 0, st>>>(g, S, w, slot);
       if (VAR == 2) left(g, S, w, slot, st);  // R2's faces need what is left of the cells
     } else {
-      hw::k_cell<DIM, SYS, VAR, false><<<blocks_for(g.plane), hw::kThreads, 0, st>>>(g, S, w, slot);
+      hw::k_cell<DIM, SYS, VAR, hw::MODE_BLOCK><<<nb, hw::kThreads, 0, st>>>(g, S, w, slot);
     }
   }
   static void left(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
@@ -47,12 +50,14 @@ struct L {
   static void face(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
     const long long nfx = (long long)(g.nx + 1) * g.ny;
     const long long nfy = DIM == 2 ? (long long)(g.ny + 1) * g.nx : 0;
-    dim3 grid(blocks_for(nfx > nfy ? nfx : nfy), DIM);
-    if (DIM == 2 && VAR != 2 && g.listed) {
-      hw::k_face<2, SYS, VAR, true><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
+    const dim3 grid(blocks_for(nfx > nfy ? nfx : nfy), DIM);
+    if (!g.face_pairs) {
+      hw::k_face<DIM, SYS, VAR, hw::MODE_FP64><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
+    } else if (DIM == 2 && VAR != 2 && g.listed) {
+      hw::k_face<2, SYS, VAR, hw::MODE_LISTED><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
       left(g, S, w, slot, st);
     } else {
-      hw::k_face<DIM, SYS, VAR, false><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
+      hw::k_face<DIM, SYS, VAR, hw::MODE_BLOCK><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
     }
   }
   static void update(const Grid& g, double* S, const Work& w, int mode, int stage, double a, double b,
@@ -195,7 +200,10 @@ inline Grid grid_of(const hweno_ctx* h) {
   g.ny = (int)h->ny;
   g.bc = h->bc;
   g.flags = h->flags;
-  g.pairs = pairs_of(h);
+  // the weighted derivative needs the weights themselves, in R2's cells or in the other schemes' faces
+  const bool vw = (h->flags & HWENO_FLAG_V_WEIGHTED) != 0, r2 = h->var == 2;
+  g.pairs = pairs_of(h) && !(vw && r2);
+  g.face_pairs = pairs_of(h) && !(vw && !r2);
   g.listed = listed_of(h);
   g.plane = (long long)h->nx * h->ny;
   g.dx = h->dx;

@@ -34,8 +34,8 @@ struct Work {
   double* B;     // stage base M(S^n): [NF][NC][plane]
   double* MD;    // modified derivatives (V~, W~): [DIM][NC][plane]
   double* NOD;   // nodal values per direction, normal frame: [DIM][NG][NC][plane]
-  float2* PRIM;  // Euler primitives (sqrt(rho), u[, v], H) as pairs (hweno_pair.cuh): [NP][plane]; grids
-                 // that take no pairs (Grid::pairs) keep them in FP64 in the same bytes
+  float2* PRIM;  // Euler primitives (sqrt(rho), u[, v], H): [NP][plane], as pairs (hweno_pair.cuh) where the
+                 // faces take pairs (Grid::face_pairs), else in FP64 in the same bytes
   double* FX;    // x-face fluxes, original frame: [NF][NC][ny][nx+1]
   double* FY;    // y-face fluxes: [NF][NC][ny+1][nx]
   unsigned long long* alpha;  // wavespeed slots (bit patterns of non-negative doubles): slot s of
@@ -262,28 +262,51 @@ __device__ __forceinline__ void r2_cell(const double (&U3)[3][NC], const double 
     r2_cell_vw<NC, SYS, false>(U3, D3, e, dir, g, md, fs, f);
 }
 
-// The modified derivative of cell p in direction d (and, for R2, the cell's face states) with the
-// FP64 weights: the cells that cell_body leaves to it.
+// Velocities, pressure, 1/rho of a cell, and its wavespeeds per direction; ROOT: 1/c as well (the FP64
+// weights' fields need both, and one chain of instructions gives both)
+template <int DIM, int SYS, bool ROOT>
+struct CellState {
+  double u = 0.0, v = 0.0, pr = 0.0, ir = 0.0, c = 0.0, ic = 0.0;
+  // returns whether the state is physical
+  __device__ __forceinline__ bool set(const double* U, const Grid& g, const FU& f, double& wsx, double& wsy) {
+    constexpr int NC = Traits<DIM, SYS>::NC;
+    if (SYS == SYS_EULER) {
+      ir = rcp(U[0], f);
+      u = f.mul(U[1], ir);
+      if (DIM == 2) v = f.mul(U[2], ir);
+      const double ke = DIM == 2 ? fma(U[1], u, f.mul(U[2], v)) : f.mul(U[1], u);
+      pr = g.gm1 * fma(-0.5, ke, U[NC - 1]);
+      const double c2 = f.mul(g.gamma * pr, ir);
+      if (ROOT) ic = rsqrt_fast(c2, f);
+      c = ROOT ? f.mul(c2, ic) : sqrt_fast(c2, f);
+      wsx = f.add(fabs(u), c);
+      wsy = DIM == 2 ? f.add(fabs(v), c) : 0.0;
+      return positive_bits(U[0]) && positive_bits(pr) && finite_bits(wsx) && finite_bits(wsy);
+    }
+    if (SYS == SYS_BURGERS) {
+      wsx = fabs(U[0]);
+      wsy = DIM == 2 ? wsx : 0.0;
+      return finite_bits(wsx);
+    }
+    wsx = fabs(g.ax);
+    wsy = DIM == 2 ? fabs(g.ay) : 0.0;
+    return true;
+  }
+};
+
+// The modified derivative of cell p in direction d (and, for R2, the cell's face states) with the FP64
+// weights, from the cell's state U and what CellState holds of it.
 template <int DIM, int SYS, int VAR>
-__device__ __forceinline__ void cell_limiter(const Grid& g, const double* __restrict__ S, const Work& w, long long p,
-                                             int d) {
+__device__ __forceinline__ void cell_limiter_of(const Grid& g, const double* __restrict__ S, const Work& w, long long p,
+                                                int i, int j, int d, const double* U, const CellState<DIM, SYS, true>& c,
+                                                const FU& f) {
   constexpr int NC = Traits<DIM, SYS>::NC;
   const long long plane = g.plane;
-  const FU f = fu_of(w.scal);
-  const int i = (int)(p % g.nx), j = (int)(p / g.nx);
   double U3[3][NC], D3[3][NC];
-  load_stencil3<DIM, SYS, VAR, NC>(g, S, d, i, j, d == 0 ? i : j, nullptr, U3, D3);
+  load_stencil3<DIM, SYS, VAR, NC>(g, S, d, i, j, d == 0 ? i : j, U, U3, D3);
   Eig<NC> e;
-  if (SYS == SYS_EULER) {
-    const double* U = U3[1];
-    const double ir = rcp(U[0], f);
-    const double u = f.mul(U[1], ir), v = NC == 4 ? f.mul(U[2], ir) : 0.0;
-    const double ke = NC == 4 ? fma(U[1], u, f.mul(U[2], v)) : f.mul(U[1], u);
-    const double pr = g.gm1 * fma(-0.5, ke, U[NC - 1]);
-    const double c2 = f.mul(g.gamma * pr, ir);
-    const double ic = rsqrt_fast(c2, f);
-    e.setup(u, v, f.mul(f.add(U[NC - 1], pr), ir), f.mul(c2, ic), ic, g.gm1);
-  }
+  if (SYS == SYS_EULER)
+    e.setup(d == 0 ? c.u : c.v, d == 0 ? c.v : c.u, f.mul(f.add(U[NC - 1], c.pr), c.ir), c.c, c.ic, g.gm1);
   double out[NC];
   if (VAR == 2) {
     double fs[4][NC];
@@ -299,6 +322,20 @@ __device__ __forceinline__ void cell_limiter(const Grid& g, const double* __rest
   if (SYS == SYS_EULER && d == 1) swap_frame<NC>(out);
 #pragma unroll
   for (int k = 0; k < NC; ++k) w.MD[((long long)d * NC + k) * plane + p] = out[k];
+}
+
+// The same from the cell alone: the cells that the pairs leave to the FP64 weights.
+template <int DIM, int SYS, int VAR>
+__device__ __forceinline__ void cell_limiter(const Grid& g, const double* __restrict__ S, const Work& w, long long p,
+                                             int d) {
+  constexpr int NC = Traits<DIM, SYS>::NC;
+  const FU f = fu_of(w.scal);
+  double U[NC], wx, wy;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) U[k] = S[k * g.plane + p];
+  CellState<DIM, SYS, true> c;
+  c.set(U, g, f, wx, wy);
+  cell_limiter_of<DIM, SYS, VAR>(g, S, w, p, (int)(p % g.nx), (int)(p / g.nx), d, U, c, f);
 }
 
 // The same in every direction with the nonlinear part in pairs (hweno_pair.cuh): U, pu, pv, pH, pc2 the
@@ -411,39 +448,14 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
   return true;
 }
 
-// Velocities, pressure, 1/rho of a cell, and its wavespeeds per direction
-template <int DIM, int SYS>
-struct CellState {
-  double u = 0.0, v = 0.0, pr = 0.0, ir = 0.0;
-  // returns whether the state is physical
-  __device__ __forceinline__ bool set(const double* U, const Grid& g, const FU& f, double& wsx, double& wsy) {
-    constexpr int NC = Traits<DIM, SYS>::NC;
-    if (SYS == SYS_EULER) {
-      ir = rcp(U[0], f);
-      u = f.mul(U[1], ir);
-      if (DIM == 2) v = f.mul(U[2], ir);
-      const double ke = DIM == 2 ? fma(U[1], u, f.mul(U[2], v)) : f.mul(U[1], u);
-      pr = g.gm1 * fma(-0.5, ke, U[NC - 1]);
-      const double c = sqrt_fast(f.mul(g.gamma * pr, ir), f);
-      wsx = f.add(fabs(u), c);
-      wsy = DIM == 2 ? f.add(fabs(v), c) : 0.0;
-      return positive_bits(U[0]) && positive_bits(pr) && finite_bits(wsx) && finite_bits(wsy);
-    }
-    if (SYS == SYS_BURGERS) {
-      wsx = fabs(U[0]);
-      wsy = DIM == 2 ? wsx : 0.0;
-      return finite_bits(wsx);
-    }
-    wsx = fabs(g.ax);
-    wsy = DIM == 2 ? fabs(g.ay) : 0.0;
-    return true;
-  }
-};
+// How a kernel takes the nonlinear part of the interpolation: all of it with the FP64 weights; or in pairs,
+// with what the pairs leave to the FP64 weights taken block by block or listed for k_left.
+enum { MODE_FP64 = 0, MODE_BLOCK = 1, MODE_LISTED = 2 };
 
 // Cell work of one stage at cell p: wavespeeds (returned in wsx, wsy), primitives, nodal values per
-// direction, modified derivatives (and, for R2, the face states of the cell).  Returns
-// false where the modified derivatives are left to cell_limiter.
-template <int DIM, int SYS, int VAR = 0>
+// direction and, LIMITER, modified derivatives (and, for R2, the face states of the cell).  Returns
+// false where the modified derivatives are left to cell_limiter (PAIRS).
+template <int DIM, int SYS, int VAR, bool PAIRS, bool LIMITER>
 __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restrict__ S, const Work& w, long long p,
                                           double& wsx, double& wsy, const PairSlots& sm) {
   using T = Traits<DIM, SYS>;
@@ -460,7 +472,7 @@ __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restric
       if (DIM == 2) Wd[k] = S[(2 * NC + k) * plane + p];
     }
     // primitives and wavespeeds
-    CellState<DIM, SYS> c;
+    CellState<DIM, SYS, !PAIRS> c;
     if (!c.set(U, g, f, wsx, wsy)) atomicOr(w.status, 1u);
     const double u = c.u, v = c.v, pr = c.pr, ir = c.ir;
     if (VAR && (g.flags & FLAG_ALPHA_LOCAL)) {
@@ -519,19 +531,20 @@ __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restric
         if (DIM == 2) nod[(2 * NC + k) * plane + p] = Mx[k];
       }
     }
-    // modified derivatives (Eq. limiter), one per direction; the weighted derivative of R2 needs the
-    // weights themselves
-    if (!g.pairs) {
-      if (SYS == SYS_EULER && VAR != 2) {
-        double* P = reinterpret_cast<double*>(w.PRIM);
-        P[p] = sqrt_fast(U[0], f);
-        P[plane + p] = u;
-        if (DIM == 2) P[2 * plane + p] = v;
-        P[DIM * plane + plane + p] = f.mul(f.add(U[NC - 1], pr), ir);
-      }
-      return false;
+    if (SYS == SYS_EULER && VAR != 2 && !(PAIRS && (VAR == 0 || g.face_pairs))) {
+      double* P = reinterpret_cast<double*>(w.PRIM);
+      P[p] = sqrt_fast(U[0], f);
+      P[plane + p] = u;
+      if (DIM == 2) P[2 * plane + p] = v;
+      P[DIM * plane + plane + p] = f.mul(f.add(U[NC - 1], pr), ir);
     }
-    if (VAR == 2 && (g.flags & FLAG_V_WEIGHTED)) return false;
+    // modified derivatives (Eq. limiter), one per direction
+    if constexpr (!PAIRS) {
+      if (LIMITER)
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) cell_limiter_of<DIM, SYS, VAR>(g, S, w, p, i, j, d, U, c, f);
+      return true;
+    }
     P2 pu = {0.0f, 0.0f}, pv = pu, pH = pu, pc2 = pu;
     if (SYS == SYS_EULER) {
       P2 q[NC], inv;
@@ -540,7 +553,7 @@ __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restric
       const P2 gm1 = P2{g.pg.gm1[0], g.pg.gm1[1]};
       p_prim<NC>(q, gm1, pu, pv, pH, pc2);
       pc2 = p_add(pc2, p_mul(gm1, pc2));  // gamma p / rho
-      if (VAR != 2) {
+      if (VAR == 0 || (VAR == 1 && g.face_pairs)) {
         const P2 sr = p_sqrt(q[0], inv);
         w.PRIM[p] = make_float2(sr.h, sr.l);
         w.PRIM[plane + p] = make_float2(pu.h, pu.l);
@@ -564,33 +577,28 @@ struct Leftover {
 
 // The cells p0 .. p0 + kThreads - 1 of a block, one per thread; every thread of the block calls it.
 // reused: the block calls it again with the same list.
-template <int DIM, int SYS, int VAR, bool LISTED>
+template <int DIM, int SYS, int VAR, int MODE>
 __device__ __forceinline__ void cell_tile(const Grid& g, const double* __restrict__ S, const Work& w, long long p0,
-                                          double& wsx, double& wsy, Leftover& lo, const PairSlots& sm,
-                                          bool reused) {
+                                          double& wsx, double& wsy, Leftover& lo, const PairSlots& sm, bool reused) {
   const long long p = p0 + threadIdx.x;
-  if (LISTED) {
+  if (MODE == MODE_LISTED) {
     // (one atomic per thread: collected by warp, the kernel takes 3 % longer with nothing to append)
-    if (p < g.plane && !cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm)) {
+    if (p < g.plane && !cell_body<DIM, SYS, VAR, true, true>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm)) {
       const unsigned int k = atomicAdd(w.status + 2, (unsigned int)DIM);
 #pragma unroll
       for (unsigned int d = 0; d < DIM; ++d) w.left_cells[k + d] = (unsigned int)p * 2u + d;
     }
     return;
   }
-  if (!g.pairs) {
-    if (p < g.plane) {
-      cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm);
-#pragma unroll 1
-      for (int d = 0; d < DIM; ++d) cell_limiter<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), d);
-    }
+  if (MODE == MODE_FP64) {
+    if (p < g.plane) cell_body<DIM, SYS, VAR, false, true>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm);
     return;
   }
   if (reused) __syncthreads();
   if (threadIdx.x == 0) lo.n = 0;
   __syncthreads();
   if (p < g.plane) {
-    if (!cell_body<DIM, SYS, VAR>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm)) {
+    if (!cell_body<DIM, SYS, VAR, true, true>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm)) {
       const int k = atomicAdd(&lo.n, DIM);
 #pragma unroll
       for (int d = 0; d < DIM; ++d) lo.item[k + d] = (unsigned short)(threadIdx.x * 2 + d);
@@ -604,14 +612,17 @@ __device__ __forceinline__ void cell_tile(const Grid& g, const double* __restric
 }
 
 // Bound by the FP64 pipe (85 % busy): 123 FP64 instructions per 2D Euler cell against 545 with the FP64
-// weights; 1024^2 0.24 ms per launch against 0.97 ms.
-template <int DIM, int SYS, int VAR, bool LISTED>
-__global__ void __launch_bounds__(kThreads, 4) k_cell(Grid g, const double* __restrict__ S, Work w, int slot) {
+// weights; 1024^2 0.24 ms per launch against 0.97 ms.  MODE_FP64 is the form of the grids that wait for one
+// thread's chain of instructions (pairs_of): no pair code, no slots, 130 registers and no spills (48^2
+// 24.3 us a launch; inside the kernel with the pairs 26.8 us).
+template <int DIM, int SYS, int VAR, int MODE>
+__global__ void __launch_bounds__(kThreads, MODE == MODE_FP64 ? 3 : 4) k_cell(Grid g, const double* __restrict__ S,
+                                                                             Work w, int slot) {
   __shared__ Leftover lo;
-  __shared__ ulonglong2 slots[4 * Traits<DIM, SYS>::NC * kThreads];
+  __shared__ ulonglong2 slots[MODE == MODE_FP64 ? 1 : 4 * Traits<DIM, SYS>::NC * kThreads];
   double wsx = 0.0, wsy = 0.0;
-  cell_tile<DIM, SYS, VAR, LISTED>(g, S, w, (long long)blockIdx.x * kThreads, wsx, wsy, lo,
-                                   PairSlots{slots + threadIdx.x}, false);
+  cell_tile<DIM, SYS, VAR, MODE>(g, S, w, (long long)blockIdx.x * kThreads, wsx, wsy, lo,
+                                 PairSlots{slots + (MODE == MODE_FP64 ? 0 : threadIdx.x)}, false);
   block_max2(wsx, wsy, w.alpha + slot * w.astride);
 }
 
@@ -684,8 +695,9 @@ __device__ __forceinline__ void r1_face_states(const double (&Uq)[4][NC], const 
 // Face work of one stage: face f of direction dir (x faces: f = j (nx+1) + i; y faces:
 // f = j nx + i), alpha = the LF coefficient of that direction.  PAIR: the nonlinear part of the
 // interpolation in pairs (hweno_pair.cuh); returns false, having written nothing, where the FP64
-// weights are needed.
-template <int DIM, int SYS, int VAR, bool PAIR>
+// weights are needed (R2: the flux of two close states in pairs).  STORED: the primitives were stored in
+// FP64; else they are formed from the states.
+template <int DIM, int SYS, int VAR, bool PAIR, bool STORED = false>
 __device__ __forceinline__ bool face_body(const Grid& g, const double* __restrict__ S, const Work& w, int dir,
                                           long long f, double alpha, const PairSlots& sm) {
   using T = Traits<DIM, SYS>;
@@ -724,10 +736,14 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
   double* out = dir == 0 ? w.FX : w.FY;
   const long long oplane = dir == 0 ? (long long)g.ny * (g.nx + 1) : (long long)(g.ny + 1) * g.nx;
   const long long fo = HW_IDX(dir == 0 ? (long long)line * (g.nx + 1) + fa : (long long)fa * g.nx + line, oplane);
-  if (DIM == 2) {
-    // Eq. (mixed), linear in the nodal values: independent of everything below.  Nodal values of
-    // mirrored neighbours (normal frame): f and the mixed value change sign except for the normal
-    // momentum, the normal-derivative flux changes sign only for the normal momentum.
+  // Eq. (mixed), linear in the nodal values: independent of everything below.  Nodal values of mirrored
+  // neighbours (normal frame): f and the mixed value change sign except for the normal momentum, the
+  // normal-derivative flux changes sign only for the normal momentum.  First where registers are short
+  // (PAIR) and for R2 (100^2: 75.7 us an evaluation, 77.2 at the end); else with the other nodal values, so
+  // that the loads of the primitives do not wait for its stores (96x170: 84.8 us, first 85.8).
+  constexpr bool kMixedFirst = PAIR || VAR == 2;
+  auto mixed = [&] {
+    if (DIM != 2) return;
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
       double o[4];
@@ -739,7 +755,8 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
       const int ko = SYS == SYS_EULER && dir == 1 && (k == 1 || k == 2) ? 3 - k : k;
       out[(foth * NC + ko) * oplane + fo] = fma(7.0 / 12.0, fu.add(o[1], o[2]), (-1.0 / 12.0) * fu.add(o[0], o[3]));
     }
-  }
+  };
+  if (kMixedFirst) mixed();
   const double a_adv = dir == 0 ? g.ax : g.ay;
   const P2 ih = p_const<float>(g.pg.ih[dir]);
   double Um[NC], Up[NC], Dm[NC], Dp[NC];
@@ -859,7 +876,7 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const double* U = Uq[1 + q];
-          if (!g.pairs) {
+          if (STORED) {
             const double* P = reinterpret_cast<const double*>(w.PRIM);
             const bool fx = VAR && fixed[1 + q];
             const double* F = g.fixP[fside[1 + q]];
@@ -891,7 +908,7 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
         r1_face_states<NC, SYS, false>(Uq, Zq, e, g, dir, Um, Up, Dm, Dp, fu);
     }
   }
-  if (VAR == 2 && g.pairs) {
+  if (VAR == 2 && PAIR) {
     double Us[NC], Ds[NC];
     P2 dif[NC], hdif[NC];
     float size[NC];
@@ -923,6 +940,7 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
     }
   }
   const bool cd2 = VAR && (g.flags & FLAG_CD2) != 0;
+  if (!kMixedFirst) mixed();
   double fh[NC], hh[NC];
 #pragma unroll
   for (int k = 0; k < NC; ++k) {
@@ -969,20 +987,19 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
 
 // The faces f0 .. f0 + kThreads - 1 (of nf) of direction dir, one per thread; every thread of the
 // block calls it.  reused: as cell_tile.
-template <int DIM, int SYS, int VAR, bool LISTED>
+template <int DIM, int SYS, int VAR, int MODE>
 __device__ __forceinline__ void face_tile(const Grid& g, const double* __restrict__ S, const Work& w, int dir,
                                           long long f0, long long nf, double alpha, Leftover& lo,
                                           const PairSlots& sm, bool reused) {
   const long long f = f0 + threadIdx.x;
-  if (LISTED && VAR != 2) {
-    if (f < nf && !face_body<DIM, SYS, VAR, true>(g, S, w, dir, f, alpha, sm))
-      w.left_faces[atomicAdd(w.status + 3, 1u)] = (unsigned int)(f + (dir == 0 ? 0 : (long long)(g.nx + 1) * g.ny));
+  // R2: only the fluxes (k_cell formed the face states)
+  if (MODE == MODE_FP64 || VAR == 2) {
+    if (f < nf) face_body<DIM, SYS, VAR, MODE != MODE_FP64, true>(g, S, w, dir, f, alpha, sm);
     return;
   }
-  // R2: only the fluxes (k_cell formed the face states); the weighted derivative needs the weights
-  // themselves
-  if (VAR == 2 || !g.pairs || (VAR && (g.flags & FLAG_V_WEIGHTED))) {
-    if (f < nf) face_body<DIM, SYS, VAR, false>(g, S, w, dir, f, alpha, sm);
+  if (MODE == MODE_LISTED) {
+    if (f < nf && !face_body<DIM, SYS, VAR, true>(g, S, w, dir, f, alpha, sm))
+      w.left_faces[atomicAdd(w.status + 3, 1u)] = (unsigned int)(f + (dir == 0 ? 0 : (long long)(g.nx + 1) * g.ny));
     return;
   }
   if (reused) __syncthreads();
@@ -1000,17 +1017,22 @@ __device__ __forceinline__ void face_tile(const Grid& g, const double* __restric
 // per SM (128 registers) cover it better than three or five (2D Euler 2048^2 with k_cell likewise: 4.70
 // against 4.75 and 4.94 ms per stage, before the pairs' loops).  2D Euler 1024^2: 0.70 ms per launch
 // against 2.33 ms with the FP64 weights.
-template <int DIM, int SYS, int VAR, bool LISTED>
-__global__ void __launch_bounds__(kThreads, 4) k_face(Grid g, const double* __restrict__ S, Work w, int slot) {
+// MODE_FP64 (small grids; the weighted derivative, which needs the weights everywhere): three blocks per SM,
+// 166 registers without spills.  The same form inside the kernel with the pairs had 128 registers and 496 B
+// of spills (916 B with the variants): 48^2 30.8 us a launch against 30.3; the weighted derivative at
+// 1024^2 2.67 ms against 2.56.
+template <int DIM, int SYS, int VAR, int MODE>
+__global__ void __launch_bounds__(kThreads, MODE == MODE_FP64 && DIM == 2 ? 3 : 4) k_face(
+    Grid g, const double* __restrict__ S, Work w, int slot) {
+  constexpr bool kSlots = SYS == SYS_EULER && VAR != 2 && MODE != MODE_FP64;  // the others use none
   __shared__ Leftover lo;
-  constexpr bool kSlots = SYS == SYS_EULER && VAR != 2;  // scalar laws and R2's faces use none
   __shared__ ulonglong2 slots[kSlots ? 4 * Traits<DIM, SYS>::NC * kThreads : 1];
   const int dir = blockIdx.y;
   const int n = dir == 0 ? g.nx : g.ny;
   const int nlines = dir == 0 ? g.ny : g.nx;
-  face_tile<DIM, SYS, VAR, LISTED>(g, S, w, dir, (long long)blockIdx.x * kThreads, (long long)(n + 1) * nlines,
-                                   __longlong_as_double((long long)w.alpha[slot * w.astride + dir]), lo,
-                                   PairSlots{slots + (kSlots ? threadIdx.x : 0)}, false);
+  face_tile<DIM, SYS, VAR, MODE>(g, S, w, dir, (long long)blockIdx.x * kThreads, (long long)(n + 1) * nlines,
+                                 __longlong_as_double((long long)w.alpha[slot * w.astride + dir]), lo,
+                                 PairSlots{slots + (kSlots ? threadIdx.x : 0)}, false);
 }
 
 // The listed cells and faces of a stage with the FP64 weights, in full warps (faces first, then cells): a

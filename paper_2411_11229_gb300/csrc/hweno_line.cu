@@ -126,7 +126,6 @@ __global__ void __launch_bounds__(kThreads) k_line_steps(Grid g, double* __restr
   gl.nx = m + 4;
   gl.plane = W;
   gl.bc = BC_TRANSMISSIVE;  // never met by what is used: the ghost cells are there
-  gl.pairs = 0;
   Work wl = w;
   wl.B = sB;
   wl.MD = sMD;
@@ -160,7 +159,7 @@ __global__ void __launch_bounds__(kThreads) k_line_steps(Grid g, double* __restr
       double U[NC];
 #pragma unroll
       for (int k = 0; k < NC; ++k) U[k] = sS[k * W + lane + 2];
-      CellState<1, SYS>().set(U, g, f, ws, wy);
+      CellState<1, SYS, true>().set(U, g, f, ws, wy);
     }
     if (ROLES == 4) {
       if (role == 0) {
@@ -203,11 +202,11 @@ __global__ void __launch_bounds__(kThreads) k_line_steps(Grid g, double* __restr
       // cells: the nodal values of all, the modified derivatives of the block's own; then faces 2 .. m + 2
       double wsx = 0.0, wsy = 0.0;
       if (t < m + 4) {
-        cell_body<1, SYS, 0>(gl, sS, wl, t, wsx, wsy, none);
+        cell_body<1, SYS, 0, false, false>(gl, sS, wl, t, wsx, wsy, none);
         if (t >= 2 && t < m + 2) cell_limiter<1, SYS, 0>(gl, sS, wl, t, 0);
       }
       __syncthreads();
-      if (t <= m) face_body<1, SYS, 0, false>(gl, sS, wl, 0, t + 2, alpha, none);
+      if (t <= m) face_body<1, SYS, 0, false, true>(gl, sS, wl, 0, t + 2, alpha, none);
       __syncthreads();
     } else {
       if (role < 2) {
@@ -224,7 +223,7 @@ __global__ void __launch_bounds__(kThreads) k_line_steps(Grid g, double* __restr
           }
       } else if (role == 2) {
         double wsx = 0.0, wsy = 0.0;
-        if (lane < m + 4) cell_body<1, SYS, 0>(gl, sS, wl, lane, wsx, wsy, none);
+        if (lane < m + 4) cell_body<1, SYS, 0, false, false>(gl, sS, wl, lane, wsx, wsy, none);
         __syncwarp();
         if (lane <= m)
 #pragma unroll

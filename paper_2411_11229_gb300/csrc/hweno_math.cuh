@@ -42,7 +42,8 @@ struct Grid {
   int nx, ny;   // ny = 1 in 1D
   int bc;
   int flags;    // FLAG_* (read by the extended kernels only)
-  int pairs;    // whether the nonlinear part is taken in pairs where it may be (see hweno_host.cuh)
+  int pairs;    // whether the nonlinear part is taken in pairs where it may be (see hweno_host.cuh), in
+  int face_pairs;  // the cells, and in the faces (the plain scheme: as in the cells)
   int listed;   // whether what is left to the FP64 weights goes to the grid's list (see hweno_host.cuh)
   long long plane;  // nx * ny
   double dx, dy, inv_dx, inv_dy;
