@@ -617,6 +617,7 @@ __device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __res
   double Uq[2][NC];                  // the inner cells
   double Um[NC], Up[NC], Dm[NC], Dp[NC];  // interface states less the corrections
   const double k21 = g.uvd[dir][0], k3 = g.uvd[dir][1], l3 = g.l3[dir], l9 = g.l9[dir];
+  bool units;
   {
     double U[4][NC], Z[4][NC];
 #pragma unroll
@@ -635,7 +636,7 @@ __device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __res
       mirror_U<NC>(U[q], refl[q]);
       mirror_D<NC>(Z[q], refl[q]);
     }
-    if (!(p_units(U[1][0], U[1][NC - 1], g.pg.hexp) && p_units(U[2][0], U[2][NC - 1], g.pg.hexp))) return false;
+    units = p_units(U[1][0], U[1][NC - 1], g.pg.hexp) && p_units(U[2][0], U[2][NC - 1], g.pg.hexp);
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
       const double a = fu.sub(U[1][k], U[0][k]), b = fu.sub(U[2][k], U[1][k]), c = fu.sub(U[3][k], U[2][k]);
@@ -697,7 +698,7 @@ __device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __res
 #pragma unroll
     for (int s = 0; s < NC; ++s) c[s] = sm.get(slot_c(s));
     e.back(c, nn);
-    if (!ok || !p_finite<NC>(nn)) return false;
+    if (!units || !ok || !p_finite<NC>(nn)) return false;
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
       const P2 a = p_lane0(nn[k]), b = p_lane1(nn[k]);
