@@ -139,7 +139,9 @@ constexpr long long kLineMaxCells = hw::kSMs * (hw::kThreads - 4LL);
 // leaves it idle and waits for each thread's chain of instructions instead, which is the longer one in
 // pairs: one evaluation of 1D Euler at 2048 cells 43 us in FP64, 53 us in pairs; of 2D Euler at 48^2
 // 62 and 74 us (with fronts 60 and 82), at 96x170 84 and 80 (83 and 98), at 128x200 123 and 88 (123 and
-// 111).  A scalar law's chain is short: at 182x181 40 and 46 us, at 256^2 58 and 48.
+// 111).  A scalar law's chain is short: at 182x181 40 and 46 us, at 256^2 58 and 48.  A 1D grid has one more
+// face than cells, and a second warp of faces on some scheduler from 19456 cells on: 1D Euler at 18849
+// 41.8 us a stage in FP64, 52.2 in pairs; at 20001 63.6 and 57.4 an evaluation.
 constexpr long long kPairMinCells = hw::kSMs * 4LL * 32;
 // Mesh sizes whose pairs (and those of their inverses and of the derivatives on them) have all of their 48
 // bits inside the FP32 range: 2^-64 to 2^64.  At 1e-36 the second half of h is an FP32 denormal.
@@ -148,7 +150,7 @@ inline bool pair_mesh(const hweno_ctx* h) {
 }
 inline int pairs_of(const hweno_ctx* h) {
   if (!pair_mesh(h)) return 0;
-  if (h->dim == 1) return h->nx > kLineMaxCells;
+  if (h->dim == 1) return h->nx >= kPairMinCells;
   return (long long)h->nx * h->ny > kPairMinCells * (h->system == hw::SYS_EULER ? 1 : 2);
 }
 

@@ -155,3 +155,20 @@ def test_constant_state_stays_constant(nx, ny, flags):
     L, M = (t.cpu().numpy() for t in s.rhs())
     assert np.array_equal(M, S)
     assert np.abs(L).max() <= 1e-13
+
+
+@pytest.mark.parametrize("kind", ["smooth", "jumps"])
+@pytest.mark.parametrize("n,kernels", [(18848, "line"), (18849, "stages"), (19455, "stages"), (19456, "stages"), (30011, "stages")])
+def test_sides_of_the_1d_rules(n, kernels, kind):
+    """Steps in one launch up to 18848 cells, pairs from 19456 (a second warp of faces to a scheduler)."""
+    S, dx = W.euler1d_random(n, seed=9, kind=kind)
+    cfg = O.make_cfg(1, O.EULER, n, dx=dx, bc=T)
+    s = Solver(1, "euler", n, dx=dx, bc="transmissive")
+    s.set_state(S)
+    for got, ext, own in zip(s.rhs(), O.rhs_ext(cfg, S)[:2], O.rhs(cfg, S)):
+        _bar(got.cpu().numpy(), ext, own)
+    s.set_time(0.0, 0.0)
+    n0 = s.launch_count()
+    s.step(0.0, 2)
+    assert s.launch_count() - n0 == (1 if kernels == "line" else 18)
+    s.sync()
