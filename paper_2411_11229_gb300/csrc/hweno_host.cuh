@@ -31,61 +31,6 @@ struct Launchers {
 
 inline unsigned blocks_for(long long n) { return (unsigned)((n + hw::kThreads - 1) / hw::kThreads); }
 
-template <int DIM, int SYS, int VAR>
-struct L {
-  static void cell(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
-    const unsigned nb = blocks_for(g.plane);
-    if (!g.pairs) {
-      hw::k_cell<DIM, SYS, VAR, hw::MODE_FP64><<<nb, hw::kThreads, 0, st>>>(g, S, w, slot);
-    } else if (DIM == 2 && g.listed) {
-      hw::k_cell<2, SYS, VAR, hw::MODE_LISTED><<<nb, hw::kThreads, 0, st>>>(g, S, w, slot);
-      if (VAR == 2) left(g, S, w, slot, st);  // R2's faces need what is left of the cells
-    } else {
-      hw::k_cell<DIM, SYS, VAR, hw::MODE_BLOCK><<<nb, hw::kThreads, 0, st>>>(g, S, w, slot);
-    }
-  }
-  static void left(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
-    hw::k_left<2, SYS, VAR><<<3 * hw::kSMs, hw::kThreads, 0, st>>>(g, S, w, slot);
-  }
-  static void face(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
-    const long long nfx = (long long)(g.nx + 1) * g.ny;
-    const long long nfy = DIM == 2 ? (long long)(g.ny + 1) * g.nx : 0;
-    const dim3 grid(blocks_for(nfx > nfy ? nfx : nfy), DIM);
-    if (!g.face_pairs) {
-      hw::k_face<DIM, SYS, VAR, hw::MODE_FP64><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
-    } else if (DIM == 2 && VAR != 2 && g.listed) {
-      hw::k_face<2, SYS, VAR, hw::MODE_LISTED><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
-      left(g, S, w, slot, st);
-    } else {
-      hw::k_face<DIM, SYS, VAR, hw::MODE_BLOCK><<<grid, hw::kThreads, 0, st>>>(g, S, w, slot);
-    }
-  }
-  static void update(const Grid& g, double* S, const Work& w, int mode, int stage, double a, double b,
-                     double dt, int slot, double* Lo, double* Mo, cudaStream_t st) {
-    hw::k_update<DIM, SYS, VAR><<<blocks_for(g.plane), hw::kThreads, 0, st>>>(g, S, w, mode, stage, a, b, dt, slot,
-                                                                            Lo, Mo);
-  }
-  static void wavespeed(const Grid& g, const double* S, const Work& w, int slot, cudaStream_t st) {
-    hw::k_wavespeed<DIM, SYS><<<blocks_for(g.plane), hw::kThreads, 0, st>>>(g, S, w, slot);
-  }
-  static void ghost(const Grid& g, const double* S, const Work& w, cudaStream_t st) {
-    hw::k_r2_ghost<DIM><<<blocks_for(2LL * DIM * w.gstride), hw::kThreads, 0, st>>>(g, S, w);
-  }
-  static constexpr Launchers table() {
-    return Launchers{&cell, &face, &update, &wavespeed, VAR == 2 ? &ghost : nullptr};
-  }
-};
-
-// [VAR][dim - 1][system]; R2 exists for the Euler equations only (for a scalar law the per-cell
-// and per-face bases coincide, and the host runs VAR 1)
-static const Launchers kTable[3][2][3] = {
-    {{L<1, hw::SYS_ADV, 0>::table(), L<1, hw::SYS_BURGERS, 0>::table(), L<1, hw::SYS_EULER, 0>::table()},
-     {L<2, hw::SYS_ADV, 0>::table(), L<2, hw::SYS_BURGERS, 0>::table(), L<2, hw::SYS_EULER, 0>::table()}},
-    {{L<1, hw::SYS_ADV, 1>::table(), L<1, hw::SYS_BURGERS, 1>::table(), L<1, hw::SYS_EULER, 1>::table()},
-     {L<2, hw::SYS_ADV, 1>::table(), L<2, hw::SYS_BURGERS, 1>::table(), L<2, hw::SYS_EULER, 1>::table()}},
-    {{L<1, hw::SYS_ADV, 1>::table(), L<1, hw::SYS_BURGERS, 1>::table(), L<1, hw::SYS_EULER, 2>::table()},
-     {L<2, hw::SYS_ADV, 1>::table(), L<2, hw::SYS_BURGERS, 1>::table(), L<2, hw::SYS_EULER, 2>::table()}}};
-
 inline size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace hwh
@@ -354,47 +299,15 @@ inline int read_status(hweno_ctx* h) {
   return st ? HWENO_ENONPHYS : HWENO_OK;
 }
 
-inline const Launchers& launchers(const hweno_ctx* h) { return kTable[h->var][h->dim - 1][h->system]; }
+// the launchers of a handle's stage kernels (hweno_api.cu holds the kernels)
+const Launchers& launchers(const hweno_ctx* h);
 
 // one spatial-operator evaluation: cell, face; then update in the requested mode
 // alpha_override (device, 2 doubles, may be null): LF coefficients to use instead of the
 // wavespeeds of S_in (the recorded alphas of an adjoint replay)
-inline int stage(hweno_ctx* h, const double* S_in, double* S_out, int mode, int st, double dt, int slot, double* Lo,
-          double* Mo, const double* alpha_override = nullptr) {
-  const Grid g = grid_of(h);
-  const Launchers& f = launchers(h);
-  if (cudaMemsetAsync(h->w.alpha + 2 * slot, 0, 2 * sizeof(unsigned long long), h->stream) != cudaSuccess)
-    return HWENO_ECUDA;
-  cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-  if (h->profiling) {
-    for (int k = 0; k < 4; ++k)
-      if (cudaEventCreate(&ev[k]) != cudaSuccess) return HWENO_ECUDA;
-    for (int k = 0; k < 4; ++k) h->events.push_back(ev[k]);
-  }
-  static const double a_k[3] = {0.0, 0.75, 1.0 / 3.0};
-  static const double b_k[3] = {1.0, 0.25, 2.0 / 3.0};
-  if (ev[0]) cudaEventRecord(ev[0], h->stream);
-  f.cell(g, S_in, h->w, slot, h->stream);
-  if (f.ghost) {
-    f.ghost(g, S_in, h->w, h->stream);
-    h->launches += 1;
-  }
-  if (alpha_override &&
-      cudaMemcpyAsync(h->w.alpha + slot * h->w.astride, alpha_override, 2 * sizeof(double), cudaMemcpyDeviceToDevice,
-                      h->stream) != cudaSuccess)
-    return HWENO_ECUDA;
-  if (ev[1]) cudaEventRecord(ev[1], h->stream);
-  // LF coefficients held for the whole step: stages 2 and 3 read the first stage's slot
-  const bool held = h->var != 0 && (h->flags & HWENO_FLAG_ALPHA_STEP) && mode == 0 && st > 0;
-  f.face(g, S_in, h->w, held ? slot - st : slot, h->stream);
-  if (ev[2]) cudaEventRecord(ev[2], h->stream);
-  f.update(g, S_out, h->w, mode, st, a_k[st], b_k[st], dt, slot, Lo, Mo, h->stream);
-  if (ev[3]) cudaEventRecord(ev[3], h->stream);
-  h->launches += 3 + g.listed;
-  return cuda_status();
-}
+int stage(hweno_ctx* h, const double* S_in, double* S_out, int mode, int st, double dt, int slot, double* Lo, double* Mo,
+          const double* alpha_override = nullptr);
 
-// one forward stage in place with fixed dt and the given LF coefficients
 // bounds-checked build: the out-of-range index records of the batched and adjoint translation
 // units (count since the last call, first source line; 0 in a normal build)
 unsigned int bounds_take_batch(int* line);
@@ -407,6 +320,7 @@ unsigned int bounds_take_adjoint(int* line);
 // was one of these.
 int line_steps(hweno_ctx* h, double dt, int nsteps, bool* done);
 
+// one forward stage in place with fixed dt and the given LF coefficients
 inline int stage_replay(hweno_ctx* h, double* S, int st, double dt, const double* alpha2_dev) {
   return stage(h, S, S, 0, st, dt, st, nullptr, nullptr, alpha2_dev);
 }
