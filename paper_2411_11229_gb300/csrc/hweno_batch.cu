@@ -43,14 +43,13 @@ struct BatchArgs {
   int slot;
 };
 
-template <int DIM>
+template <int DIM, int MODE>
 __device__ __forceinline__ void batch_cells(const BatchInst& I, long long p0, int tpi, int slot, Leftover& lo,
                                             const PairSlots& sm) {
   double wsx = 0.0, wsy = 0.0;
   for (int t = 0; t < tpi; ++t) {
     double a = 0.0, b = 0.0;
-    cell_tile<DIM, SYS_EULER, 0, MODE_BLOCK>(I.g, I.S, I.w, p0 + (long long)t * kThreads, a, b, lo, sm,
-                                 true);
+    cell_tile<DIM, SYS_EULER, 0, MODE>(I.g, I.S, I.w, p0 + (long long)t * kThreads, a, b, lo, sm, true);
     wsx = speed_bits(a) > speed_bits(wsx) ? a : wsx;
     wsy = speed_bits(b) > speed_bits(wsy) ? b : wsy;
   }
@@ -58,14 +57,13 @@ __device__ __forceinline__ void batch_cells(const BatchInst& I, long long p0, in
   __syncthreads();  // the reduction's shared arrays are reused by the next item
 }
 
-template <int DIM>
+template <int DIM, int MODE>
 __device__ __forceinline__ void batch_faces(const BatchInst& I, int dir, long long f0, int tpi, int slot,
                                             Leftover& lo, const PairSlots& sm) {
   const long long nf = dir == 0 ? (long long)(I.g.nx + 1) * I.g.ny : (long long)(I.g.ny + 1) * I.g.nx;
   const double alpha = __longlong_as_double((long long)I.w.alpha[slot * I.w.astride + dir]);
   for (int t = 0; t < tpi; ++t)
-    face_tile<DIM, SYS_EULER, 0, MODE_BLOCK>(I.g, I.S, I.w, dir, f0 + (long long)t * kThreads, nf, alpha, lo,
-                                 sm, true);
+    face_tile<DIM, SYS_EULER, 0, MODE>(I.g, I.S, I.w, dir, f0 + (long long)t * kThreads, nf, alpha, lo, sm, true);
 }
 
 template <int DIM>
@@ -84,28 +82,31 @@ __device__ __forceinline__ void batch_update(const BatchInst& I, long long p0, i
 }
 
 // One Runge-Kutta stage of every instance.  Launched cooperatively with every block resident.
+// MODE1, MODE2: how the lines and the grids take the nonlinear part.
+template <int MODE1, int MODE2>
 __global__ void __launch_bounds__(kThreads) k_batch_stage(BatchArgs a) {
+  constexpr bool kPairs = MODE1 != MODE_FP64 || MODE2 != MODE_FP64;
   __shared__ Leftover lo;
-  __shared__ ulonglong2 slots[kStencilSlots * kThreads];
-  const PairSlots sm{slots + threadIdx.x};
+  __shared__ ulonglong2 slots[kPairs ? kStencilSlots * kThreads : 1];
+  const PairSlots sm{slots + (kPairs ? threadIdx.x : 0)};
   cg::grid_group grid = cg::this_grid();
   const long long span = (long long)kThreads * a.tiles_per_item;
   for (int it = blockIdx.x; it < a.ncells; it += gridDim.x) {
     const int2 c = a.cells[it];
     const BatchInst& I = a.inst[HW_IDX(c.x, a.ninst)];
     if (I.dim == 1)
-      batch_cells<1>(I, c.y * span, a.tiles_per_item, a.slot, lo, sm);
+      batch_cells<1, MODE1>(I, c.y * span, a.tiles_per_item, a.slot, lo, sm);
     else
-      batch_cells<2>(I, c.y * span, a.tiles_per_item, a.slot, lo, sm);
+      batch_cells<2, MODE2>(I, c.y * span, a.tiles_per_item, a.slot, lo, sm);
   }
   grid.sync();
   for (int it = blockIdx.x; it < a.nfaces; it += gridDim.x) {
     const int4 f = a.faces[it];
     const BatchInst& I = a.inst[HW_IDX(f.x, a.ninst)];
     if (I.dim == 1)
-      batch_faces<1>(I, 0, f.z * span, a.tiles_per_item, a.slot, lo, sm);
+      batch_faces<1, MODE1>(I, 0, f.z * span, a.tiles_per_item, a.slot, lo, sm);
     else
-      batch_faces<2>(I, f.y, f.z * span, a.tiles_per_item, a.slot, lo, sm);
+      batch_faces<2, MODE2>(I, f.y, f.z * span, a.tiles_per_item, a.slot, lo, sm);
   }
   grid.sync();
   for (int it = blockIdx.x; it < a.ncells; it += gridDim.x) {
@@ -121,29 +122,29 @@ __global__ void __launch_bounds__(kThreads) k_batch_stage(BatchArgs a) {
 // The same stage as persistent launches per phase and dimension (cell, face and update work of
 // the 2D items, then of the 1D items), each kernel at the register budget of its own code path;
 // stream order replaces the grid barriers.
-template <int DIM>
-__global__ void __launch_bounds__(kThreads, 4) k_batch_cells(BatchArgs a) {
+template <int DIM, int MODE>
+__global__ void __launch_bounds__(kThreads, MODE == MODE_FP64 ? 3 : 4) k_batch_cells(BatchArgs a) {
   __shared__ Leftover lo;
-  __shared__ ulonglong2 slots[4 * Traits<DIM, SYS_EULER>::NC * kThreads];
-  const PairSlots sm{slots + threadIdx.x};
+  __shared__ ulonglong2 slots[MODE == MODE_FP64 ? 1 : 4 * Traits<DIM, SYS_EULER>::NC * kThreads];
+  const PairSlots sm{slots + (MODE == MODE_FP64 ? 0 : threadIdx.x)};
   const long long span = (long long)kThreads * a.tiles_per_item;
   const int first = DIM == 2 ? 0 : a.ncells2, last = DIM == 2 ? a.ncells2 : a.ncells;
   for (int it = first + blockIdx.x; it < last; it += gridDim.x) {
     const int2 c = a.cells[it];
-    batch_cells<DIM>(a.inst[HW_IDX(c.x, a.ninst)], c.y * span, a.tiles_per_item, a.slot, lo, sm);
+    batch_cells<DIM, MODE>(a.inst[HW_IDX(c.x, a.ninst)], c.y * span, a.tiles_per_item, a.slot, lo, sm);
   }
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(kThreads, 4) k_batch_faces(BatchArgs a) {
+template <int DIM, int MODE>
+__global__ void __launch_bounds__(kThreads, MODE == MODE_FP64 ? 3 : 4) k_batch_faces(BatchArgs a) {
   __shared__ Leftover lo;
-  __shared__ ulonglong2 slots[4 * Traits<DIM, SYS_EULER>::NC * kThreads];
-  const PairSlots sm{slots + threadIdx.x};
+  __shared__ ulonglong2 slots[MODE == MODE_FP64 ? 1 : 4 * Traits<DIM, SYS_EULER>::NC * kThreads];
+  const PairSlots sm{slots + (MODE == MODE_FP64 ? 0 : threadIdx.x)};
   const long long span = (long long)kThreads * a.tiles_per_item;
   const int first = DIM == 2 ? 0 : a.nfaces2, last = DIM == 2 ? a.nfaces2 : a.nfaces;
   for (int it = first + blockIdx.x; it < last; it += gridDim.x) {
     const int4 f = a.faces[it];
-    batch_faces<DIM>(a.inst[HW_IDX(f.x, a.ninst)], DIM == 2 ? f.y : 0, f.z * span, a.tiles_per_item, a.slot, lo, sm);
+    batch_faces<DIM, MODE>(a.inst[HW_IDX(f.x, a.ninst)], DIM == 2 ? f.y : 0, f.z * span, a.tiles_per_item, a.slot, lo, sm);
   }
 }
 
@@ -172,6 +173,7 @@ unsigned int bounds_take_batch(int* line) {
 
 struct hweno_batch {
   int n;
+  int pairs[2];                       // [1D, 2D]: whether the phase kernels take the nonlinear part in pairs
   std::vector<hweno_ctx> inst;        // per-instance parameters and device views
   std::vector<size_t> state_off;      // offset of instance i in the packed state (doubles)
   size_t state_total;
@@ -198,6 +200,31 @@ struct hweno_batch {
 namespace {
 
 constexpr int kMaxTilesPerItem = 4;
+
+// Faces of the lines, or of the grids, of a batch above which their kernels take the nonlinear part in pairs:
+// more than a warp of them to a scheduler.  Below, the schedulers wait for each warp's chain of
+// instructions, the longer one in pairs.  Per stage, FP64 and pairs: lines, 1 to 9 of 2048 cells 38 to 46 and
+// 50 to 53 us, 10 of them 62 and 58, 40 of 1024 85 and 68; one grid of 64^2 or 96^2 60 and 42 to 50 (a
+// smooth wave) or 83 to 87 (fronts), of 101^2 83 and 53 or 98, of 128^2 82 and 47 or 93 to 98.
+constexpr size_t kBatchPairFaces = hw::kSMs * 4ULL * 32;
+
+using BatchKernel = void (*)(hw::BatchArgs);
+// the kernels of a batch: the cooperative stage, and the phases [1D, 2D][cells, faces, update]
+BatchKernel stage_kernel(const hweno_batch* b) {
+  using namespace hw;
+  static const BatchKernel kern[2][2] = {{k_batch_stage<MODE_FP64, MODE_FP64>, k_batch_stage<MODE_FP64, MODE_BLOCK>},
+                                         {k_batch_stage<MODE_BLOCK, MODE_FP64>, k_batch_stage<MODE_BLOCK, MODE_BLOCK>}};
+  return kern[b->pairs[0]][b->pairs[1]];
+}
+BatchKernel phase_kernel(const hweno_batch* b, int d, int ph) {
+  using namespace hw;
+  static const BatchKernel kern[2][2][3] = {
+      {{k_batch_cells<1, MODE_FP64>, k_batch_faces<1, MODE_FP64>, k_batch_update<1>},
+       {k_batch_cells<2, MODE_FP64>, k_batch_faces<2, MODE_FP64>, k_batch_update<2>}},
+      {{k_batch_cells<1, MODE_BLOCK>, k_batch_faces<1, MODE_BLOCK>, k_batch_update<1>},
+       {k_batch_cells<2, MODE_BLOCK>, k_batch_faces<2, MODE_BLOCK>, k_batch_update<2>}}};
+  return kern[b->pairs[d]][d][ph];
+}
 
 int build_items(hweno_batch* b, std::vector<int2>& cells, std::vector<int4>& faces) {
   const long long span = (long long)hw::kThreads * b->tiles_per_item;
@@ -271,14 +298,11 @@ int launch_stage(hweno_batch* b, int st) {
   if (b->mode == 1) {
     const int items[2][3] = {{b->ncells - b->ncells2, b->nfaces - b->nfaces2, b->ncells - b->ncells2},
                              {b->ncells2, b->nfaces2, b->ncells2}};
-    void (*kern[2][3])(hw::BatchArgs) = {
-        {hw::k_batch_cells<1>, hw::k_batch_faces<1>, hw::k_batch_update<1>},
-        {hw::k_batch_cells<2>, hw::k_batch_faces<2>, hw::k_batch_update<2>}};
     for (int ph = 0; ph < 3; ++ph)
       for (int d = 1; d >= 0; --d) {
         if (items[d][ph] == 0) continue;
         const int grid = std::max(1, std::min(items[d][ph], b->num_sms * b->occ_phase[d][ph]));
-        kern[d][ph]<<<grid, hw::kThreads, 0, b->stream>>>(a);
+        phase_kernel(b, d, ph)<<<grid, hw::kThreads, 0, b->stream>>>(a);
         b->launches += 1;
       }
     if (cudaGetLastError() != cudaSuccess) return HWENO_ECUDA;
@@ -294,7 +318,7 @@ int launch_stage(hweno_batch* b, int st) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, hw::k_batch_stage, a) != cudaSuccess) return HWENO_ECUDA;
+  if (cudaLaunchKernelEx(&cfg, stage_kernel(b), a) != cudaSuccess) return HWENO_ECUDA;
   b->launches += 1;
   return HWENO_OK;
 }
@@ -336,7 +360,8 @@ std::mutex g_tune_mu;
 std::map<std::string, std::pair<int, int>> g_tune_cache;  // batch signature -> (tiles/item, blocks/SM)
 
 std::string signature(const hweno_batch* b) {
-  std::string s;
+  std::string s = b->pairs[0] ? "p" : "f";  // the kernels' occupancies differ
+  s += b->pairs[1] ? "p;" : "f;";
   for (const hweno_ctx& h : b->inst)
     s += std::to_string(h.dim) + ":" + std::to_string(h.nx) + "x" + std::to_string(h.ny) + ";";
   return s;
@@ -387,6 +412,13 @@ int hweno_batch_create(int n, const hweno_desc* descs, hweno_batch_t** out) {
     nfaces += ((h.nx + 1) * h.ny + hw::kThreads - 1) / hw::kThreads;
     if (h.dim == 2) nfaces += ((h.ny + 1) * h.nx + hw::kThreads - 1) / hw::kThreads;
   }
+  size_t faces[2] = {0, 0};
+  bool mesh = true;
+  for (const hweno_ctx& h : b->inst) {
+    faces[h.dim - 1] += nfaces_of(&h);
+    mesh = mesh && pair_mesh(&h);
+  }
+  for (int d = 0; d < 2; ++d) b->pairs[d] = mesh && faces[d] > kBatchPairFaces;
   b->ws_tables = align_up(n * sizeof(hw::BatchInst)) + align_up((size_t)4 * 2 * n * 8) +
                  align_up(ncells * sizeof(int2)) + align_up(nfaces * sizeof(int4));
   b->ws_total = b->ws_inst_total + b->ws_tables;
@@ -404,14 +436,12 @@ int hweno_batch_create(int n, const hweno_desc* descs, hweno_batch_t** out) {
   if (cudaGetDevice(&dev) == cudaSuccess && cudaGetDeviceProperties(&prop, dev) == cudaSuccess)
     b->num_sms = prop.multiProcessorCount;
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hw::k_batch_stage, hw::kThreads, 0) == cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, stage_kernel(b), hw::kThreads, 0) == cudaSuccess)
     b->max_blocks_per_sm = occ;
-  void (*kern[2][3])(hw::BatchArgs) = {{hw::k_batch_cells<1>, hw::k_batch_faces<1>, hw::k_batch_update<1>},
-                                       {hw::k_batch_cells<2>, hw::k_batch_faces<2>, hw::k_batch_update<2>}};
   for (int d = 0; d < 2; ++d)
     for (int ph = 0; ph < 3; ++ph) {
       int o = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern[d][ph], hw::kThreads, 0) != cudaSuccess) o = 1;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, phase_kernel(b, d, ph), hw::kThreads, 0) != cudaSuccess) o = 1;
       b->occ_phase[d][ph] = std::max(1, o);
     }
   cudaGetLastError();
@@ -464,7 +494,6 @@ int hweno_batch_bind(hweno_batch_t* b, double* state_dev, void* ws) {
     h.w.alpha = b->alpha + 2 * i;
     h.w.astride = 2 * b->n;
     hi[i].g = grid_of(&h);
-    hi[i].g.pairs = hi[i].g.face_pairs = pair_mesh(&h);  // many instances share the FP64 pipe
     hi[i].w = h.w;
     hi[i].S = h.state;
     hi[i].dim = h.dim;
