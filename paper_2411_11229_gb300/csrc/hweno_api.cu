@@ -355,18 +355,21 @@ int hweno_run(hweno_t* h, double t_end, int64_t max_steps, int64_t* steps_done) 
   int rc = hweno_set_time(h, 0.0, t_end);
   if (rc) return rc;
   constexpr int kChunk = 16;  // CFL steps issued between two looks at the device clock
-  // Record one chunk as a CUDA graph on a private stream (the handle's stream may be the legacy
+  // One chunk recorded as a CUDA graph on a private stream (the handle's stream may be the legacy
   // default stream, which cannot be captured); steps past the end time leave the state unchanged,
-  // so a whole chunk can be issued without knowing where in it the end time falls.
+  // so a whole chunk can be issued without knowing where in it the end time falls.  Recorded when the first
+  // chunk turns out not to be one of line_steps, which is one launch as it is.
   cudaStream_t user = h->stream, priv = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
   long long chunk_launches = 0;
-  const bool line = h->dim == 1 && h->var == 0 && h->nx <= kLineMaxCells;  // one launch a chunk as it is
-  if (!h->profiling && !line && max_steps >= kChunk &&
-      cudaStreamCreateWithFlags(&priv, cudaStreamNonBlocking) == cudaSuccess &&
-      cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess &&
-      cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess) {
+  bool recorded = h->profiling || max_steps < kChunk;
+  auto record = [&] {
+    recorded = true;
+    if (cudaStreamCreateWithFlags(&priv, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&join, cudaEventDisableTiming) != cudaSuccess)
+      return;
     h->stream = priv;
     const long long l0 = h->launches;
     cudaGraph_t gr = nullptr;
@@ -383,7 +386,7 @@ int hweno_run(hweno_t* h, double t_end, int64_t max_steps, int64_t* steps_done) 
     if (gr) cudaGraphDestroy(gr);
     h->stream = user;
     cudaGetLastError();  // a failed capture leaves the plain path
-  }
+  };
   rc = HWENO_OK;
   for (;;) {
     double v[4] = {0, 0, 0, 0};
@@ -401,6 +404,11 @@ int hweno_run(hweno_t* h, double t_end, int64_t max_steps, int64_t* steps_done) 
     }
     if (v[1] >= t_end || done >= max_steps) break;
     const int64_t left = max_steps - done;
+    bool line = false;
+    rc = line_steps(h, 0.0, (int)(left < kChunk ? left : kChunk), &line);
+    if (rc) break;
+    if (line) continue;
+    if (!recorded) record();
     if (exec && left >= kChunk) {
       if (cudaEventRecord(fork, user) != cudaSuccess || cudaStreamWaitEvent(priv, fork, 0) != cudaSuccess ||
           cudaGraphLaunch(exec, priv) != cudaSuccess || cudaEventRecord(join, priv) != cudaSuccess ||
