@@ -383,6 +383,13 @@ int hweno_rhs_static(int dim, int system, int64_t nx, int64_t ny, double dx, dou
  * r_dev[i] = 1/x_dev[i] for i < n, launched on `stream`.  Device arrays; EINVAL on NULL/n < 0. */
 int hweno_selftest_rcp(const double *x_dev, double *r_dev, int64_t n, void *stream);
 
+/* Self-test of the library's FP64 square root and its reciprocal (the hardware approximation of
+ * 1/sqrt(x) refined by one third-order step; within one unit in the last place for positive x, denormals
+ * included; used for the sound speeds, and with them for the LF coefficients and the step size, for the
+ * Roe averages and the characteristic fields): s_dev[i] = sqrt(x_dev[i]), r_dev[i] = 1/sqrt(x_dev[i]) for
+ * i < n, launched on `stream`.  Device arrays; EINVAL on NULL/n < 0. */
+int hweno_selftest_sqrt(const double *x_dev, double *s_dev, double *r_dev, int64_t n, void *stream);
+
 /* Probe of the FP64 issue rate of the current GPU, the peak of the stage kernels' ALU roofline
  * (they are bound by the FP64 pipe, not by memory; Sec. 4's CFL-0.6 SSP-RK3 stepping of the
  * scheme is FP64 arithmetic throughout).  Launches, on `stream`, eight resident blocks of 256

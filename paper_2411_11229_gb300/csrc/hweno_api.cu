@@ -9,6 +9,14 @@ __global__ void k_rcp_check(const double* __restrict__ x, double* __restrict__ r
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) r[i] = rcp(x[i]);
 }
+__global__ void k_sqrt_check(const double* __restrict__ x, double* __restrict__ s, double* __restrict__ r, long long n) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const FU f = HW_PLAIN_FU;
+  if (i < n) {
+    s[i] = sqrt_full(x[i], f);
+    r[i] = rsqrt_full(x[i], f);
+  }
+}
 
 // FP64 issue probe: kDfmaChains independent chains a <- a b + c per thread, kDfmaIters times.  b
 // and c are read from a per-thread address (p[0] = p[1] = b, p[2] = p[3] = c), so they live in
@@ -610,6 +618,13 @@ int hweno_selftest_rcp(const double* x_dev, double* r_dev, int64_t n, void* stre
   if (!x_dev || !r_dev || n < 0) return HWENO_EINVAL;
   if (n == 0) return HWENO_OK;
   hw::k_rcp_check<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(x_dev, r_dev, n);
+  return cuda_status();
+}
+
+int hweno_selftest_sqrt(const double* x_dev, double* s_dev, double* r_dev, int64_t n, void* stream) {
+  if (!x_dev || !s_dev || !r_dev || n < 0) return HWENO_EINVAL;
+  if (n == 0) return HWENO_OK;
+  hw::k_sqrt_check<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(x_dev, s_dev, r_dev, n);
   return cuda_status();
 }
 

@@ -267,6 +267,11 @@ __device__ __forceinline__ void r2_cell(const double (&U3)[3][NC], const double 
 template <int DIM, int SYS, bool ROOT>
 struct CellState {
   double u = 0.0, v = 0.0, pr = 0.0, ir = 0.0, c = 0.0, ic = 0.0;
+  __device__ __forceinline__ bool speeds(double& wsx, double& wsy, const FU& f) const {
+    wsx = f.add(fabs(u), c);
+    wsy = DIM == 2 ? f.add(fabs(v), c) : 0.0;
+    return finite_bits(wsx) && finite_bits(wsy);
+  }
   // returns whether the state is physical
   __device__ __forceinline__ bool set(const double* U, const Grid& g, const FU& f, double& wsx, double& wsy) {
     constexpr int NC = Traits<DIM, SYS>::NC;
@@ -279,9 +284,13 @@ struct CellState {
       const double c2 = f.mul(g.gamma * pr, ir);
       if (ROOT) ic = rsqrt_fast(c2, f);
       c = ROOT ? f.mul(c2, ic) : sqrt_fast(c2, f);
-      wsx = f.add(fabs(u), c);
-      wsy = DIM == 2 ? f.add(fabs(v), c) : 0.0;
-      return positive_bits(U[0]) && positive_bits(pr) && finite_bits(wsx) && finite_bits(wsy);
+      bool ok = speeds(wsx, wsy, f) && positive_bits(U[0]) && positive_bits(pr);
+      if (!ok && denormal_bits(c2)) {  // off the usual way: the other cells do not pay for it
+        if (ROOT) ic = rsqrt_full(c2, f);
+        c = sqrt_full(c2, f);
+        ok = speeds(wsx, wsy, f) && positive_bits(U[0]) && positive_bits(pr);
+      }
+      return ok;
     }
     if (SYS == SYS_BURGERS) {
       wsx = fabs(U[0]);
@@ -899,7 +908,7 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
         const double vb = DIM == 2 ? fu.mul(fma(sq[0], vq[0], fu.mul(sq[1], vq[1])), iw) : 0.0;
         const double Hb = fu.mul(fma(sq[0], Hq[0], fu.mul(sq[1], Hq[1])), iw);
         const double c2 = g.gm1 * fma(-0.5, DIM == 2 ? fma(ub, ub, fu.mul(vb, vb)) : fu.mul(ub, ub), Hb);
-        const double ic = rsqrt_fast(c2, fu);
+        const double ic = rsqrt_full(c2, fu);
         e.setup(ub, vb, Hb, fu.mul(c2, ic), ic, g.gm1);
       }
       if (VAR && (g.flags & FLAG_V_WEIGHTED))

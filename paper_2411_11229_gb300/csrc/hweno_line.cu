@@ -75,7 +75,7 @@ __device__ __forceinline__ void line_side(const Grid& g, const double* S, int si
     const double sr = __shfl_down_sync(0xffffffffu, sl, 1);
     const double iw = rcp(f.add(sl, sr), f);
     const double ub = f.mul(fma(sl, ul, f.mul(sr, ur)), iw), Hb = f.mul(fma(sl, Hl, f.mul(sr, Hr)), iw);
-    const double c2 = g.gm1 * fma(-0.5, f.mul(ub, ub), Hb), ic = rsqrt_fast(c2, f);
+    const double c2 = g.gm1 * fma(-0.5, f.mul(ub, ub), Hb), ic = rsqrt_full(c2, f);
     e.setup(ub, 0.0, Hb, f.mul(c2, ic), ic, g.gm1);
     e.project(dl, wl, f);
     e.project(dr, wr, f);

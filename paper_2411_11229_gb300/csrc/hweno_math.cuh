@@ -122,7 +122,9 @@ __device__ __forceinline__ double rcp(double x, const FU& f = HW_PLAIN_FU) {
 }
 // sqrt(x) and 1/sqrt(x) for normal, positive x, likewise: r = rsqrt.approx.ftz.f64, e = 1 - x r^2, and
 // (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + ...: five FP64 instructions each, against 12 slots of the FP64
-// pipe for sqrt() and 9 for rsqrt().  NaN for x <= 0.
+// pipe for sqrt() and 9 for rsqrt().  At most one unit in the last place: the residual's own rounding is
+// halved by the series (a quarter to a half of a unit), the last sum adds half of one, and the terms left
+// out are 5 e^3/16 with e of 2^-20.
 __device__ __forceinline__ double rsqrt_approx(double x) {
   double r;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -135,6 +137,15 @@ __device__ __forceinline__ double sqrt_fast(double x, const FU& f) {
 __device__ __forceinline__ double rsqrt_fast(double x, const FU& f) {
   const double r = rsqrt_approx(x), e = fma(-f.mul(x, r), r, f.one);
   return fma(r, f.mul(e, fma(0.375, e, 0.5)), r);
+}
+// The same with denormals, which the approximation takes for zero: through a power of four.  NaN for x <= 0 and
+// for an infinity.
+__device__ __forceinline__ bool denormal_bits(double x) { return (__double2hiint(x) & 0x7fffffff) < 0x00100000; }
+__device__ __forceinline__ double sqrt_full(double x, const FU& f) {
+  return denormal_bits(x) ? 0x1p-54 * sqrt_fast(x * 0x1p108, f) : sqrt_fast(x, f);
+}
+__device__ __forceinline__ double rsqrt_full(double x, const FU& f) {
+  return denormal_bits(x) ? 0x1p54 * rsqrt_fast(x * 0x1p108, f) : rsqrt_fast(x, f);
 }
 
 // ---------------------------------------------------------------------------------------------
