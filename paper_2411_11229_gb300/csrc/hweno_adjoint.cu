@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_cell(Grid g, const double* __r
   }
   const long long n = aw.cells ? min((long long)aw.count[0], 2 * g.plane) : 2 * g.plane;
   for (; k < n; k += (long long)gridDim.x * kThreads) {
-    const unsigned int c = aw.cells ? aw.cells[k] : (unsigned int)k;
+    const unsigned int c = aw.cells ? aw.cells[HW_IDX(k, 2 * g.plane)] : (unsigned int)k;
     if ((long long)(c >> 1) < g.plane) adj_cell<DIM>(g, S, muM, aw, (int)(c & 1u), HW_IDX(c >> 1, g.plane));
   }
 }
@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_face(Grid g, const double* __r
   const long long all = nfx + (long long)(g.ny + 1) * g.nx;
   const long long n = aw.faces ? min((long long)aw.count[1], all) : all;
   for (; k < n; k += (long long)gridDim.x * kThreads) {
-    const long long f = HW_IDX(aw.faces ? (long long)aw.faces[k] : k, all);
+    const long long f = HW_IDX(aw.faces ? (long long)aw.faces[HW_IDX(k, all)] : k, all);
     if (f < all) adj_face<DIM>(g, S, muL, aw, alpha2, f < nfx ? 0 : 1, f < nfx ? f : f - nfx);
   }
 }
@@ -589,8 +589,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_cell_pair(Grid g, const dou
   extern __shared__ ulonglong2 adj_pair_slots[];
   if (p < g.plane && !adj_cell_pair(g, S, muM, aw, HW_IDX(p, g.plane), PairSlots{adj_pair_slots + threadIdx.x})) {
     const unsigned int k = atomicAdd(aw.count, 2u);
-    aw.cells[k] = (unsigned int)p * 2u;
-    aw.cells[k + 1] = (unsigned int)p * 2u + 1u;
+    aw.cells[HW_IDX(k, 2 * g.plane)] = (unsigned int)p * 2u;
+    aw.cells[HW_IDX((long long)k + 1, 2 * g.plane)] = (unsigned int)p * 2u + 1u;
   }
 }
 
@@ -857,7 +857,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_face_pair(Grid g, const dou
   const long long f = (long long)blockIdx.x * kThreads + threadIdx.x;
   extern __shared__ ulonglong2 adj_pair_slots[];
   if (f < nf && !adj_face_pair(g, S, muL, aw, alpha2, dir, f, PairSlots{adj_pair_slots + threadIdx.x}))
-    aw.faces[atomicAdd(aw.count + 1, 1u)] = (unsigned int)(f + (dir == 0 ? 0 : nfx));
+    aw.faces[HW_IDX(atomicAdd(aw.count + 1, 1u), nfx + (long long)(g.ny + 1) * g.nx)] =
+        (unsigned int)(f + (dir == 0 ? 0 : nfx));
 }
 
 // -------------------------------------------------------------------------------------------

@@ -595,7 +595,8 @@ __device__ __forceinline__ void cell_tile(const Grid& g, const double* __restric
     if (p < g.plane && !cell_body<DIM, SYS, VAR, true, true>(g, S, w, HW_IDX(p, g.plane), wsx, wsy, sm)) {
       const unsigned int k = atomicAdd(w.status + 2, (unsigned int)DIM);
 #pragma unroll
-      for (unsigned int d = 0; d < DIM; ++d) w.left_cells[k + d] = (unsigned int)p * 2u + d;
+      for (unsigned int d = 0; d < DIM; ++d)
+        w.left_cells[HW_IDX((long long)k + d, DIM * g.plane)] = (unsigned int)p * 2u + d;
     }
     return;
   }
@@ -1007,8 +1008,10 @@ __device__ __forceinline__ void face_tile(const Grid& g, const double* __restric
     return;
   }
   if (MODE == MODE_LISTED) {
-    if (f < nf && !face_body<DIM, SYS, VAR, true>(g, S, w, dir, f, alpha, sm))
-      w.left_faces[atomicAdd(w.status + 3, 1u)] = (unsigned int)(f + (dir == 0 ? 0 : (long long)(g.nx + 1) * g.ny));
+    if (f < nf && !face_body<DIM, SYS, VAR, true>(g, S, w, dir, f, alpha, sm)) {
+      const long long nfx = (long long)(g.nx + 1) * g.ny, all = nfx + (DIM == 2 ? (long long)(g.ny + 1) * g.nx : 0);
+      w.left_faces[HW_IDX(atomicAdd(w.status + 3, 1u), all)] = (unsigned int)(f + (dir == 0 ? 0 : nfx));
+    }
     return;
   }
   if (reused) __syncthreads();
@@ -1055,13 +1058,13 @@ __global__ void __launch_bounds__(kThreads, 3) k_left(Grid g, const double* __re
   const PairSlots none{nullptr};
   for (long long k = (long long)blockIdx.x * kThreads + threadIdx.x; k < nfw + nc; k += (long long)gridDim.x * kThreads) {
     if (k < nf) {
-      const long long f = HW_IDX(w.left_faces[k], all);
+      const long long f = HW_IDX(w.left_faces[HW_IDX(k, all)], all);
       const int dir = f < nfx ? 0 : 1;
       if (f < all)
         face_body<DIM, SYS, VAR, false>(g, S, w, dir, f - (dir == 0 ? 0 : nfx),
                                         __longlong_as_double((long long)w.alpha[slot * w.astride + dir]), none);
     } else if (k >= nfw) {
-      const unsigned int c = w.left_cells[k - nfw];
+      const unsigned int c = w.left_cells[HW_IDX(k - nfw, DIM * g.plane)];
       if ((long long)(c >> 1) < g.plane) cell_limiter<DIM, SYS, VAR>(g, S, w, HW_IDX(c >> 1, g.plane), (int)(c & 1u));
     }
   }
