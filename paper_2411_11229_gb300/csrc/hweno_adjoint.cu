@@ -511,14 +511,14 @@ __device__ __forceinline__ bool adj_cell_pair(const Grid& g, const double* __res
 #pragma unroll
     for (int k = 0; k < NC; ++k) sm.set(slot_w(k, v), p_renorm(q[k]));
   }
-  const P4 eps = p_const<F2>(g.pg.eps), id = p_const<F2>(g.pg.id1);
+  const P4 eps = p_const<F2>(g.pg.eps), id = p_const<F2>(g.pg.id1), Gd = p_const<F2>(g.pg.Gdp);
   bool ok = true;
 #pragma unroll 1
   for (int s = 0; s < NC; ++s) {
     P4 w0, w1, w2, w3;
-    sm.set(slot_c(s), p_correction_vjp<CORR_LIMITED>(sm.get(slot_w(s, 0)), sm.get(slot_w(s, 1)), sm.get(slot_w(s, 2)),
-                                                     sm.get(slot_w(s, 3)), h, eps, id, g.pg.Gd, sm.get(slot_c(s)), w0,
-                                                     w1, w2, w3, ok));
+    sm.set(slot_c(s), p_correction_vjp<CORR_LIMITED, false>(sm.get(slot_w(s, 0)), sm.get(slot_w(s, 1)),
+                                                            sm.get(slot_w(s, 2)), sm.get(slot_w(s, 3)), h, eps, id, Gd,
+                                                            sm.get(slot_c(s)), w0, w1, w2, w3, ok));
     sm.set(slot_w(s, 0), w0);
     sm.set(slot_w(s, 1), w1);
     sm.set(slot_w(s, 2), w2);
@@ -597,6 +597,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_cell_pair(Grid g, const dou
 // -------------------------------------------------------------------------------------------
 // The contributions of a 2D face with the transpose of the interpolation's nonlinear part in pairs;
 // false where the FP64 kernel is needed.
+template <bool SMALL32>
 __device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __restrict__ S,
                                               const double* __restrict__ muL, const AdjWork& aw,
                                               const double* __restrict__ alpha2, int dir, long long f, const PairSlots& sm) {
@@ -759,9 +760,9 @@ __device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __res
   for (int s = 0; s < NC; ++s) {
     bool ok = true;
     P4 w0, w1, w2, w3;
-    sm.set(slot_c(s), p_correction_vjp<CORR_FACE>(sm.get(slot_w(s, 0)), sm.get(slot_w(s, 1)), sm.get(slot_w(s, 2)),
-                                                  sm.get(slot_w(s, 3)), h, eps, ig, g.pg.G, sm.get(slot_c(s)), w0, w1,
-                                                  w2, w3, ok));
+    sm.set(slot_c(s), p_correction_vjp<CORR_FACE, SMALL32>(sm.get(slot_w(s, 0)), sm.get(slot_w(s, 1)),
+                                                           sm.get(slot_w(s, 2)), sm.get(slot_w(s, 3)), h, eps, ig,
+                                                           p_const<F2>(g.pg.Gp), sm.get(slot_c(s)), w0, w1, w2, w3, ok));
     sm.set(slot_w(s, 0), w0);
     sm.set(slot_w(s, 1), w1);
     sm.set(slot_w(s, 2), w2);
@@ -849,6 +850,7 @@ __device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __res
 // Bound by the FP64 pipe (72 % busy; the fluxes' transposes) with the pairs' latency between.  1024^2: 2.1 ms
 // per launch against 5.95 ms for the FP64 kernel; two or four blocks per SM: the adjoint step 11.6 and
 // 11.7 ms against 11.4 ms.
+template <bool SMALL32>
 __global__ void __launch_bounds__(kThreads, 3) k_adj_face_pair(Grid g, const double* __restrict__ S,
                                                                const double* __restrict__ muL, AdjWork aw,
                                                                const double* __restrict__ alpha2) {
@@ -856,7 +858,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_face_pair(Grid g, const dou
   const long long nfx = (long long)(g.nx + 1) * g.ny, nf = dir == 0 ? nfx : (long long)(g.ny + 1) * g.nx;
   const long long f = (long long)blockIdx.x * kThreads + threadIdx.x;
   extern __shared__ ulonglong2 adj_pair_slots[];
-  if (f < nf && !adj_face_pair(g, S, muL, aw, alpha2, dir, f, PairSlots{adj_pair_slots + threadIdx.x}))
+  if (f < nf && !adj_face_pair<SMALL32>(g, S, muL, aw, alpha2, dir, f, PairSlots{adj_pair_slots + threadIdx.x}))
     aw.faces[HW_IDX(atomicAdd(aw.count + 1, 1u), nfx + (long long)(g.ny + 1) * g.nx)] =
         (unsigned int)(f + (dir == 0 ? 0 : nfx));
 }
@@ -1158,7 +1160,8 @@ int stage_vjp(hweno_ctx* h, const Grid& g, const double* S, const double* alpha2
     // most of the work in pairs, the rest (listed on the way) in FP64: two blocks per SM take it in turn
     const unsigned bl = 2u * hw::kSMs;
     constexpr size_t pair_sm = (size_t)hw::kPairSlots * hw::kThreads * sizeof(ulonglong2);
-    if (cudaFuncSetAttribute(hw::k_adj_face_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_sm) !=
+    const auto face_pair = g.pg.ig1[0] >= hw::kSmall32 ? hw::k_adj_face_pair<true> : hw::k_adj_face_pair<false>;
+    if (cudaFuncSetAttribute(face_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_sm) !=
             cudaSuccess ||
         cudaFuncSetAttribute(hw::k_adj_cell_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_sm) !=
             cudaSuccess)
@@ -1167,7 +1170,7 @@ int stage_vjp(hweno_ctx* h, const Grid& g, const double* S, const double* alpha2
     if (g.plane >= kAdjPairMinCells && pair_mesh(h)) {
       if (cudaMemsetAsync(aw.count, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) return HWENO_ECUDA;
       hw::k_adj_cell_pair<<<bc, hw::kThreads, pair_sm, st>>>(g, S, muM, aw);
-      hw::k_adj_face_pair<<<dim3(bf, 2), hw::kThreads, pair_sm, st>>>(g, S, muL, aw, alpha2);
+      face_pair<<<dim3(bf, 2), hw::kThreads, pair_sm, st>>>(g, S, muL, aw, alpha2);
       h->launches += 2;
     } else {
       fw.cells = fw.faces = nullptr;

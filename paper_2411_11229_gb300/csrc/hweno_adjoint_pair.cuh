@@ -55,9 +55,13 @@ enum { CORR_LIMITED, CORR_FACE };
 // Backward of p_stencil and the correction of a kind: nb the adjoint of the correction; the adjoints
 // of d01, d12, y0, y2 are written, the correction itself is returned, and ok is cleared where it may
 // not be taken from pairs.  The tie |X| = |Y| takes half of
-// each, as d|x| = 0 at 0 does.
-template <int KIND>
-__device__ __forceinline__ P4 p_correction_vjp(P4 d01, P4 d12, P4 y0, P4 y2, P4 h, P4 eps, P4 inv_l, float G_, P4 nb,
+// each, as d|x| = 0 at 0 does.  SMALL32: the small term of the denominator, tau (G Q + e0 (e1 + e2)), in FP32.  The
+// derivatives, beside the linear part's of order one, are right to 2^-55 with 1/gamma_1 = 200, and 2^-53 with
+// 40, 2^-49 with 4; in pairs (the limiter, with its 1/d_1 of 20, and faces below kSmall32) to 2^-53 or better
+// whatever the linear weights.
+constexpr float kSmall32 = 100.0f;
+template <int KIND, bool SMALL32>
+__device__ __forceinline__ P4 p_correction_vjp(P4 d01, P4 d12, P4 y0, P4 y2, P4 h, P4 eps, P4 inv_l, P4 G, P4 nb,
                                                P4& d01b, P4& d12b, P4& y0b, P4& y2b, bool& ok) {
   // forward, as p_stencil and p_correction
   const P4 e1 = p_add(p_sqr(d01), eps), e2 = p_add(p_sqr(d12), eps);
@@ -75,15 +79,12 @@ __device__ __forceinline__ P4 p_correction_vjp(P4 d01, P4 d12, P4 y0, P4 y2, P4 
   const P4 tau = p_sqr(p_maxabs(X, Y));
   const P4 A1 = p_add(X, Y), A2 = p_sub(X, Y), e0 = p_add(e1, A1);
   const P4 S1 = p_mul(A1, e2), S2 = p_mul(A2, e1), Q = p_mul(e1, e2), PP = p_mul(e0, Q);
-  // the small term of the denominator, tau (G Q + e0 (e1 + e2)): FP32 is enough beside the face's 1/gamma_1
-  // = 200 (derivatives right to 2^-53), not beside the limiter's 1/d_1 = 20 (2^-49; in pairs 2^-55)
-  const F2 G = f_all<F2>(G_);
   const P4 e12 = p_add(e1, e2);
   P4 GQR;
-  if (KIND == CORR_LIMITED)
-    GQR = p_add(p_mulf(Q, G_), p_mul(e0, e12));
+  if (!SMALL32)
+    GQR = p_add(p_mul(Q, G), p_mul(e0, e12));
   else
-    GQR.h = f_fma(G, Q.h, f_mul(e0.h, e12.h));
+    GQR.h = f_fma(G.h, Q.h, f_mul(e0.h, e12.h));
   ok = p_smooth(tau.h, e0.h, e1.h, e2.h, PP.h) && ok;
   P4 q1, q2;
   if (KIND == CORR_LIMITED) {
@@ -97,7 +98,7 @@ __device__ __forceinline__ P4 p_correction_vjp(P4 d01, P4 d12, P4 y0, P4 y2, P4 
     q2 = p_add(p_mix(a, a2), b);
   }
   P4 den = p_mul(inv_l, PP);
-  if (KIND == CORR_LIMITED)
+  if (!SMALL32)
     den = p_add(den, p_mul(tau, GQR));
   else
     den.l = f_fma(tau.h, GQR.h, den.l);
@@ -110,17 +111,17 @@ __device__ __forceinline__ P4 p_correction_vjp(P4 d01, P4 d12, P4 y0, P4 y2, P4 
   const P4 q1b = p_mul(Nb, S1), q2b = p_mul(Nb, S2), S1b = p_mul(Nb, q1), S2b = p_mul(Nb, q2);
   const P4 Pb = p_mul(inv_l, denb);
   P4 Qb = p_mul(Pb, e0), e0b = p_mul(Pb, Q), e1b, e2b;
-  if (KIND == CORR_LIMITED) {
+  if (!SMALL32) {
     const P4 Rb = p_mul(denb, tau), t = p_mul(Rb, e0);
     p_acc(taub, denb, GQR);
-    Qb = p_add(Qb, p_mulf(Rb, G_));
+    p_acc(Qb, Rb, G);
     p_acc(e0b, Rb, e12);
     e1b = p_add(p_add(p_mul(Qb, e2), p_mul(S2b, A2)), t);
     e2b = p_add(p_add(p_mul(Qb, e1), p_mul(S1b, A1)), t);
   } else {
     const F2 Rb = f_mul(denb.h, tau.h);
     taub.l = f_fma(denb.h, GQR.h, taub.l);
-    Qb.l = f_fma(Rb, G, Qb.l);
+    Qb.l = f_fma(Rb, G.h, Qb.l);
     e0b.l = f_fma(Rb, e12.h, e0b.l);
     e1b = p_add(p_mul(Qb, e2), p_mul(S2b, A2));
     e2b = p_add(p_mul(Qb, e1), p_mul(S1b, A1));

@@ -245,6 +245,8 @@ inline Grid grid_of(const hweno_ctx* h) {
   to_pair(g.Gd + 2.0, g.pg.id1);
   g.pg.G = (float)g.G;
   g.pg.Gd = (float)g.Gd;
+  to_pair(g.G, g.pg.Gp);
+  to_pair(g.Gd, g.pg.Gdp);
   g.pg.hexp = 0;
   for (int d = 0; d < h->dim; ++d) g.pg.hexp = std::max(g.pg.hexp, std::ilogb(hs[d]));
   g.grav = h->grav;

@@ -34,6 +34,7 @@ struct Traits {
 // exponent of the larger mesh size, not below 0 (p_units).
 struct PairGrid {
   float h[2][2], ih[2][2], gm1[2], eps[2], ig1[2], id1[2], G, Gd;
+  float Gp[2], Gdp[2];  // G and Gd as pairs (the adjoint)
   int hexp;
 };
 
