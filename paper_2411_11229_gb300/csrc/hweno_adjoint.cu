@@ -431,7 +431,7 @@ __device__ __forceinline__ bool adj_cell_pair(const Grid& g, const double* __res
   const long long plane = g.plane;
   const FU fu = fu_of(aw.scal);
   const int i = (int)(p % g.nx), j = (int)(p / g.nx);
-  bool refl[2][2];
+  bool refl[2][2], units;
   double ob[2][NC];
   P4 U1[NC];
   {
@@ -440,7 +440,7 @@ __device__ __forceinline__ bool adj_cell_pair(const Grid& g, const double* __res
     double Uc[NC];
 #pragma unroll
     for (int k = 0; k < NC; ++k) Uc[k] = S[k * plane + p];
-    if (!p_units(Uc[0], Uc[NC - 1], g.pg.hexp)) return false;
+    units = p_units(Uc[0], Uc[NC - 1], g.pg.hexp);
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
       const int n = d == 0 ? g.nx : g.ny, a0 = d == 0 ? i : j, fld = d == 0 ? 1 : 2;
@@ -526,7 +526,7 @@ __device__ __forceinline__ bool adj_cell_pair(const Grid& g, const double* __res
   }
 #pragma unroll
   for (int s = 0; s < NC; ++s) c[s] = sm.get(slot_c(s));
-  if (!ok || !p_finite<NC>(c)) return false;
+  if (!units || !ok || !p_finite<NC>(c)) return false;
   EigPBar<F2> eb;
   eb.zero();
   p_back_eig(c, qb, eb);

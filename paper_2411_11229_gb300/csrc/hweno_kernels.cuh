@@ -356,7 +356,8 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
                                                   P2 pc2, const PairSlots& sm, const FU& f) {
   constexpr int NC = Traits<DIM, SYS>::NC;
   const long long plane = g.plane;
-  if (SYS == SYS_EULER && !p_units(U[0], U[NC - 1], g.pg.hexp)) return false;
+  // (asked for last: a return here would hold up the loads of the neighbours)
+  const bool units = SYS != SYS_EULER || p_units(U[0], U[NC - 1], g.pg.hexp);
   // FP64: p_0'(x_i) = 3/4 (u_{i+1} - u_{i-1})/h - (v_{i-1} + v_{i+1})/4 and (R2) the derivatives at the two
   // faces; the linear parts of R2's values less the centre value in pairs, which hold them to the last
   // bit of the states where the stencil's differences are small beside these
@@ -427,7 +428,7 @@ __device__ __forceinline__ bool cell_limiter_pair(const Grid& g, const double* _
   }
   const P4 h = p_pack(p_const<float>(g.pg.h[0]), p_const<float>(g.pg.h[DIM - 1]));
   P4 nm[NC], np[NC], nt[NC];
-  if (!p_cell<NC, SYS, VAR == 2>(sm, e, h, g.pg, nm, np, nt)) return false;
+  if (!p_cell<NC, SYS, VAR == 2>(sm, e, h, g.pg, nm, np, nt) || !units) return false;
 #pragma unroll
   for (int d = 0; d < DIM; ++d) {
     const P2 ih = p_const<float>(g.pg.ih[d]);
@@ -811,9 +812,8 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
       if (VAR && fixed[q]) load_fixed<NC, SYS>(g, fside[q], dir, Uq[q], Zq[q]);
     }
     if (PAIR) {
-      if (SYS == SYS_EULER &&
-          !(p_units(Uq[1][0], Uq[1][NC - 1], g.pg.hexp) && p_units(Uq[2][0], Uq[2][NC - 1], g.pg.hexp)))
-        return false;
+      const bool units = SYS != SYS_EULER || (p_units(Uq[1][0], Uq[1][NC - 1], g.pg.hexp) &&
+                                              p_units(Uq[2][0], Uq[2][NC - 1], g.pg.hexp));
       double dU[3][NC];
 #pragma unroll
       for (int q = 0; q < 3; ++q)
@@ -864,7 +864,7 @@ __device__ __forceinline__ bool face_body(const Grid& g, const double* __restric
       P4 n[NC];
       P2 sum[NC], dif[NC], hdif[NC];
       float size[NC];
-      if (!p_face<NC, SYS>(dU, Zq, da, zo, zi, e, g.pg, dir, sm, n, sum, dif, hdif, size)) return false;
+      if (!p_face<NC, SYS>(dU, Zq, da, zo, zi, e, g.pg, dir, sm, n, sum, dif, hdif, size) || !units) return false;
       if (SYS == SYS_EULER) {
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
