@@ -263,7 +263,8 @@ __device__ __forceinline__ void r2_cell(const double (&U3)[3][NC], const double 
 }
 
 // Velocities, pressure, 1/rho of a cell, and its wavespeeds per direction; ROOT: 1/c as well (the FP64
-// weights' fields need both, and one chain of instructions gives both)
+// weights' fields need both, and one chain of instructions gives both; in 1D, whose steps in one launch
+// give the two to different warps, they are apart: 849 us against 856 for ten steps of 16383 cells)
 template <int DIM, int SYS, bool ROOT>
 struct CellState {
   double u = 0.0, v = 0.0, pr = 0.0, ir = 0.0, c = 0.0, ic = 0.0;
@@ -307,15 +308,23 @@ struct CellState {
 // weights, from the cell's state U and what CellState holds of it.
 template <int DIM, int SYS, int VAR>
 __device__ __forceinline__ void cell_limiter_of(const Grid& g, const double* __restrict__ S, const Work& w, long long p,
-                                                int i, int j, int d, const double* U, const CellState<DIM, SYS, true>& c,
+                                                int i, int j, int d, const double* U,
+                                                const CellState<DIM, SYS, DIM == 2>& c,
                                                 const FU& f) {
   constexpr int NC = Traits<DIM, SYS>::NC;
   const long long plane = g.plane;
   double U3[3][NC], D3[3][NC];
   load_stencil3<DIM, SYS, VAR, NC>(g, S, d, i, j, d == 0 ? i : j, U, U3, D3);
   Eig<NC> e;
-  if (SYS == SYS_EULER)
-    e.setup(d == 0 ? c.u : c.v, d == 0 ? c.v : c.u, f.mul(f.add(U[NC - 1], c.pr), c.ir), c.c, c.ic, g.gm1);
+  if (SYS == SYS_EULER) {
+    double cc = c.c, ic = c.ic;
+    if (DIM == 1) {
+      const double c2 = f.mul(g.gamma * c.pr, c.ir);
+      ic = rsqrt_full(c2, f);
+      cc = f.mul(c2, ic);
+    }
+    e.setup(d == 0 ? c.u : c.v, d == 0 ? c.v : c.u, f.mul(f.add(U[NC - 1], c.pr), c.ir), cc, ic, g.gm1);
+  }
   double out[NC];
   if (VAR == 2) {
     double fs[4][NC];
@@ -342,7 +351,7 @@ __device__ __forceinline__ void cell_limiter(const Grid& g, const double* __rest
   double U[NC], wx, wy;
 #pragma unroll
   for (int k = 0; k < NC; ++k) U[k] = S[k * g.plane + p];
-  CellState<DIM, SYS, true> c;
+  CellState<DIM, SYS, DIM == 2> c;
   c.set(U, g, f, wx, wy);
   cell_limiter_of<DIM, SYS, VAR>(g, S, w, p, (int)(p % g.nx), (int)(p / g.nx), d, U, c, f);
 }
@@ -482,7 +491,7 @@ __device__ __forceinline__ bool cell_body(const Grid& g, const double* __restric
       if (DIM == 2) Wd[k] = S[(2 * NC + k) * plane + p];
     }
     // primitives and wavespeeds
-    CellState<DIM, SYS, !PAIRS> c;
+    CellState<DIM, SYS, !PAIRS && DIM == 2> c;
     if (!c.set(U, g, f, wsx, wsy)) atomicOr(w.status, 1u);
     const double u = c.u, v = c.v, pr = c.pr, ir = c.ir;
     if (VAR && (g.flags & FLAG_ALPHA_LOCAL)) {

@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kThreads) k_line_steps(Grid g, double* __restr
       double U[NC];
 #pragma unroll
       for (int k = 0; k < NC; ++k) U[k] = sS[k * W + lane + 2];
-      CellState<1, SYS, true>().set(U, g, f, ws, wy);
+      CellState<1, SYS, false>().set(U, g, f, ws, wy);
     }
     if (ROLES == 4) {
       if (role == 0) {
