@@ -52,7 +52,8 @@ struct hweno_ctx {
   unsigned char* ws;
   hw::Work w;
   long long launches;
-  // optional per-kernel timing: events recorded around the three launches of every stage
+  // optional per-kernel timing: events recorded around the launches of every stage (cell; face, with what is
+  // left to the FP64 weights; update)
   bool profiling;
   std::vector<cudaEvent_t> events;  // groups of 4: before cell, before face, before update, after
   double kernel_ms[3];

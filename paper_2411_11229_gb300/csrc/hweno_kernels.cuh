@@ -714,8 +714,8 @@ __device__ __forceinline__ void r1_face_states(const double (&Uq)[4][NC], const 
 // ---------------------------------------------------------------------------------------------
 // Face work of one stage: face f of direction dir (x faces: f = j (nx+1) + i; y faces:
 // f = j nx + i), alpha = the LF coefficient of that direction.  PAIR: the nonlinear part of the
-// interpolation in pairs (hweno_pair.cuh); returns false, having written nothing, where the FP64
-// weights are needed (R2: the flux of two close states in pairs).  STORED: the primitives were stored in
+// interpolation in pairs (hweno_pair.cuh); returns false, having written the mixed flux at most, where the
+// FP64 weights are needed (R2: the flux of two close states in pairs).  STORED: the primitives were stored in
 // FP64; else they are formed from the states.
 template <int DIM, int SYS, int VAR, bool PAIR, bool STORED = false>
 __device__ __forceinline__ bool face_body(const Grid& g, const double* __restrict__ S, const Work& w, int dir,

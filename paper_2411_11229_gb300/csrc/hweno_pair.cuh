@@ -91,7 +91,10 @@ __device__ __forceinline__ float f_rsqrt(float x) {
 }
 __device__ __forceinline__ F2 f_rsqrt(F2 a) { return f_pack(f_rsqrt(f_lane0(a)), f_rsqrt(f_lane1(a))); }
 
-// A value h + l per lane; l is of the order of h's last bits, or of those of what h was cancelled from
+// A value h + l per lane; l is of the order of h's last bits, or of those of what h was cancelled from.  Sums are
+// Knuth's two-sum (The Art of Computer Programming 2, 4.2.2), products take the low part from an FMA and
+// quotients one correction from the exact remainder (Dekker, Numer. Math. 18, 1971), the low parts
+// added in plain FP32.
 template <class F>
 struct P {
   F h, l;
