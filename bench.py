@@ -45,8 +45,8 @@ FACE_TRAFFIC_BYTES_PER_FACE = 285.6  # ncu dram bytes per face, 2048^2 capture o
 E2E_DEPTH = 3
 # from the same capture: FP64 pipe activity and FP64 instructions per face (the hardware's side of
 # the roofline fraction, which counts the scheme's operations as written)
-FACE_FP64_PIPE_ACTIVE = 0.882
-FACE_FP64_INSTR_PER_FACE = 178.0
+FACE_FP64_PIPE_ACTIVE = 0.894
+FACE_FP64_INSTR_PER_FACE = 177.0
 
 
 def _dist():

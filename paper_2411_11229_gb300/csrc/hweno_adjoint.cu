@@ -847,7 +847,7 @@ __device__ __forceinline__ bool adj_face_pair(const Grid& g, const double* __res
   return true;
 }
 
-// Bound by the FP64 pipe (72 % busy; the fluxes' transposes) with the pairs' latency between.  1024^2: 2.1 ms
+// Bound by the FP64 pipe (72 % busy; the fluxes' transposes) with the pairs' latency between.  1024^2: 2.0 ms
 // per launch against 5.95 ms for the FP64 kernel; two or four blocks per SM: the adjoint step 11.6 and
 // 11.7 ms against 11.4 ms.
 template <bool SMALL32>
